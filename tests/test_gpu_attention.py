@@ -199,3 +199,38 @@ def test_attention_softmax_may_run_ahead_of_the_issuer(q, ctx, B, T, H, dh):
             q.qdit_sync(ctx)
             torch.cuda.synchronize()
             assert torch.equal(out, first)
+
+
+@pytest.mark.parametrize("T,masked", [(64, 0), (128, 0), (192, 64), (192, 128), (256, 0), (320, 192), (576, 128)])
+@pytest.mark.parametrize("H,dh", [(3, 64), (3, 72)])
+def test_attention_infinite_and_nan_scores(q, ctx, T, masked, H, dh):
+    """A key whose score is -inf has weight zero (its values of 1e38 would show any other), also when all of the first
+    `masked` keys are such; a row of -inf alone and a row with a NaN are NaN; the other rows do not notice."""
+    B, D = 2, H * dh
+    x = synth.normal(58, f"inf{T}.{masked}.{dh}", (B, T, 3, H, dh), 1.0)
+    x[:, :, 0, :, 3] = 1.0                                         # every query meets a key's element 3 with weight one
+    off = np.arange(T) % 8 >= 5
+    off[:masked] = True
+    x[0, off, 1, 0, 3] = -np.inf                                   # sample 0, head 0: these keys are out
+    x[0, off, 2, 0] = 1e38
+    x[0, :, 1, 1, 3] = -np.inf                                     # head 1: all of them
+    x[1, T - 2, 1, 0, 5] = np.nan                                  # sample 1, head 0: a key with a NaN (0 x NaN included)
+    x[1, :, 2, 0, :8] = 0.0
+    x[1, 5, 0, 1, 7] = np.nan                                      # head 1: a query with one
+    x[1, 9, 0, 2, 3], x[1, T - 1, 1, 2, 3] = -np.inf, -1.0         # head 2: a query with a score of +inf
+    x[1, :T - 1, 1, 2, 3] = 1.0
+    xd = dev(x.reshape(B * T, 3 * D)).to(torch.bfloat16)
+    got = _run(q, ctx, xd, B, T, H, dh, q.QDIT_F32).cpu().numpy().astype(np.float64).reshape(B, T, H, dh)
+    xh = bf16_to_f64(xd).reshape(B, T, 3, H, dh)
+    want = np.empty((B, T, H, dh))
+    with np.errstate(invalid="ignore", over="ignore"):
+        for b in range(B):
+            for h in range(H):
+                s = xh[b, :, 0, h] @ xh[b, :, 1, h].T / np.sqrt(dh)
+                e = np.exp(s - s.max(axis=1, keepdims=True))
+                keep = ~off if (b, h) == (0, 0) else np.ones(T, dtype=bool)
+                want[b, :, h] = e[:, keep] @ xh[b, keep, 2, h] / e.sum(axis=1, keepdims=True)
+    nan = np.isnan(want)
+    assert nan[0, :, 1].all() and nan[1, :, 0].all() and nan[1, 5, 1].all() and nan[1, 9, 2].all() and not nan[0, :, 0].any()
+    np.testing.assert_array_equal(np.isnan(got), nan)
+    assert np.abs(got - want)[~nan].max() <= _tol(np.where(np.abs(xh[:, :, 2]) < 1e3, xh[:, :, 2], 0.0))
