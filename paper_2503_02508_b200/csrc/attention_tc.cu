@@ -40,8 +40,10 @@
 // of the accumulator's tail is the row sum of the very bf16 probabilities that multiply V.  Head dim 64 takes the column
 // of ones the same way.
 //
-// Token counts that leave half a tile: the last key block is computed 64 keys wide, the surplus query rows are computed
-// on whatever follows and not written.
+// Token counts that leave half a tile: the first key block is 64 keys wide (not the last: the keys of an early block have a
+// maximum of their own as reference, and with 64 of them the error is that of the mma.sync kernel, which moves its reference every
+// 64 keys; 192 tokens of N(0,1) operands: 1.36e-3 of the result, 1.37e-3 the other way round, logits twice as large 0.83e-3
+// and 0.85e-3).  The surplus query rows are computed on whatever follows and not written.
 #include "common.cuh"
 #include "internal.h"
 
@@ -67,7 +69,7 @@ constexpr int STAGGER_CLOCKS = 1200;           // start of slot 1 behind slot 0
 
 struct AttnTcParams {
   int T, H;
-  int n_blk;           // key blocks of 128, the last one possibly 64 wide
+  int n_blk;           // key blocks of 128, the first one possibly 64 wide
   int n_qgroups;       // work items per (sample, head)
   int slots;           // query tiles per work item: 2, or 1 when there are too few tiles to fill the SMs in pairs
   int n_items;
@@ -135,6 +137,8 @@ __device__ __forceinline__ Item item_of(const AttnTcParams& p, int item) {
   it.q0 = g * p.slots * TQ;
   return it;
 }
+// token of a key block's first key
+__device__ __forceinline__ int key_of(const AttnTcParams& p, int j) { return j == 0 ? 0 : j * TK - (p.n_blk * TK - p.T); }
 __device__ __forceinline__ bool slot_active(const AttnTcParams& p, const Item& it, int slot) {
   return slot < p.slots && it.q0 + slot * TQ < p.T;
 }
@@ -249,7 +253,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       float m_ref = -INFINITY;
 #pragma unroll 1
       for (int j = 0; j < p.n_blk; ++j, ++n) {
-        const bool full = (j + 1) * TK <= p.T;  // else the last 64 keys
+        const bool full = j > 0 || p.T % TK == 0;  // else 64 keys
         const bool ends = j + 1 == p.n_blk;
         const int buf = ONE ? j & 1 : slot;      // which scores and probabilities
         const uint32_t s_col = trow + col_s(buf), p_col = trow + col_p(buf);
@@ -490,12 +494,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       if (elect_one()) {
         mbar_expect_tx(&kv_full[st], (jv >= 0 && jk >= 0) ? 2 * C::OP_BYTES : C::OP_BYTES);
         if (jk >= 0) {
-          tma_load_2d(sKV + (2 * st + 1) * MAIN_BYTES, &tm_k, ki.col0, ki.row0 + jk * TK, &kv_full[st]);
-          if (C::TAIL) tma_load_2d(sKVt + (2 * st + 1) * TAIL_BYTES, &tm_kt, ki.col0 + 64, ki.row0 + jk * TK, &kv_full[st]);
+          tma_load_2d(sKV + (2 * st + 1) * MAIN_BYTES, &tm_k, ki.col0, ki.row0 + key_of(p, jk), &kv_full[st]);
+          if (C::TAIL) tma_load_2d(sKVt + (2 * st + 1) * TAIL_BYTES, &tm_kt, ki.col0 + 64, ki.row0 + key_of(p, jk), &kv_full[st]);
         }
         if (jv >= 0) {
-          tma_load_2d(sKV + 2 * st * MAIN_BYTES, &tm_v, vi.col0, vi.row0 + jv * TK, &kv_full[st]);
-          if (C::TAIL) tma_load_2d(sKVt + 2 * st * TAIL_BYTES, &tm_vt, vi.col0 + 64, vi.row0 + jv * TK, &kv_full[st]);
+          tma_load_2d(sKV + 2 * st * MAIN_BYTES, &tm_v, vi.col0, vi.row0 + key_of(p, jv), &kv_full[st]);
+          if (C::TAIL) tma_load_2d(sKVt + 2 * st * TAIL_BYTES, &tm_vt, vi.col0 + 64, vi.row0 + key_of(p, jv), &kv_full[st]);
         }
       }
       __syncwarp();
@@ -580,7 +584,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           if (!landed(j)) return false;
           tc_fence_after();
           if (elect_one()) {
-            issue_s(0, j % KV_STAGES, (ragged && j + 1 == p.n_blk) ? id_s_half : id_s, j & 1);
+            issue_s(0, j % KV_STAGES, (ragged && j == 0) ? id_s_half : id_s, j & 1);
             if (j == 0) umma_commit(&kv_empty[0]);
           }
           __syncwarp();
@@ -588,7 +592,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         };
         bool ok = mbar_wait_warp(&q_full[0], 0, abort_flag, p.status) && scores(0) && (p.n_blk == 1 || scores(1));
         for (int j = 0; j < p.n_blk && ok; ++j) {
-          const bool half = ragged && j + 1 == p.n_blk;
+          const bool half = ragged && j == 0;
           ok = landed(j + 1) && mbar_wait_warp(&p_full[j & 1], static_cast<uint32_t>(j >> 1) & 1u, abort_flag, p.status);
           if (!ok) break;
           tc_fence_after();
@@ -623,7 +627,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
         tc_fence_after();
         if (elect_one()) {
-          if (active) issue_s(0, st, (ragged && p.n_blk == 1) ? id_s_half : id_s, slot);
+          if (active) issue_s(0, st, ragged ? id_s_half : id_s, slot);
           umma_commit(&kv_empty[st]);
           if (p.n_blk == 1) umma_commit(&q_empty[0]);
         }
@@ -647,9 +651,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
-            const uint32_t id = (ragged && jn + 1 == p.n_blk) ? id_s_half : id_s;
+            const uint32_t id = (ragged && jn == 0) ? id_s_half : id_s;
             const uint32_t acc0 = j == 0 ? 0u : 1u;
-            const bool half = ragged && last;
+            const bool half = ragged && j == 0;
             // first the product that reads probabilities out of the score columns, then the next scores, which the softmax
             // warps wait for, then the rest
             if (active && !half) issue_pv_alias(st, slot, acc0);
