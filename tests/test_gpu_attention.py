@@ -257,3 +257,32 @@ def test_attention_is_as_exact_as_the_mma_sync_kernel(q, ctx, T, sharpness):
     finally:
         q.qdit_set_option(ctx, q.QDIT_OPT_ATTN, 0)
     assert err[0] <= 1.005 * err[1] < 2e-3, err
+
+
+@pytest.mark.parametrize("B,T,H,dh", [(13, 320, 12, 64), (10, 320, 16, 72)])   # three query tiles per head, 468 and 480 in all
+def test_attention_tiles_are_dealt_out_evenly(q, ctx, B, T, H, dh):
+    """Token counts with an odd number of query tiles: no SM gets twice the others' work.  Against the mma.sync kernel, whose
+    small blocks the hardware deals out: 0.63 .. 0.73 of its time (items of two tiles, or of one at a head's end: 0.96 .. 1.06)."""
+    D = H * dh
+    xd = dev(synth.normal(60, f"deal{dh}", (B * T, 3 * D), 1.0)).to(torch.bfloat16)
+    out, base = torch.empty((B * T, D), dtype=torch.bfloat16, device="cuda"), xd.data_ptr()
+
+    def launches(n):
+        for _ in range(n):
+            q.qdit_attention(ctx, base, base + 2 * D, base + 4 * D, 3 * D, B, H, T, dh, 1.0 / np.sqrt(dh), out, q.QDIT_BF16, None)
+
+    times = {0: [], 1: []}
+    start, stop = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    try:
+        for _ in range(7):
+            for kernel, got in times.items():
+                q.qdit_set_option(ctx, q.QDIT_OPT_ATTN, kernel)
+                launches(5)
+                start.record()
+                launches(40)
+                stop.record()
+                torch.cuda.synchronize()
+                got.append(start.elapsed_time(stop))
+    finally:
+        q.qdit_set_option(ctx, q.QDIT_OPT_ATTN, 0)
+    assert np.median(times[0]) < 0.85 * np.median(times[1]), times
