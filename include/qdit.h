@@ -80,8 +80,8 @@ int64_t qdit_launch_count(const qdit_ctx* ctx);
  *   QDIT_OPT_GEMM_BN                0 (default): automatic; 64 | 128 | 192: token-major GEMM kernel with 128 x BN tiles
  *   QDIT_OPT_GEMM_T                 0 (default): automatic; 128 | 256: channel-major GEMM kernel with 128 x BT tiles
  *   QDIT_OPT_GEMM_GENERIC_EPILOGUE  1: the GEMM kernels' run-time-flag epilogue instead of the specialised classes
- *   QDIT_OPT_ATTN                   0 (default): the tcgen05 attention kernel; 1: the mma.sync attention kernel;
- *                                   2: as 0
+ *   QDIT_OPT_ATTN                   0 (default): the mma.sync attention kernel at 64 tokens, the tcgen05 kernel at more;
+ *                                   1: the mma.sync kernel for every token count; 2: the tcgen05 kernel for every token count
  *   QDIT_OPT_CONDITIONING_CHUNK     sampling steps whose conditioning a sampler evaluates at once: 0 (default) as many
  *                                   as fit a 4 GB modulation table, -1 step by step, n > 0 at most n (read by
  *                                   qdit_sampler_create)

@@ -1,6 +1,6 @@
 // Non-causal softmax attention in bf16 between the quantized linears: the entry point qdit_attention and the
-// mma.sync kernel that QDIT_OPT_ATTN = 1 selects (an independent implementation of the same operation; the tcgen05
-// kernel in attention_tc.cu takes every call by default).
+// mma.sync kernel that serves 64 tokens (and any count with QDIT_OPT_ATTN = 1); the tcgen05 kernel in attention_tc.cu takes
+// the others.
 //
 // One CTA = 128 (or 64) queries of one (sample, head); one warp per 16 query rows.  Q and 64-key K/V tiles
 // are staged by TMA (a 4-deep ring with mbarrier completion: at 256 tokens the whole K and V of the head are
@@ -314,7 +314,12 @@ extern "C" int32_t qdit_attention(qdit_ctx* ctx, const void* q, const void* k, c
     QDIT_TRY(qdit_check_qparams(ctx, out_qp, out_scale_dev != nullptr));
     p.qa = make_quant_args(*out_qp, out_scale_dev);
   }
-  if (ctx->opt[QDIT_OPT_ATTN] != 1)
+  // 64 tokens: half of a tcgen05 tile would be surplus rows, and the mma.sync kernel runs four CTAs per SM there (1 x 6, 10 x 16
+  // and 32 x 16 heads of 72, bf16 output: 3.0 / 4.2 / 7.9 us against 4.2 / 5.7 / 9.2).  From 128 tokens the tcgen05 kernel is
+  // faster, but for a few tens of heads at 192 tokens (16 x 72: 4.8 against 5.8): the choice does not depend on their number,
+  // so that a sample's bits do not depend on the batch.
+  const int choice = ctx->opt[QDIT_OPT_ATTN];
+  if (choice == 2 || (choice == 0 && T > 64))
     return qdit_launch_attention_tc(ctx, q, k, v, ld, B, H, T, dh, softmax_scale, out, out_dtype, p.qa);
   const bool wide = T % 128 == 0;  // 128 queries per CTA when the token count allows
   if (dh == 64) return wide ? launch_attention<64, 8>(ctx, q, k, v, ld, B, H, T, p) : launch_attention<64, 4>(ctx, q, k, v, ld, B, H, T, p);
