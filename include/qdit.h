@@ -130,7 +130,9 @@ enum { QDIT_QUANT_STATIC = 0, QDIT_QUANT_DYNAMIC = 1, QDIT_QUANT_DYNAMIC_TOKEN =
  *          M floats); the linear layer takes these scales with QDIT_EPI_ROW_SCALE.  (The paper quantizes
  *          activations tensor-wise, Experimental Settings; the per-token form is the variant of the
  *          quantization baselines it compares with.)
- * K must be a multiple of 8; M or K of 0 is a no-op. */
+ * K must be a multiple of 8; M or K of 0 is a no-op.  In every mode the call works in q and dyn_scale alone (q holds
+ * intermediate values until the codes replace them): calls with different q and dyn_scale may run beside each other, a
+ * captured one also after its context is gone. */
 int32_t qdit_quantize_act(qdit_ctx* ctx, const void* x, int x_dtype, int64_t M, int64_t K, int64_t ldx,
                           int mode, const qdit_qparams* qp, float* dyn_scale, void* q, int64_t ldq);
 

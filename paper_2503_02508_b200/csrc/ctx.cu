@@ -161,10 +161,8 @@ int32_t qdit_create(qdit_ctx** out, int device, void* cuda_stream) {
   }
   if (cudaMalloc(&ctx->d_status, sizeof(int)) != cudaSuccess ||
       cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&ctx->d_partial, sizeof(float) * prop.multiProcessorCount * QDIT_PARTIALS_PER_SM) != cudaSuccess ||
       cudaMallocHost(&ctx->h_status, sizeof(int)) != cudaSuccess) {
     if (ctx->d_status) cudaFree(ctx->d_status);
-    if (ctx->d_partial) cudaFree(ctx->d_partial);
     delete ctx;
     return QDIT_ERR_CUDA;
   }
@@ -174,7 +172,6 @@ int32_t qdit_create(qdit_ctx** out, int device, void* cuda_stream) {
   if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
       qres != cudaDriverEntryPointSuccess || !fn) {
     cudaFree(ctx->d_status);
-    cudaFree(ctx->d_partial);
     cudaFreeHost(ctx->h_status);
     delete ctx;
     return QDIT_ERR_CUDA;
@@ -213,7 +210,6 @@ int32_t qdit_destroy(qdit_ctx* ctx) {
   if (!ctx) return QDIT_ERR_INVALID_ARG;
   cudaSetDevice(ctx->device);
   if (ctx->d_status) cudaFree(ctx->d_status);
-  if (ctx->d_partial) cudaFree(ctx->d_partial);
   if (ctx->h_status) cudaFreeHost(ctx->h_status);
   for (auto& r : ctx->prof) {
     cudaEventDestroy(r.start);

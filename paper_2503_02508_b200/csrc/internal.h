@@ -33,15 +33,12 @@ struct TmapKeyHash {
   }
 };
 
-constexpr int QDIT_PARTIALS_PER_SM = 16;
-
 struct qdit_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   int* d_status = nullptr;  // device status word
   int* h_status = nullptr;  // pinned host mirror
   int num_sms = 0;
-  float* d_partial = nullptr;  // [num_sms * QDIT_PARTIALS_PER_SM] partial maxima of the dynamic quantizer (scratch of one call)
   int64_t launches = 0;
   // Kernel-selection options (qdit_set_option).  Set once at creation from the QDIT_* environment variables of the
   // same names, afterwards only through the call; no kernel launch reads the environment.
@@ -163,6 +160,7 @@ static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t
 
 // ---- internal launchers used by the model/sampler orchestration (all enqueue on ctx->stream) ----
 // Dynamic symmetric quantizer of a whole tensor: codes, the scale in *scale (required), max|x| folded into *running (optional).
+// Works in q and *scale alone.
 int32_t launch_quant_dynamic(qdit_ctx* ctx, const void* x, int x_dtype, int64_t M, int64_t K, int64_t ldx, float* scale, float* running,
                              void* q, int64_t ldq);
 int32_t launch_absmax_to_scale(qdit_ctx* ctx, const float* absmax_dev, float* scale_dev, float* running_absmax, int n);

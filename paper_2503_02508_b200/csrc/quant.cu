@@ -79,20 +79,41 @@ __global__ void __launch_bounds__(256) act_quant_token_kernel(const T* __restric
 }
 
 // ----------------------------------------------------------------------------- dynamic quantizer
-// Partial maxima, one per CTA, in the context's scratch (no accumulator to clear); then, for a tensor of few CTAs, the
-// quantizer itself reduces them: two launches, which is what the time of a small tensor consists of (64 x 1152: 8.3 us with
-// four launches, 3.4 with two).  A large tensor takes one more launch of one CTA and the plain quantizer behind it.
-template <typename T>
-__global__ void __launch_bounds__(256) absmax_partial_kernel(const T* __restrict__ x, int64_t M, int64_t K, int64_t ldx,
-                                                             float* __restrict__ partial) {
+// Two launches, which is what the time of a small tensor consists of (64 x 1152: 8.3 us with four, 3.2 with two): partial
+// maxima, one per CTA, and a quantizer whose CTAs all reduce them.  The partials lie in the output itself, which the codes
+// overwrite: memory of the call alone, whatever else runs beside it (a captured launch replayed on another stream as well).  Every
+// quantizer CTA has a copy of its own, in the part of the output that it is about to write, because no other part is safe from
+// being overwritten first.  A tensor of more than DYN_PIECES has one copy, at the front, and a launch of one CTA between that
+// reads it before the plain quantizer starts (4300 x 1152, bf16: 9.5 us).
+//
+// The output in pieces of 8 codes (two floats): parts of `size` pieces, the last two of equal length, so that none is shorter than
+// half of it and its partials fit.
+constexpr int DYN_PARTIALS = 256;        // most CTAs that form partial maxima when every part has a copy
+constexpr int64_t DYN_PIECES = 600000;
+__device__ __forceinline__ int64_t part_first(int64_t total, int parts, int size, int c) {
+  if (c == 0) return 0;
+  return c < parts - 1 ? static_cast<int64_t>(c) * size : c == parts ? total : (static_cast<int64_t>(parts - 2) * size + total) / 2;
+}
+// Row of a piece of such a tensor without a division: per_row_inv = ceil(2^40 / per_row) (exact for piece * per_row < 2^40), or 0 if
+// all pieces lie in row 0.
+inline uint64_t inverse_of(int64_t per_row) { return per_row > DYN_PIECES ? 0 : ((1ull << 40) + per_row - 1) / per_row; }
+__device__ __forceinline__ uint32_t row_of(uint32_t piece, uint64_t per_row_inv) { return static_cast<uint32_t>(piece * per_row_inv >> 40); }
+__device__ __forceinline__ float* partial_at(uint8_t* q, int64_t ldq, uint32_t per_row, uint64_t per_row_inv, int64_t first, int i) {
+  const uint32_t piece = static_cast<uint32_t>(first) + (i >> 1), row = row_of(piece, per_row_inv);
+  return reinterpret_cast<float*>(q + static_cast<int64_t>(row) * ldq + (piece - row * per_row) * 8) + (i & 1);
+}
+
+template <typename T, int THREADS>
+__global__ void __launch_bounds__(THREADS) absmax_partial_kernel(const T* __restrict__ x, int64_t M, int64_t K, int64_t ldx,
+                                                                 uint8_t* __restrict__ q, int64_t ldq, uint64_t per_row_inv, int copies, int size) {
   grid_dependency_wait();
   grid_dependency_release();
   const int64_t vec_per_row = K / 8;
   const int64_t total = M * vec_per_row;
   float m = 0.0f;
-  for (int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
-       idx += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t row = idx / vec_per_row;
+  for (int64_t idx = static_cast<int64_t>(blockIdx.x) * THREADS + threadIdx.x; idx < total;
+       idx += static_cast<int64_t>(gridDim.x) * THREADS) {
+    const int64_t row = total <= DYN_PIECES ? row_of(static_cast<uint32_t>(idx), per_row_inv) : idx / vec_per_row;
     const int64_t col = (idx - row * vec_per_row) * 8;
     float v[8];
     Load8<T>::load(x + row * ldx + col, v);
@@ -100,22 +121,20 @@ __global__ void __launch_bounds__(256) absmax_partial_kernel(const T* __restrict
     for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
   }
   m = warp_max(m);
-  __shared__ float smax[8];
+  __shared__ float smax[THREADS / 32];
   if ((threadIdx.x & 31) == 0) smax[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    m = threadIdx.x < (blockDim.x >> 5) ? smax[threadIdx.x] : 0.0f;
-    m = warp_max(m);
-    if (threadIdx.x == 0) partial[blockIdx.x] = m;
-  }
+  m = warp_max(smax[threadIdx.x & (THREADS / 32 - 1)]);
+  for (int c = threadIdx.x; c < copies; c += THREADS) 
+    *partial_at(q, ldq, static_cast<uint32_t>(vec_per_row), per_row_inv, part_first(total, copies, size, c), blockIdx.x) = m;
 }
 
 // The partials -> s = max / 127 (1 for an empty range); thread 0 of CTA 0 leaves it in *scale and folds the maximum into
-// *running (both optional).  256 threads.
-__device__ __forceinline__ float scale_of_partials(const float* __restrict__ partial, int n_partial, float* __restrict__ scale,
-                                                   float* __restrict__ running) {
+// *running (both optional).  256 threads; on return all of them have read their partials.
+__device__ __forceinline__ float scale_of_partials(uint8_t* q, int64_t ldq, uint32_t per_row, uint64_t per_row_inv, int64_t first, int n_partial,
+                                                   float* __restrict__ scale, float* __restrict__ running) {
   float m = 0.0f;
-  for (int i = threadIdx.x; i < n_partial; i += 256) m = fmaxf(m, partial[i]);
+  for (int i = threadIdx.x; i < n_partial; i += 256) m = fmaxf(m, __ldcg(partial_at(q, ldq, per_row, per_row_inv, first, i)));
   m = warp_max(m);
   __shared__ float smax[8];
   if ((threadIdx.x & 31) == 0) smax[threadIdx.x >> 5] = m;
@@ -131,27 +150,34 @@ __device__ __forceinline__ float scale_of_partials(const float* __restrict__ par
   }
   return s;
 }
-__global__ void __launch_bounds__(256) partials_to_scale_kernel(const float* __restrict__ partial, int n_partial, float* __restrict__ scale,
-                                                                float* __restrict__ running) {
+__global__ void __launch_bounds__(256) partials_to_scale_kernel(uint8_t* q, int64_t ldq, uint32_t per_row, uint64_t per_row_inv, int n_partial,
+                                                                float* __restrict__ scale, float* __restrict__ running) {
   grid_dependency_wait();
   grid_dependency_release();
-  scale_of_partials(partial, n_partial, scale, running);
+  scale_of_partials(q, ldq, per_row, per_row_inv, 0, n_partial, scale, running);
 }
-// one thread per 8 elements
-template <typename T>
-__global__ void __launch_bounds__(256) act_quant_dynamic_kernel(const T* __restrict__ x, int64_t M, int64_t K, int64_t ldx,
-                                                                const float* __restrict__ partial, int n_partial,
-                                                                float* __restrict__ scale, float* __restrict__ running,
-                                                                uint8_t* __restrict__ q, int64_t ldq) {
+// V pieces per thread
+template <typename T, int V>
+__global__ void __launch_bounds__(256) act_quant_dynamic_kernel(const T* __restrict__ x, int64_t M, int64_t K, int64_t ldx, uint64_t per_row_inv, int n_partial,
+                                                                float* __restrict__ scale, float* __restrict__ running, uint8_t* q, int64_t ldq) {
   grid_dependency_wait();
   grid_dependency_release();
-  const int64_t vec_per_row = K / 8, idx = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
-  const bool live = idx < M * vec_per_row;
-  const int64_t row = idx / vec_per_row, col = (idx - row * vec_per_row) * 8;
-  float v[8];
-  if (live) Load8<T>::load(x + row * ldx + col, v);
-  const float inv = __fdiv_rn(1.0f, scale_of_partials(partial, n_partial, scale, running));
-  if (live) *reinterpret_cast<uint2*>(q + row * ldq + col) = quantize_pack8(v, inv, 0.0f, -127.0f, 127.0f);
+  const uint32_t per_row = static_cast<uint32_t>(K / 8);
+  const int64_t total = M * (K / 8);
+  const int64_t first = part_first(total, gridDim.x, 256 * V, blockIdx.x), last = part_first(total, gridDim.x, 256 * V, blockIdx.x + 1);
+  float v[V][8];
+  uint8_t* dst[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const uint32_t piece = static_cast<uint32_t>(first) + threadIdx.x + 256u * k, row = row_of(piece, per_row_inv);
+    const int64_t col = static_cast<int64_t>(piece - row * per_row) * 8;
+    dst[k] = piece < last ? q + row * ldq + col : nullptr;
+    if (dst[k]) Load8<T>::load(x + row * ldx + col, v[k]);
+  }
+  const float inv = __fdiv_rn(1.0f, scale_of_partials(q, ldq, per_row, per_row_inv, first, n_partial, scale, running));
+#pragma unroll
+  for (int k = 0; k < V; ++k)
+    if (dst[k]) *reinterpret_cast<uint2*>(dst[k]) = quantize_pack8(v[k], inv, 0.0f, -127.0f, 127.0f);
 }
 
 // scale[i] = absmax[i] / 127 (1 if the range is empty); optionally widens a running maximum.
@@ -475,18 +501,27 @@ cudaError_t launch_act_quant(qdit_ctx* ctx, void (*kernel)(KArgs...), dim3 grid,
 
 template <typename T>
 int32_t quant_dynamic(qdit_ctx* ctx, const T* x, int64_t M, int64_t K, int64_t ldx, float* scale, float* running, uint8_t* q, int64_t ldq) {
-  const int64_t want = (M * (K / 8) + 255) / 256;
-  const int64_t most = static_cast<int64_t>(ctx->num_sms) * QDIT_PARTIALS_PER_SM;
-  const int grid = static_cast<int>(want < most ? want : most);
+  const int64_t total = M * (K / 8);
+  const uint64_t per_row_inv = inverse_of(K / 8);
   ProfScope prof(ctx, QDIT_PROF_ACT_QUANT, static_cast<double>(M) * K * (sizeof(T) + 1.0));
-  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, absmax_partial_kernel<T>, dim3(grid), dim3(256), 0, x, M, K, ldx, ctx->d_partial));
-  QDIT_TRY(qdit_after_launch(ctx, "absmax_partial_kernel"));
-  if (want <= most) {
-    QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, act_quant_dynamic_kernel<T>, dim3(grid), dim3(256), 0, x, M, K, ldx, ctx->d_partial, grid, scale,
-                                                running, q, ldq));
+  if (total <= DYN_PIECES) {
+    // one piece per thread for up to 512 parts; then two, four, eight.  With more parts than SMs one larger CTA per SM forms the
+    // partials (512 x 1152, bf16: 4.0 us, with one CTA per part 4.4; two pieces per thread there 4.6)
+    const int v = total <= 512 * 256 ? 1 : total <= 300 * 512 ? 2 : total <= 300 * 1024 ? 4 : 8;
+    const int parts = static_cast<int>((total + 256 * v - 1) / (256 * v));
+    const int n_partial = parts < ctx->num_sms ? parts : ctx->num_sms < DYN_PARTIALS ? ctx->num_sms : DYN_PARTIALS;
+    const int threads = n_partial == parts ? 256 : v == 1 ? 512 : 1024;
+    const auto quantize = v == 1 ? act_quant_dynamic_kernel<T, 1> : v == 2 ? act_quant_dynamic_kernel<T, 2> : v == 4 ? act_quant_dynamic_kernel<T, 4> : act_quant_dynamic_kernel<T, 8>;
+    QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, threads == 256 ? absmax_partial_kernel<T, 256> : threads == 512 ? absmax_partial_kernel<T, 512> : absmax_partial_kernel<T, 1024>, dim3(n_partial), dim3(threads), 0, x, M, K,
+                                                ldx, q, ldq, per_row_inv, parts, 256 * v));
+    QDIT_TRY(qdit_after_launch(ctx, "absmax_partial_kernel"));
+    QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, quantize, dim3(parts), dim3(256), 0, x, M, K, ldx, per_row_inv, n_partial, scale, running, q, ldq));
     return qdit_after_launch(ctx, "act_quant_dynamic_kernel");
   }
-  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, partials_to_scale_kernel, dim3(1), dim3(256), 0, ctx->d_partial, grid, scale, running));
+  const int n_partial = ctx->num_sms * 8;   // fewer than the pieces of a tensor that comes here
+  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, absmax_partial_kernel<T, 256>, dim3(n_partial), dim3(256), 0, x, M, K, ldx, q, ldq, per_row_inv, 1, 0));
+  QDIT_TRY(qdit_after_launch(ctx, "absmax_partial_kernel"));
+  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, partials_to_scale_kernel, dim3(1), dim3(256), 0, q, ldq, static_cast<uint32_t>(K / 8), per_row_inv, n_partial, scale, running));
   QDIT_TRY(qdit_after_launch(ctx, "partials_to_scale_kernel"));
   const QuantArgs qa = make_quant_args(qdit_qparams{1.0f, 0, -127, 127}, scale);
   const int64_t threads = M * ((K + 15) / 16);

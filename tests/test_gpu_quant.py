@@ -265,3 +265,64 @@ def test_large_quantizer_gives_the_codes_of_its_parts(q, ctx, M, K, dtype):
         q.qdit_quantize_act(ctx, x[r:], kind, n, K, K, q.QDIT_QUANT_STATIC, q.qparams(0.03), None, parts[r:], K)
     q.qdit_sync(ctx)
     assert torch.equal(whole, parts)
+
+
+@pytest.mark.parametrize("M,K,ld", [(1, 8, 16), (257, 8, 8), (511, 1032, 1048), (1024, 1024, 1024), (1025, 1024, 1032), (150, 8192, 8192), (151, 8192, 8200), (300, 8192, 8192),
+                                    (301, 8192, 8200), (4687, 1024, 1032), (4688, 1024, 1024)])
+@pytest.mark.parametrize("where", [0, 1])   # the largest value in the first or the last element
+def test_dynamic_quantizer_keeps_its_partials_in_the_output(q, ctx, M, K, ld, where):
+    """Sizes at the edges of the launch forms (one, two, four and eight pieces per thread, one copy of the partial maxima); pitches wider than
+    the rows: nothing outside of them is written."""
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    x = torch.randn(M, ld, generator=g, device="cuda")
+    x[0 if where == 0 else M - 1, 0 if where == 0 else K - 1] = -37.5
+    scale = torch.full((1,), -1.0, device="cuda")
+    out = torch.full((M, ld), 9, dtype=torch.int8, device="cuda")
+    q.qdit_quantize_act(ctx, x, q.QDIT_F32, M, K, ld, q.QDIT_QUANT_DYNAMIC, None, scale, out, ld)
+    q.qdit_sync(ctx)
+    s = torch.tensor(37.5, device="cuda") / 127.0
+    assert scale[0] == s
+    assert torch.equal(out[:, :K], torch.clamp(torch.round(x[:, :K] * (1.0 / s)), -127, 127).to(torch.int8))
+    assert (out[:, K:] == 9).all()
+
+
+def test_captured_dynamic_quantizers_share_nothing(q):
+    """Launches captured from one context and replayed beside its later calls, and after it is gone: every call works in its own
+    output and scale alone."""
+    M, K = 512, 1152
+    own, side = torch.cuda.Stream(), torch.cuda.Stream()
+    c = q.qdit_create(0, own.cuda_stream)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    xs = [torch.randn(M, K, generator=g, device="cuda") * f for f in (1.0, 50.0)]
+    outs = [torch.empty(M, K, dtype=torch.int8, device="cuda") for _ in xs]
+    scales = [torch.zeros(1, device="cuda") for _ in xs]
+    want = [(x.abs().amax() / 127.0).reshape(1) for x in xs]
+    codes = [torch.clamp(torch.round(x * (1.0 / s)), -127, 127).to(torch.int8) for x, s in zip(xs, want)]
+    torch.cuda.synchronize()
+
+    def quantize(i, n):
+        for _ in range(n):
+            q.qdit_quantize_act(c, xs[i], q.QDIT_F32, M, K, K, q.QDIT_QUANT_DYNAMIC, None, scales[i], outs[i], K)
+
+    with torch.cuda.stream(own):
+        quantize(0, 1)
+    own.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=own):
+        quantize(1, 50)
+
+    def check():
+        torch.cuda.synchronize()
+        for i in range(2):
+            assert torch.equal(scales[i], want[i]) and torch.equal(outs[i], codes[i])
+
+    for _ in range(20):
+        with torch.cuda.stream(side):
+            graph.replay()
+        quantize(0, 50)
+        check()
+    q.qdit_destroy(c)
+    scales[1].zero_()
+    with torch.cuda.stream(side):
+        graph.replay()
+    check()
