@@ -51,13 +51,9 @@ struct TWarps {
   static constexpr int EPI_WARPS = EPI == 4 ? 12 : (STAGED ? QDIT_T_STAGED_WARPS : 12);
   static constexpr int SPLIT = EPI_WARPS / 4;
   static constexpr int THREADS = 64 + EPI_WARPS * 32;
-#ifndef QDIT_T_GATED_TILES
-#define QDIT_T_GATED_TILES 2
-#endif
-  // 2 KB tiles of 32 tokens x 32 channels bf16 per warp: class 1 two output tiles used in turn; class 3 the residual
-  // tile plus one tile shared by the cache copy and the output (2) or one tile each (3)
-  static constexpr int TILES = GATED ? QDIT_T_GATED_TILES : 2;
-  static constexpr int STAGING_PER_WARP = STAGED ? TILES * 2048 : 0;
+  // two 2 KB tiles of 32 tokens x 32 channels bf16 per warp: class 1 two output tiles used in turn; class 3 the residual
+  // tile and one shared by the cache copy and the output
+  static constexpr int STAGING_PER_WARP = STAGED ? 2 * 2048 : 0;
   // class 2 (8-bit codes): the four quadrant warps that work on the same token chunk share a tile of 32 tokens x 128
   // channels (4 KB), two tiles used in turn per group of four
   static constexpr bool GROUPED = EPI == 2;
@@ -385,9 +381,6 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
       uint8_t* stg = staging + e * TW::STAGING_PER_WARP;
       // class 1: two output tiles used in turn; class 3: tile 0 receives the residual, tile 1 carries the cache copy and then the output
       const uint32_t tile0 = smem_u32(stg), tile1 = tile0 + 2048u;
-      constexpr bool SEPARATE = TW::TILES == 3;                       // class 3: the output has a tile of its own
-      const uint32_t tile_o = SEPARATE ? tile0 + 4096u : tile1;
-      uint8_t* const stg_o = stg + (SEPARATE ? 4096 : 2048);
       const uint32_t row_off = frag_row_offset(lane);
       uint64_t* rbar = &res_bar[e];
       uint32_t r_phase = 0;
@@ -501,12 +494,8 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             out_turn ^= 1;
           } else {
             // cache copy (the branch output before the gate), if one is kept
-            // tile 1 is free once the store that last used it has read it: the previous chunk's output store, or
-            // (separate tiles) the previous chunk's cache store, one group further back
             if (flags & QDIT_EPI_CACHE_STORE) {
-              if (lane == 0) {
-                if (SEPARATE) tma_store_wait_read<1>(); else tma_store_wait_read<0>();
-              }
+              if (lane == 0) tma_store_wait_read<0>();  // tile 1 is free once the previous chunk's output store has read it
               __syncwarp();
               frag_store_tile(tile1 + row_off, f);
               fence_async_smem();
@@ -546,15 +535,13 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                 r_inflight = true;
               }
             }
-            if (lane == 0) {  // the output tile is free: this chunk's cache store has read it, or (separate tiles) the previous chunk's output store
-              if (SEPARATE) tma_store_wait_read<1>(); else tma_store_wait_read<0>();
-            }
+            if (lane == 0) tma_store_wait_read<0>();  // the store that last used tile 1 has read it: this chunk's cache copy or the previous output
             __syncwarp();
-            frag_store_tile(tile_o + row_off, f);
+            frag_store_tile(tile1 + row_off, f);
             fence_async_smem();
             __syncwarp();
             if (lane == 0) {
-              tma_store_2d(&tmap_out, stg_o, c0q, m_base);
+              tma_store_2d(&tmap_out, stg + 2048, c0q, m_base);
               tma_store_commit();
             }
           }
