@@ -482,11 +482,14 @@ def test_code_output_leaves_the_padding_of_its_rows_alone(q, ctx, N, ldo):
 
 
 @pytest.mark.parametrize("M,N,K", [
-    (1, 8, 512),         # smallest split: two CTAs with two k-blocks each
+    (1, 8, 512),         # four k-blocks: too short to split
+    (8, 8, 1024),        # shortest split reduction: one tile, four CTAs with two k-blocks each
     (64, 392, 4608),     # six CTAs per tile, ragged columns (392 = 6 * 64 + 8)
-    (100, 1152, 1040),   # ragged rows, 9 k-blocks over four CTAs, the last one short
+    (100, 1152, 1040),   # four CTAs per tile: ragged rows, 9 k-blocks, the last one short
     (256, 1152, 4608),   # three CTAs per tile: row groups 6, 5, 5
-    (300, 1152, 800),    # two or three CTAs per tile, short reduction
+    (300, 1152, 800),    # seven k-blocks: too short to split
+    (300, 1152, 1536),   # two CTAs per tile: ragged rows
+    (512, 1152, 4608),   # two CTAs per tile: 72 tiles
     (1040, 2312, 256),   # channel-major kernel: ragged rows and columns
     (1025, 2304, 1152),
     (4000, 1160, 1152),  # channel-major gated layer: 32 x 7 token-major tiles of 192 exceed one wave
@@ -532,10 +535,11 @@ def test_automatic_kernel_gives_the_bits_of_the_token_major_kernel(q, ctx, M, N,
     assert torch.equal(got[1], ref[1])
 
 
-@pytest.mark.parametrize("M,N,K", [(1, 8, 1024), (64, 392, 4608), (100, 1152, 1056), (256, 1152, 4608), (512, 1152, 4608)])
+@pytest.mark.parametrize("M,N,K", [(1, 8, 1024), (64, 392, 4608), (100, 1152, 1056), (256, 1152, 4608), (300, 1152, 1536),
+                                   (512, 1152, 4608)])
 @pytest.mark.parametrize("kind", ["i32", "gated", "gelu"])
 def test_packed_weights_with_a_split_reduction(q, ctx, M, N, K, kind):
-    """Packed 4-bit weights widened inside the split-reduction kernel: the bits of the one-code-per-byte layer."""
+    """Packed 4-bit weights widened inside the split-reduction kernel: the bits of the one-code-per-byte layer, whole reductions."""
     T = 32
     codes = _w4_codes(93, f"w4s.{N}.{K}", N, K)
     A, W8, W4 = dev_i8(_codes(93, f"a{M}.{K}", (M, K), -127, 127)), dev_i8(codes), torch.from_numpy(quant.pack_int4(codes)).cuda()
@@ -550,6 +554,10 @@ def test_packed_weights_with_a_split_reduction(q, ctx, M, N, K, kind):
         if i == 0:
             q.qdit_w4a8_linear(ctx, A, W4, M, N, K, q.qparams(0.03), None, flags, epi, out[0], N)
         else:
-            q.qdit_w8a8_linear(ctx, A, W8, M, N, K, q.qparams(0.03), None, flags, epi, out[1], N)
+            try:
+                q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 64)   # unsplit
+                q.qdit_w8a8_linear(ctx, A, W8, M, N, K, q.qparams(0.03), None, flags, epi, out[1], N)
+            finally:
+                q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 0)
         q.qdit_sync(ctx)
     assert torch.equal(out[0], out[1]) and torch.equal(cache[0], cache[1])
