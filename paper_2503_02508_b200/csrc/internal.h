@@ -70,7 +70,8 @@ struct ProfScope {
 
 // Launches `kernel` on the context's stream.  With ctx->overlap_launches the launch carries the
 // programmatic-stream-serialization attribute: the kernel may start its preamble before the previous kernel
-// of the stream has finished, and MUST call grid_dependency_wait() before its first global-memory access.
+// of the stream has finished, and MUST call grid_dependency_wait() before its first access to global memory that an earlier
+// launch of the stream may write (weights that are constant since the model was created may be fetched before).
 template <typename... KArgs, typename... Args>
 cudaError_t qdit_launch_overlapped(qdit_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                    Args&&... args) {
@@ -163,7 +164,7 @@ static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t
 // Works in q and *scale alone.
 int32_t launch_quant_dynamic(qdit_ctx* ctx, const void* x, int x_dtype, int64_t M, int64_t K, int64_t ldx, float* scale, float* running,
                              void* q, int64_t ldq);
-int32_t launch_absmax_to_scale(qdit_ctx* ctx, const float* absmax_dev, float* scale_dev, float* running_absmax, int n);
+int32_t launch_absmax_to_scale(qdit_ctx* ctx, const float* absmax_dev, float* scale_dev, int n);
 // Quantizes an f32 tensor [M,K] (contiguous) with the scale held in device memory.
 int32_t qdit_quantize_act_dev(qdit_ctx* ctx, const float* x, int64_t M, int64_t K, qdit_qparams qp,
                               const float* scale_dev, uint8_t* q);

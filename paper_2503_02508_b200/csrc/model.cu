@@ -439,7 +439,7 @@ int32_t qdit_model_begin_calibration(qdit_ctx* ctx, qdit_model* m) {
 
 int32_t qdit_model_finish_calibration(qdit_ctx* ctx, qdit_model* m) {
   if (!ctx || !m) return QDIT_ERR_INVALID_ARG;
-  QDIT_TRY(launch_absmax_to_scale(ctx, m->d_absmax_run, m->d_scales, nullptr, m->n_scales()));
+  QDIT_TRY(launch_absmax_to_scale(ctx, m->d_absmax_run, m->d_scales, m->n_scales()));
   m->scales_set = true;
   return QDIT_OK;
 }

@@ -180,17 +180,12 @@ __global__ void __launch_bounds__(256) act_quant_dynamic_kernel(const T* __restr
     if (dst[k]) *reinterpret_cast<uint2*>(dst[k]) = quantize_pack8(v[k], inv, 0.0f, -127.0f, 127.0f);
 }
 
-// scale[i] = absmax[i] / 127 (1 if the range is empty); optionally widens a running maximum.
-__global__ void absmax_to_scale_kernel(const float* __restrict__ absmax, float* __restrict__ scale,
-                                       float* __restrict__ running, int n) {
+// scale[i] = absmax[i] / 127 (1 if the range is empty).
+__global__ void absmax_to_scale_kernel(const float* __restrict__ absmax, float* __restrict__ scale, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float a = absmax[i];
-  if (running) running[i] = fmaxf(running[i], a);
-  if (scale) {
-    const float s = __fdiv_rn(a, 127.0f);
-    scale[i] = s > 0.0f ? s : 1.0f;
-  }
+  const float s = __fdiv_rn(absmax[i], 127.0f);
+  scale[i] = s > 0.0f ? s : 1.0f;
 }
 
 // ----------------------------------------------------------------------------- channel-wise weight quantizer
@@ -470,7 +465,7 @@ void launch_ln_q8(qdit_ctx* ctx, const void* x, int64_t M, const float* shift, c
                          ld_mod, static_cast<uint8_t*>(out), qa, static_cast<int>(rows));
 }
 
-// Row range per CTA: `per_sm` CTAs per SM, at least one row per warp, at most what keeps a range within two samples.
+// Row range per CTA: `per_sm` CTAs per SM, at least eight rows, at most what keeps a range within two samples.
 int64_t ln_rows_per_cta(const qdit_ctx* ctx, int64_t M, int64_t T, int per_sm) {
   const int64_t ctas = per_sm * static_cast<int64_t>(ctx->num_sms);
   int64_t rows = (M + ctas - 1) / ctas;
@@ -538,9 +533,9 @@ int32_t launch_quant_dynamic(qdit_ctx* ctx, const void* x, int x_dtype, int64_t 
   return quant_dynamic(ctx, static_cast<const float*>(x), M, K, ldx, scale, running, static_cast<uint8_t*>(q), ldq);
 }
 
-int32_t launch_absmax_to_scale(qdit_ctx* ctx, const float* absmax_dev, float* scale_dev, float* running_absmax, int n) {
+int32_t launch_absmax_to_scale(qdit_ctx* ctx, const float* absmax_dev, float* scale_dev, int n) {
   if (n <= 0) return QDIT_OK;
-  absmax_to_scale_kernel<<<(n + 127) / 128, 128, 0, ctx->stream>>>(absmax_dev, scale_dev, running_absmax, n);
+  absmax_to_scale_kernel<<<(n + 127) / 128, 128, 0, ctx->stream>>>(absmax_dev, scale_dev, n);
   return qdit_after_launch(ctx, "absmax_to_scale_kernel");
 }
 
