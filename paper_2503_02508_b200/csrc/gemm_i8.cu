@@ -86,50 +86,56 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   const int num_kb = (p.K + BK - 1) / BK;
   const int total_tiles = p.num_m_tiles * p.num_n_tiles;
 
+  // One elected thread runs each of the two roles, so that the operands of its instructions stay in uniform registers.  (Behind
+  // `lane == 0` 8192 x 1152 x 4608 takes 40.1 us, with the whole warp in the role and an election at each issue 41.5, so 38.0;
+  // 700 x 1152 x 4608 13.3, 11.5 and 8.2.)  With the small tiles of few rows the roles look at their next barrier before they issue
+  // the current stage (9.6 us without that); 192 columns per stage leave the time, and the look costs 1 %.
+  constexpr bool AHEAD = BN != 192;
+  auto wait_for = [&](bool seen, uint64_t* bar, uint32_t parity) { return seen || mbar_wait(bar, parity, abort_flag, p.status); };
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true, seen = true;   // seen: the stage about to be filled is known to be free
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      const int m0 = (tile / p.num_n_tiles) * BM;
-      const int n0 = (tile % p.num_n_tiles) * BN;
-      for (int kb = 0; kb < num_kb; ++kb) {
-        if (!mbar_wait_seen(seen, &empty_bar[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
-        const bool wrap = stage + 1 == STAGES;
-        seen = mbar_test_wait(&empty_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 0u : 1u));
-        if (elect_one()) {
+    if (elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true, seen = true;   // seen: the stage about to be filled is known to be free
+      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+        const int m0 = (tile / p.num_n_tiles) * BM;
+        const int n0 = (tile % p.num_n_tiles) * BN;
+        for (int kb = 0; kb < num_kb; ++kb) {
+          if (!wait_for(seen, &empty_bar[stage], phase ^ 1u)) { ok = false; break; }
+          const bool wrap = stage + 1 == STAGES;
+          seen = AHEAD && mbar_test_wait(&empty_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 0u : 1u));
           mbar_expect_tx(&full_bar[stage], C::STAGE_BYTES);
           tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, kb * BK, m0, &full_bar[stage]);
           tma_load_2d(sB + stage * C::B_BYTES, &tmap_w, kb * BK, n0, &full_bar[stage]);
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
-    }
-    if (!ok) {
-      // give copies already in flight time to land before the CTA's shared memory is released
-      for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+      if (!ok) {
+        // give copies already in flight time to land before the CTA's shared memory is released
+        for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+      }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    int stage = 0;
-    uint32_t phase = 0;
-    int it = 0;
-    bool ok = true, seen = false;   // seen: the stage about to be multiplied is known to have landed
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++it) {
-      const int as = it & 1;
-      const uint32_t aphase = static_cast<uint32_t>(it >> 1) & 1u;
-      if (!mbar_wait_warp(&tempty_bar[as], aphase ^ 1u, abort_flag, p.status)) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(as * BN);
-      for (int kb = 0; kb < num_kb; ++kb) {
-        if (!mbar_wait_seen(seen, &full_bar[stage], phase, abort_flag, p.status)) { ok = false; break; }
-        const bool wrap = stage + 1 == STAGES;
-        seen = mbar_test_wait(&full_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 1u : 0u));
+    if (elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0;
+      int it = 0;
+      bool ok = true, seen = false;   // seen: the stage about to be multiplied is known to have landed
+      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++it) {
+        const int as = it & 1;
+        const uint32_t aphase = static_cast<uint32_t>(it >> 1) & 1u;
+        if (!wait_for(false, &tempty_bar[as], aphase ^ 1u)) { ok = false; break; }
         tc_fence_after();
-        const uint64_t a_desc = umma_desc_k_sw128(smem_u32(sA + stage * C::A_BYTES));
-        const uint64_t b_desc = umma_desc_k_sw128(smem_u32(sB + stage * C::B_BYTES));
-        if (elect_one()) {
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(as * BN);
+        for (int kb = 0; kb < num_kb; ++kb) {
+          if (!wait_for(seen, &full_bar[stage], phase)) { ok = false; break; }
+          const bool wrap = stage + 1 == STAGES;
+          seen = AHEAD && mbar_test_wait(&full_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 1u : 0u));
+          tc_fence_after();
+          const uint64_t a_desc = umma_desc_k_sw128(smem_u32(sA + stage * C::A_BYTES));
+          const uint64_t b_desc = umma_desc_k_sw128(smem_u32(sB + stage * C::B_BYTES));
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
             // advancing K by 32 bytes inside the swizzle row = +2 in the (address >> 4) field
@@ -137,11 +143,10 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                     b_desc + static_cast<uint64_t>(k * (UMMA_K >> 4)), idesc, (kb | k) != 0 ? 1u : 0u);
           }
           umma_commit(&empty_bar[stage]);  // frees the smem stage once these MMAs have read it
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        __syncwarp();
-        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        if (ok) umma_commit(&tfull_bar[as]);  // accumulator complete
       }
-      if (ok && elect_one()) umma_commit(&tfull_bar[as]);  // accumulator complete
     }
   } else {
     // -------------------------------------------------------------------- epilogue warps
@@ -224,14 +229,18 @@ int pick_bn(int M, int N, int num_sms, int forced) {
 }
 
 // CTAs that share the reduction of a 128 x 64 tile: the most for which all clusters are resident at once (a second wave
-// would cost more than the split gains: 256 x 1152 x 4608 takes 13.7 us with 36 clusters of 4, 7.8 with 36 of 3).  A k-block
-// costs about 0.2 us and the exchange 0.8, so each CTA has to be spared at least six k-blocks and keep two (512 x 1152 x
-// 1152, nine k-blocks: 5.7 us whole, 6.3 split in two; 256 x 1152 x 4608: 12.0 whole).
-int pick_split(qdit_ctx* ctx, int M, int N, int K) {
+// would cost more than the split gains: 256 x 1152 x 4608 takes 13.7 us with 36 clusters of 4, 7.4 with 36 of 3), if each CTA keeps two
+// k-blocks and is spared `spare` of them.  A k-block costs the whole-reduction kernel 0.11 us and the exchange about two: 20.
+// (Whole / split: 256 x 1152 x 4608 7.9 / 7.4 us with 24 spared, 512 x 1152 x 4608 8.1 / 8.5 with 18, 512 x 1152 x 2304 5.5 / 6.3,
+// 256 x 1152 x 1152 5.0 / 5.6.)  Two cases gain more: with packed weights the whole-reduction kernel widens them at 0.3 us per
+// k-block, and the epilogues with run-time flags (f32 output, per-token scales) are slow on one SM, whereas a cluster splits the
+// epilogue too (f32 output, 256 x 384 x 1536: 6.4 / 5.3 us, 256 x 1152 x 1152: 6.1 / 5.8): 6.
+constexpr int SPLIT_SPARE = 20, SPLIT_SPARE_SLOW = 6;
+int pick_split(qdit_ctx* ctx, int M, int N, int K, int spare) {
   const int64_t tiles = static_cast<int64_t>((M + BM - 1) / BM) * ((N + 63) / 64);
   const int num_kb = (K + BK - 1) / BK;
   for (int s : {6, 4, 3, 2})
-    if (num_kb >= 2 * s && num_kb - (num_kb + s - 1) / s >= 6 && tiles * s <= ctx->num_sms && tiles <= qdit_gemm_sk_clusters(ctx, s)) return s;
+    if (num_kb >= 2 * s && num_kb - (num_kb + s - 1) / s >= spare && tiles * s <= ctx->num_sms && tiles <= qdit_gemm_sk_clusters(ctx, s)) return s;
   return 1;
 }
 
@@ -333,7 +342,7 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
       W = w8_scratch;
     } else {
       // (few tiles split by the same rule as below: 256 / 512 x 1152 x 4608 take 8.5 / 10.3 us against 17.7 / 17.9)
-      const int split = ctx->opt[QDIT_OPT_GEMM_BN] == 0 ? pick_split(ctx, p.M, p.N, p.K) : 1;
+      const int split = ctx->opt[QDIT_OPT_GEMM_BN] == 0 ? pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) : 1;
       return split > 1 ? qdit_launch_gemm_sk(ctx, A, W, p, a_unsigned, split, true) : qdit_launch_gemm_w4(ctx, A, W, p, a_unsigned);
     }
   }
@@ -343,10 +352,10 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
   const bool row_scale = (flags & QDIT_EPI_ROW_SCALE) != 0;
   if (!row_scale && ctx->opt[QDIT_OPT_GEMM_T] != 0) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, ctx->opt[QDIT_OPT_GEMM_T]);
   // Kernel choice: layers with many rows run channel-major with 128 x 256 tiles when their epilogue has a staged form there
-  // (a TMA store per 32-token chunk; 8192 rows, us, against token-major: QKV 27 / 31, fc1 39 / 48, proj 15.5 / 20, fc2 38 /
-  // 44, per-token scales 27 / 45, f32 output 36 / 48); few rows, narrow outputs and every other epilogue run token-major.
+  // (a TMA store per 32-token chunk; 8192 rows, us, against token-major: QKV 30 / 33, fc1 39 / 48, proj 17 / 20, fc2 39 /
+  // 46, per-token scales 30 / 45, f32 output 37 / 51); few rows, narrow outputs and every other epilogue run token-major.
   // The gated layers are narrow (1152 columns): up to the row count where 128 x 192 token-major tiles fill one wave, the
-  // smaller tiles spread over more SMs (fc2 at 1024 / 2048 / 3072 rows: 12.7 / 15.4 / 16.9 us against 17.4 / 17.7 / 18.2).
+  // smaller tiles spread over more SMs (fc2 at 1024 / 2048 / 3072 rows: 8.8 / 14.0 / 17.8 us against 17.1 / 20.0 / 20.1).
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0 && p.M >= 1024 && !(row_scale && ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE])) {
     // (8-bit rows leave through TMA stores of whole 16-byte pieces: the width and the pitch have to be multiples of 16)
     const bool staged_form = cls == 1 || cls == 5 || cls == 6 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0);
@@ -355,7 +364,8 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
       return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
   }
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0) {
-    const int split = pick_split(ctx, p.M, p.N, p.K);
+    const bool fast = cls >= 1 && cls <= 3 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE];
+    const int split = pick_split(ctx, p.M, p.N, p.K, fast ? SPLIT_SPARE : SPLIT_SPARE_SLOW);
     if (split > 1) return qdit_launch_gemm_sk(ctx, A, W, p, a_unsigned, split, false);
   }
   switch (pick_bn(p.M, p.N, ctx->num_sms, ctx->opt[QDIT_OPT_GEMM_BN])) {

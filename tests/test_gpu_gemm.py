@@ -482,14 +482,15 @@ def test_code_output_leaves_the_padding_of_its_rows_alone(q, ctx, N, ldo):
 
 
 @pytest.mark.parametrize("M,N,K", [
-    (1, 8, 512),         # four k-blocks: too short to split
-    (8, 8, 1024),        # shortest split reduction: one tile, four CTAs with two k-blocks each
+    (1, 8, 512),         # one small tile, four k-blocks: not split
+    (8, 8, 1024),        # f32, per-token, raw: shortest split reduction, one tile, four CTAs with two k-blocks each
+    (8, 8, 3072),        # the others: 24 k-blocks over six CTAs
     (64, 392, 4608),     # six CTAs per tile, ragged columns (392 = 6 * 64 + 8)
-    (100, 1152, 1040),   # four CTAs per tile: ragged rows, 9 k-blocks, the last one short
+    (100, 1152, 1040),   # 9 k-blocks, the last one short: four CTAs per tile with those outputs, else whole
+    (200, 832, 3440),    # four CTAs per tile: ragged rows, 27 k-blocks, the last one short
     (256, 1152, 4608),   # three CTAs per tile: row groups 6, 5, 5
-    (300, 1152, 800),    # seven k-blocks: too short to split
-    (300, 1152, 1536),   # two CTAs per tile: ragged rows
-    (512, 1152, 4608),   # two CTAs per tile: 72 tiles
+    (300, 1152, 800),    # seven k-blocks: not split
+    (300, 1152, 5120),   # two CTAs per tile: ragged rows
     (1040, 2312, 256),   # channel-major kernel: ragged rows and columns
     (1025, 2304, 1152),
     (4000, 1160, 1152),  # channel-major gated layer: 32 x 7 token-major tiles of 192 exceed one wave
