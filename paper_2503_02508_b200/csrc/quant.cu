@@ -7,10 +7,14 @@ namespace {
 
 using namespace qd;
 
-// A quantizer of more CTAs than this neither starts early nor lets its successor: a launch latency is nothing to it, and the
-// layer that follows ran slower for it (64417 x 4608 x 1152, quantizer and layer: 478 us overlapped, 458 not; 64417 x 3456 x 1152: 362 and 350;
-// 4096 CTAs are about three waves).
-constexpr unsigned OVERLAP_CTAS = 4096;
+// Quantizers of few CTAs start before the kernel in front of them has ended.  More of them would be packed onto the SMs that this kernel
+// leaves free, eight to an SM, and those set the pace when it is over: per-token quantizer and layer, 1024 x 1152 x 4608 (128 CTAs)
+// 35.6 us started early, 22.5 not; 512 rows (64) 21.8 and 14.2; 256 rows (32) 12.8 and 13.4.  The static one has a fourth of that work
+// per CTA: 2048 x 3456 x 1152 (576 CTAs) 14.3 and 13.5, 512 rows (144) 8.5 and 7.9, 64 x 1152 x 4608 (72) 7.9 and 8.8.
+constexpr unsigned EARLY_CTAS = 128, EARLY_TOKEN_CTAS = 48;
+// A static quantizer of more CTAs than this does not let its successor start early either (64417 x 4608 x 1152, 18000 CTAs, quantizer
+// and layer: 478 us with it, 458 without; 64417 x 3456 x 1152: 362 and 350; no difference from 1000 to 4600 CTAs).
+constexpr unsigned RELEASE_CTAS = 4096;
 
 // ----------------------------------------------------------------------------- activation quantizer
 // One thread per 16 consecutive elements of a row (two 8-element halves); K % 8 == 0.
@@ -18,7 +22,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) act_quant_kernel(const T* __restrict__ x, int64_t M, int64_t K, int64_t ldx,
                                                         QuantArgs qa, uint8_t* __restrict__ q, int64_t ldq) {
   grid_dependency_wait();
-  if (gridDim.x <= OVERLAP_CTAS) grid_dependency_release();
+  if (gridDim.x <= RELEASE_CTAS) grid_dependency_release();
   const int64_t chunks_per_row = (K + 15) / 16;
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (idx >= M * chunks_per_row) return;
@@ -488,8 +492,8 @@ void launch_ln(qdit_ctx* ctx, const void* x, int64_t M, int D, int64_t T, float 
 
 namespace {
 template <typename... KArgs, typename... Args>
-cudaError_t launch_act_quant(qdit_ctx* ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args&&... args) {
-  if (grid.x <= OVERLAP_CTAS) return qdit_launch_overlapped(ctx, kernel, grid, block, smem, args...);
+cudaError_t launch_act_quant(qdit_ctx* ctx, unsigned early_ctas, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args&&... args) {
+  if (grid.x <= early_ctas) return qdit_launch_overlapped(ctx, kernel, grid, block, smem, args...);
   kernel<<<grid, block, smem, ctx->stream>>>(static_cast<KArgs>(args)...);
   return cudaGetLastError();
 }
@@ -520,7 +524,7 @@ int32_t quant_dynamic(qdit_ctx* ctx, const T* x, int64_t M, int64_t K, int64_t l
   QDIT_TRY(qdit_after_launch(ctx, "partials_to_scale_kernel"));
   const QuantArgs qa = make_quant_args(qdit_qparams{1.0f, 0, -127, 127}, scale);
   const int64_t threads = M * ((K + 15) / 16);
-  QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, act_quant_kernel<T>, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0, x, M, K, ldx, qa,
+  QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_CTAS, act_quant_kernel<T>, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0, x, M, K, ldx, qa,
                                               q, ldq));
   return qdit_after_launch(ctx, "act_quant_kernel");
 }
@@ -544,7 +548,7 @@ int32_t qdit_quantize_act_dev(qdit_ctx* ctx, const float* x, int64_t M, int64_t 
   if (M == 0 || K == 0) return QDIT_OK;
   const QuantArgs qa = make_quant_args(qp, scale_dev);
   const int64_t threads = M * ((K + 15) / 16);
-  QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, act_quant_kernel<float>, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0, x, M, K, K, qa, q, K));
+  QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_CTAS, act_quant_kernel<float>, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0, x, M, K, K, qa, q, K));
   return qdit_after_launch(ctx, "act_quant_kernel");
 }
 
@@ -570,10 +574,10 @@ int32_t qdit_quantize_act(qdit_ctx* ctx, const void* x, int x_dtype, int64_t M, 
     if (!dyn_scale) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "per-token mode needs dyn_scale [M]");
     const unsigned grid = static_cast<unsigned>((M + 7) / 8);
     if (x_dtype == QDIT_BF16)
-      QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, act_quant_token_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, static_cast<const __nv_bfloat16*>(x), M, K, ldx, dyn_scale,
+      QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_TOKEN_CTAS, act_quant_token_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, static_cast<const __nv_bfloat16*>(x), M, K, ldx, dyn_scale,
                                                                         static_cast<uint8_t*>(q), ldq));
     else
-      QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, act_quant_token_kernel<float>, dim3(grid), dim3(256), 0, static_cast<const float*>(x), M, K, ldx, dyn_scale,
+      QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_TOKEN_CTAS, act_quant_token_kernel<float>, dim3(grid), dim3(256), 0, static_cast<const float*>(x), M, K, ldx, dyn_scale,
                                                                    static_cast<uint8_t*>(q), ldq));
     return qdit_after_launch(ctx, "act_quant_token_kernel");
   } else if (mode == QDIT_QUANT_DYNAMIC) {
@@ -586,10 +590,10 @@ int32_t qdit_quantize_act(qdit_ctx* ctx, const void* x, int x_dtype, int64_t M, 
   const unsigned grid = static_cast<unsigned>((threads + 255) / 256);
   ProfScope prof(ctx, QDIT_PROF_ACT_QUANT, static_cast<double>(M) * K * (esz + 1.0));
   if (x_dtype == QDIT_BF16)
-    QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, act_quant_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, static_cast<const __nv_bfloat16*>(x), M, K, ldx, qa,
+    QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_CTAS, act_quant_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, static_cast<const __nv_bfloat16*>(x), M, K, ldx, qa,
                                                                    static_cast<uint8_t*>(q), ldq));
   else
-    QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, act_quant_kernel<float>, dim3(grid), dim3(256), 0, static_cast<const float*>(x), M, K, ldx, qa,
+    QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_CTAS, act_quant_kernel<float>, dim3(grid), dim3(256), 0, static_cast<const float*>(x), M, K, ldx, qa,
                                                            static_cast<uint8_t*>(q), ldq));
   return qdit_after_launch(ctx, "act_quant_kernel");
 }
