@@ -524,7 +524,8 @@ int32_t quant_dynamic(qdit_ctx* ctx, const T* x, int64_t M, int64_t K, int64_t l
   QDIT_TRY(qdit_after_launch(ctx, "partials_to_scale_kernel"));
   const QuantArgs qa = make_quant_args(qdit_qparams{1.0f, 0, -127, 127}, scale);
   const int64_t threads = M * ((K + 15) / 16);
-  QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_CTAS, act_quant_kernel<T>, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0, x, M, K, ldx, qa,
+  // (the launch in front is one CTA: nothing to be packed beside)
+  QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, RELEASE_CTAS, act_quant_kernel<T>, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0, x, M, K, ldx, qa,
                                               q, ldq));
   return qdit_after_launch(ctx, "act_quant_kernel");
 }
