@@ -86,7 +86,7 @@ int64_t qdit_launch_count(const qdit_ctx* ctx);
  *                                   as fit a 4 GB modulation table, -1 step by step, n > 0 at most n (read by
  *                                   qdit_sampler_create)
  *   QDIT_OPT_ATTN_STAGGER_NS        0..20000 (default 2000): accepted and reported, without effect: the attention kernel
- *                                   keeps one CTA per SM and staggers its two softmax streams itself */
+ *                                   keeps one CTA per SM */
 enum {
   QDIT_OPT_PDL = 0, QDIT_OPT_GEMM_BN = 1, QDIT_OPT_GEMM_T = 2, QDIT_OPT_GEMM_GENERIC_EPILOGUE = 3, QDIT_OPT_ATTN = 4,
   QDIT_OPT_CONDITIONING_CHUNK = 5, QDIT_OPT_ATTN_STAGGER_NS = 6, QDIT_OPT_COUNT = 7
