@@ -47,8 +47,8 @@ struct GemmParams {
 // Epilogue classes.  The three block-level layers get kernels whose epilogue flags are compile-time
 // constants (no flag branches, no dead registers, a smaller instruction footprint: instruction-fetch stalls
 // were a top stall reason of the all-in-one kernel); class 0 keeps the flags as run-time values.
-//   1 bias -> bf16; 2 bias, GELU -> 8-bit codes; 3 (and 4, its short-reduction form in gemm_i8_t.cu) bias, optional cache
-//   copy, x gate, + residual -> bf16; channel-major kernel only: 5 as 1 with per-token activation scales; 6 bias -> f32
+//   1 bias -> bf16; 2 bias, GELU -> 8-bit codes; 3 (and 4, its short-reduction form in gemm_i8_t.cu and gemm_i8_p.cu) bias,
+//   optional cache copy, x gate, + residual -> bf16; pair kernel only: 5 as 1 with per-token activation scales; 6 bias -> f32
 constexpr uint32_t EPI_FLAGS_QKV = QDIT_EPI_BIAS | QDIT_EPI_OUT_BF16;
 constexpr uint32_t EPI_FLAGS_FC1 = QDIT_EPI_BIAS | QDIT_EPI_GELU | QDIT_EPI_QUANT_OUT;
 constexpr uint32_t EPI_FLAGS_GATED = QDIT_EPI_BIAS | QDIT_EPI_GATE | QDIT_EPI_RESIDUAL | QDIT_EPI_OUT_BF16;
@@ -273,6 +273,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc
 
 // Channel-major accumulator kernel (gemm_i8_t.cu): tiles of 128 channels x bt tokens, bt in {128, 256}.
 int32_t qdit_launch_gemm_t(qdit_ctx* ctx, const void* A, const void* W, qgemm::GemmParams& p, bool a_unsigned, int bt);
+
+// Token-major tiles of 256 tokens by pairs of CTAs (gemm_i8_p.cu), for the epilogue classes 1, 2 (width and pitch multiples of 16), 3 (samples
+// of whole 32-token chunks), 5 and 6.
+int32_t qdit_launch_gemm_pair(qdit_ctx* ctx, const void* A, const void* W, const qgemm::GemmParams& p, bool a_unsigned);
 
 // Token-major tiles of 128 x 64 whose reduction is split over clusters of `split` (2, 3, 4 or 6) CTAs (gemm_i8_sk.cu);
 // K > (split - 1) * 128; packed4: W holds 4-bit codes two per byte.  qdit_gemm_sk_clusters: clusters of that size the device holds at once.

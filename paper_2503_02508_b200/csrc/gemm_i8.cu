@@ -351,17 +351,24 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
   const int cls = epi_class(p.flags);
   const bool row_scale = (flags & QDIT_EPI_ROW_SCALE) != 0;
   if (!row_scale && ctx->opt[QDIT_OPT_GEMM_T] != 0) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, ctx->opt[QDIT_OPT_GEMM_T]);
-  // Kernel choice: layers with many rows run channel-major with 128 x 256 tiles when their epilogue has a staged form there
-  // (a TMA store per 32-token chunk; 8192 rows, us, against token-major: QKV 30 / 33, fc1 39 / 48, proj 17 / 20, fc2 39 /
-  // 46, per-token scales 30 / 45, f32 output 37 / 51); few rows, narrow outputs and every other epilogue run token-major.
-  // The gated layers are narrow (1152 columns): up to the row count where 128 x 192 token-major tiles fill one wave, the
-  // smaller tiles spread over more SMs (fc2 at 1024 / 2048 / 3072 rows: 8.8 / 14.0 / 17.8 us against 17.1 / 20.0 / 20.1).
-  if (ctx->opt[QDIT_OPT_GEMM_BN] == 0 && p.M >= 1024 && !(row_scale && ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE])) {
-    // (8-bit rows leave through TMA stores of whole 16-byte pieces: the width and the pitch have to be multiples of 16)
-    const bool staged_form = cls == 1 || cls == 5 || cls == 6 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0);
-    if (staged_form && p.N >= 2304) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
-    if (cls == 3 && p.N >= 1024 && p.tokens % 32 == 0 && ((p.M + BM - 1) / BM) * ((p.N + 191) / 192) > ctx->num_sms)
-      return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
+  // Kernel choice.  A layer whose 128 x 192 tiles fill no more than one wave runs token-major, one CTA per tile (below): pairs gain
+  // nothing there (2048 x 3456 x 384: 4.8 us against 5.0, 1024 x 1152 x 1152 gated 5.3 and 6.5).  From the second wave on pairs of CTAs
+  // are faster (us, single CTAs / pairs: QKV of XL/2 2048 rows 11.0 / 9.0, 8192 26.7 / 24.0, 65536 222 / 182; fc1 40.1 / 35.4 and
+  // 310 / 295; fc2 5000 rows 31.2 / 24.4, 8192 35.6 / 34.8, 65536 276 / 256; proj 14.9 / 11.3, 15.2 / 15.1, 117 / 113).  Per-token
+  // scales and f32 output take pairs earlier, because their token-major epilogue decides at run time what to do (512 x 3456 x 1152:
+  // 8.6 / 5.9 and 8.2 / 6.4), unless the split reduction, which splits the epilogue too, serves them.  Between one and two waves of
+  // token-major tiles lie row counts at which 128 x 256 channel-major tiles make exactly one (QKV 1280 rows: 7.2 against 7.7 us, with
+  // per-token scales 11.0 / 12.1; proj and fc2 at 4096: 9.7 / 10.5 and 18.4 / 20.3).
+  if (ctx->opt[QDIT_OPT_GEMM_BN] == 0 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE]) {
+    // (8-bit rows leave through TMA stores of whole 16-byte pieces, and a 32-token chunk of a gated layer has one gate row)
+    const bool staged = cls == 1 || cls == 5 || cls == 6 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0) || (cls == 3 && p.tokens % 32 == 0);
+    const bool slow = cls == 5 || cls == 6;
+    const bool one_wave = static_cast<int64_t>((p.M + BM - 1) / BM) * ((p.N + 191) / 192) <= ctx->num_sms;
+    if (staged && (slow ? p.M > BM && pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) == 1 : !one_wave)) {
+      const bool t_wave = p.M >= 1024 && static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) <= ctx->num_sms;
+      if (t_wave && (cls == 3 || (cls != 2 && p.N >= 2304))) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
+      return qdit_launch_gemm_pair(ctx, A, W, p, a_unsigned);
+    }
   }
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0) {
     const bool fast = cls >= 1 && cls <= 3 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE];

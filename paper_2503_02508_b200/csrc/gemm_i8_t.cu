@@ -25,11 +25,8 @@
 // stores (warp-level stores of 64-byte row pieces reach 4.2 TB/s on this chip, TMA stores of the same tiles
 // 6.7 TB/s, and they do not hold the issuing warp), and the residual of the gated epilogue arrives the same way
 // in reverse (TMA load one chunk ahead, ldmatrix.trans).
-// The epilogue that writes 8-bit codes (bias + GELU -> codes, class 2) keeps a channel per thread (per-channel
-// scalars, tcgen05.ld 32x32b) and writes each code with a one-byte shared-memory store into a tile of 32 tokens x 128
-// channels that the four quadrant warps of a token chunk fill together; one thread hands it to a TMA store (full
-// 128-byte rows; per-thread global stores of this layout are 32-byte pieces of 8 rows, which held that layer at the
-// speed of its stores).
+// It serves the row counts at which its tiles make exactly one wave of the chip (see the dispatch in gemm_i8.cu); pairs of CTAs
+// (gemm_i8_p.cu) serve the others.
 #include "gemm_common.cuh"
 
 
@@ -54,11 +51,7 @@ struct TWarps {
   // two 2 KB tiles of 32 tokens x 32 channels bf16 per warp: class 1 two output tiles used in turn; class 3 the residual
   // tile and one shared by the cache copy and the output
   static constexpr int STAGING_PER_WARP = STAGED ? 2 * 2048 : 0;
-  // class 2 (8-bit codes): the four quadrant warps that work on the same token chunk share a tile of 32 tokens x 128
-  // channels (4 KB), two tiles used in turn per group of four
-  static constexpr bool GROUPED = EPI == 2;
-  static constexpr int GROUP_TILE_BYTES = 32 * BC;
-  static constexpr int STAGING_BYTES = STAGED ? EPI_WARPS * STAGING_PER_WARP : GROUPED ? SPLIT * 2 * GROUP_TILE_BYTES : 0;
+  static constexpr int STAGING_BYTES = STAGED ? EPI_WARPS * STAGING_PER_WARP : 0;
 };
 
 template <int BT, int EPI>
@@ -126,37 +119,6 @@ __device__ __forceinline__ void epilogue_chunk_t(const GemmParams& p, const uint
         }
       }
     }
-  }
-}
-
-// GELU layer (bias + GELU -> 8-bit codes): the math runs channel-major with scalar parameters; the code of token j
-// goes to byte (j, col) of the group's tile with a one-byte store (a warp instruction writes 32 consecutive bytes).
-template <int EPI>
-__device__ __forceinline__ void epilogue_chunk_t_codes(const GemmParams& p, const uint32_t (&v)[32], float sc, float bias, int zcs,
-                                                       float o_inv, uint32_t tile_col_addr) {
-  const uint32_t flags = epi_flags<EPI>(p);
-  // The epilogue of the GELU layer has the most arithmetic per element, so work that a symmetric quantizer does not
-  // need (zero-point terms) is skipped through branches that are uniform over the whole grid.
-  float f[32];
-  if (p.a_zp == 0) {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) f[j] = static_cast<float>(static_cast<int>(v[j]));
-  } else {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) f[j] = static_cast<float>(static_cast<int>(v[j]) - zcs);
-  }
-  const float lo_f = p.o_qmin - p.o_zp, hi_f = p.o_qmax - p.o_zp;
-  const uint32_t zp = static_cast<uint32_t>(static_cast<int>(p.o_zp));
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    float x = (flags & QDIT_EPI_BIAS) ? __fmaf_rn(f[j], sc, bias) : __fmul_rn(f[j], sc);
-    if (flags & QDIT_EPI_GELU) x = gelu_tanh_f(x);
-    // clip(rne(t) + z, qmin, qmax) == rne(clamp(t, qmin - z, qmax - z)) + z; adding 1.5 * 2^23 rounds to nearest-even and
-    // leaves the integer in the low mantissa bits; the low byte is the stored code
-    const float q = fminf(fmaxf(__fmul_rn(x, o_inv), lo_f), hi_f);
-    uint32_t m = static_cast<uint32_t>(__float_as_int(__fadd_rn(q, 12582912.0f)));
-    if (zp != 0u) m += zp;
-    asm volatile("st.shared.u8 [%0], %1;" ::"r"(tile_col_addr + static_cast<uint32_t>(j * BC)), "r"(m) : "memory");
   }
 }
 
@@ -249,7 +211,7 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sW = smem;
   uint8_t* sX = smem + STAGES * C::W_BYTES;
-  uint8_t* staging = smem + STAGES * C::STAGE_BYTES;  // classes 1, 3: [EPI_WARPS][tiles][2 KB]; class 2: [SPLIT][2][4 KB]; 1024-byte aligned
+  uint8_t* staging = smem + STAGES * C::STAGE_BYTES;  // [EPI_WARPS][2 tiles of 2 KB]; 1024-byte aligned
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(staging + TW::STAGING_BYTES);
   uint64_t* empty_bar = full_bar + STAGES;
   uint64_t* tfull_bar = empty_bar + STAGES;
@@ -295,16 +257,10 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
   // tiles: channel block fastest, so CTAs running together share the activation tile
   const int num_c_tiles = p.num_n_tiles, total_tiles = p.num_m_tiles * p.num_n_tiles;
 
-  // The producer and the issuer look at their next barrier before they issue the work of the current one.  One elected
-  // thread runs each role; only next to the code epilogue, whose twelve warps are busy all the time, the whole warp does, and
-  // elects at each issue (fc1 at 65536 / 8192 rows: 300 / 38.8 us against 316 / 40.0; QKV, proj and fc2 lose 1-4 % that way).
-  constexpr bool WARP_ROLES = TW::GROUPED;
-  auto wait_for = [&](bool seen, uint64_t* bar, uint32_t parity) -> bool {
-    if constexpr (WARP_ROLES) return mbar_wait_seen(seen, bar, parity, abort_flag, p.status);
-    return seen || mbar_wait(bar, parity, abort_flag, p.status);
-  };
+  // The producer and the issuer, one elected thread each, look at their next barrier before they issue the work of the current one.
+  auto wait_for = [&](bool seen, uint64_t* bar, uint32_t parity) { return seen || mbar_wait(bar, parity, abort_flag, p.status); };
   if (warp == 0) {
-    if (WARP_ROLES || elect_one()) {
+    if (elect_one()) {
       // ------------------------------------------------------------------ TMA producer
       int stage = 0;
       uint32_t phase = 0;
@@ -316,11 +272,9 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
           if (!wait_for(seen, &empty_bar[stage], phase ^ 1u)) { ok = false; break; }
           const bool wrap = stage + 1 == STAGES;
           seen = mbar_test_wait(&empty_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 0u : 1u));
-          if (!WARP_ROLES || elect_one()) {
-            mbar_expect_tx(&full_bar[stage], C::STAGE_BYTES);
-            tma_load_2d(sW + stage * C::W_BYTES, &tmap_w, kb * BK, c0, &full_bar[stage]);
-            tma_load_2d(sX + stage * C::X_BYTES, &tmap_x, kb * BK, t0, &full_bar[stage]);
-          }
+          mbar_expect_tx(&full_bar[stage], C::STAGE_BYTES);
+          tma_load_2d(sW + stage * C::W_BYTES, &tmap_w, kb * BK, c0, &full_bar[stage]);
+          tma_load_2d(sX + stage * C::X_BYTES, &tmap_x, kb * BK, t0, &full_bar[stage]);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
@@ -329,7 +283,7 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    if (WARP_ROLES || elect_one()) {
+    if (elect_one()) {
       // ------------------------------------------------------------------ MMA issuer
       int stage = 0;
       uint32_t phase = 0;
@@ -348,18 +302,15 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
           tc_fence_after();
           const uint64_t w_desc = umma_desc_k_sw128(smem_u32(sW + stage * C::W_BYTES));
           const uint64_t x_desc = umma_desc_k_sw128(smem_u32(sX + stage * C::X_BYTES));
-          if (!WARP_ROLES || elect_one()) {
 #pragma unroll
-            for (int k = 0; k < BK / UMMA_K; ++k) {
-              umma_i8(d_tmem, w_desc + static_cast<uint64_t>(k * (UMMA_K >> 4)),
-                      x_desc + static_cast<uint64_t>(k * (UMMA_K >> 4)), idesc, (kb | k) != 0 ? 1u : 0u);
-            }
-            umma_commit(&empty_bar[stage]);
+          for (int k = 0; k < BK / UMMA_K; ++k) {
+            umma_i8(d_tmem, w_desc + static_cast<uint64_t>(k * (UMMA_K >> 4)),
+                    x_desc + static_cast<uint64_t>(k * (UMMA_K >> 4)), idesc, (kb | k) != 0 ? 1u : 0u);
           }
-          if (WARP_ROLES) __syncwarp();
+          umma_commit(&empty_bar[stage]);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok && (!WARP_ROLES || elect_one())) umma_commit(&tfull_bar[as]);
+        if (ok) umma_commit(&tfull_bar[as]);
       }
     }
   } else {
@@ -551,11 +502,6 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
       if (r_inflight) mbar_wait(rbar, r_phase, abort_flag, p.status);
       if (lane == 0) tma_store_wait_all();
     } else {
-      // class 2: the tile pair of this warp's group (the four quadrant warps with the same `part`), used in turn
-      uint8_t* const gtile = staging + part * (2 * TW::GROUP_TILE_BYTES);
-      const bool issuer = quad == 0 && lane == 0;   // one thread per group hands the tiles to TMA
-      int turn = 0;
-      if (TW::GROUPED && issuer) tma_prefetch_desc(&tmap_out);
       int it = 0;
       for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
         const int as = it & 1;
@@ -593,27 +539,9 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             if (lane == 0) mbar_arrive_relaxed(&tempty_bar[as]);
           }
           const int m_base = t0 + c * 32;
-          if (m_base < p.M) {   // uniform over the four warps of a group: they work on the same token chunk
-            if (TW::GROUPED) {
-              uint8_t* const buf = gtile + turn * TW::GROUP_TILE_BYTES;
-              epilogue_chunk_t_codes<EPI>(p, v, sc, bias, zcs, o_inv, smem_u32(buf) + static_cast<uint32_t>(quad * 32 + lane));
-              fence_async_smem();
-              // the store that used the other tile (issued one chunk ago) has read it before anybody passes the barrier,
-              // so the next chunk may overwrite it
-              if (issuer) tma_store_wait_read<0>();
-              asm volatile("bar.sync %0, %1;" ::"r"(1 + part), "r"(128) : "memory");
-              if (issuer) {
-                tma_store_2d(&tmap_out, buf, (tile % num_c_tiles) * BC, m_base);
-                tma_store_commit();
-              }
-              turn ^= 1;
-            } else if (n_ok) {
-              epilogue_chunk_t<EPI>(p, v, n, m_base, sc, bias, zcs, o_inv);
-            }
-          }
+          if (m_base < p.M && n_ok) epilogue_chunk_t<EPI>(p, v, n, m_base, sc, bias, zcs, o_inv);
         }
       }
-      if (TW::GROUPED && issuer) tma_store_wait_all();
     }
   }
 
@@ -634,7 +562,6 @@ int32_t launch_t_epi(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p,
   QDIT_TRY(qdit_get_tmap(ctx, A, p.M, p.K, p.K, BT, BK, 1, 1, &tx));
   // staged epilogues: 32 tokens x 32 channels bf16 tiles (64-byte rows, 64B swizzle) of the output, the cache slot and the residual
   CUtensorMap to = tx, tc = tx, tr = tx;
-  if (TWarps<EPI>::GROUPED) QDIT_TRY(qdit_get_tmap(ctx, p.out, p.M, p.N, p.ldo, 32, BC, 0, 1, &to));   // 32 tokens x 128 channels of bytes
   if (EPI == 6) {
     QDIT_TRY(qdit_get_tmap(ctx, p.out, p.M, p.N, p.ldo, 16, 32, 1, 4, &to));   // 16 tokens x 32 channels of f32
     tc = tr = to;
@@ -662,7 +589,6 @@ template <int BT>
 int32_t launch_t(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p, bool a_unsigned) {
   switch (ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE] ? 0 : epi_class(p.flags)) {
     case 1: return launch_t_epi<BT, 1>(ctx, A, W, p, a_unsigned);
-    case 2: return launch_t_epi<BT, 2>(ctx, A, W, p, a_unsigned);
     case 3:
       // A short reduction leaves the gated epilogue (residual in, two tiles out per chunk) as the longer part of a tile,
       // and with few tiles per CTA the last one is exposed: three warps per lane quadrant instead of two shorten it,

@@ -562,3 +562,57 @@ def test_packed_weights_with_a_split_reduction(q, ctx, M, N, K, kind):
                 q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 0)
         q.qdit_sync(ctx)
     assert torch.equal(out[0], out[1]) and torch.equal(cache[0], cache[1])
+
+
+@pytest.mark.parametrize("M,N,K,T", [
+    (129, 392, 400, 32),        # f32 and per-token scales: one pair, its second CTA one row, ragged channels, a short last k-block
+    (4801, 1160, 1152, 64),     # second wave of gated tiles: a last row of tiles with one token, a last column with 8 channels
+    (5000, 1152, 2304, 1000),   # gated by the long-reduction form, samples longer than a tile; 1000 % 32 != 0: not by pairs
+    (5120, 1152, 2304, 256),
+    (1300, 4624, 128, 32),      # one k-block: the ring is longer than the reduction
+    (19200, 384, 384, 256),     # narrow layer, many tiles per pair
+    (300, 44000, 1152, 32),     # weights of more than 48 MB: tiles along the tokens first
+])
+@pytest.mark.parametrize("kind,zp", [("f32", 0), ("bf16", 0), ("bf16", 131), ("row", 0), ("gelu", 0), ("gelu", 131), ("gated", 0), ("gated_nocache", 131)])
+def test_pair_kernel_gives_the_bits_of_the_token_major_kernel(q, ctx, M, N, K, T, kind, zp):
+    """Pairs of CTAs: whatever tile width the rule takes, exact integer sums and the same f32 epilogue as the plain token-major
+    kernel with run-time epilogue flags; the padding of the rows stays untouched."""
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    lo, hi = (0, 256) if zp else (-127, 128)
+    A = torch.randint(lo, hi, (M, K), generator=g, device="cuda").to(torch.uint8 if zp else torch.int8)
+    W = torch.randint(-127, 128, (N, K), generator=g, device="cuda", dtype=torch.int8)
+    ws, bi = torch.rand(N, generator=g, device="cuda") * 2e-4 + 1e-5, torch.randn(N, generator=g, device="cuda") * 0.5
+    colsum = W.sum(dim=1, dtype=torch.int32)
+    gate, resid = torch.randn(-(-M // T), N, generator=g, device="cuda") * 0.5, torch.randn(M, N, generator=g, device="cuda").bfloat16()
+    rows = torch.rand(M, generator=g, device="cuda") + 0.1
+    flags = {"f32": q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_F32, "bf16": q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_BF16,
+             "row": q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_BF16 | q.QDIT_EPI_ROW_SCALE,
+             "gelu": q.QDIT_EPI_BIAS | q.QDIT_EPI_GELU | q.QDIT_EPI_QUANT_OUT,
+             "gated": q.QDIT_EPI_BIAS | q.QDIT_EPI_GATE | q.QDIT_EPI_RESIDUAL | q.QDIT_EPI_OUT_BF16 | q.QDIT_EPI_CACHE_STORE,
+             "gated_nocache": q.QDIT_EPI_BIAS | q.QDIT_EPI_GATE | q.QDIT_EPI_RESIDUAL | q.QDIT_EPI_OUT_BF16}[kind]
+    dtype = {"f32": torch.float32, "gelu": torch.int8}.get(kind, torch.bfloat16)
+    ldo = -(-N // 16) * 16 + 16
+    qp = q.qparams(0.03, zp, 0, 255) if zp else q.qparams(0.03)
+
+    def run():
+        out = torch.full((M, ldo), 3, dtype=dtype, device="cuda")
+        if kind.startswith("gated"):
+            out[:, :N] = resid                 # in place, as in a block
+        cache = torch.full((M, N), 3, dtype=torch.bfloat16, device="cuda")
+        epi = q.epilogue(w_scale=ws, w_colsum=colsum, bias=bi, gate=gate, ld_gate=N, tokens_per_sample=T, residual=out,
+                         cache_out=cache if kind == "gated" else None, out_qp=q.qparams(0.02, 5, -100, 90), a_scale_rows=rows)
+        torch.cuda.synchronize()
+        q.qdit_w8a8_linear(ctx, A, W, M, N, K, qp, None, flags, epi, out, ldo)
+        q.qdit_sync(ctx)
+        return out, cache
+
+    got = run()
+    try:
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 64)
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, 1)
+        ref = run()
+    finally:
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 0)
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, 0)
+    assert torch.equal(got[0], ref[0])
+    assert torch.equal(got[1], ref[1])
