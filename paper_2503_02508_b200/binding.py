@@ -479,5 +479,17 @@ def qdit_sampler_cache(s):
     return lib.qdit_sampler_cache(s)
 
 
+# The calls that a program makes per layer are marshalled natively (csrc/marshal.c); the functions above of the same names serve what
+# that does not take: keywords, numpy arrays, and every call that ends in an exception.
+_NATIVE = ("qdit_quantize_act", "qdit_w8a8_linear", "qdit_w4a8_linear", "qdit_attention", "qdit_adaln_modulate")
+try:
+    from . import _marshal
+except ImportError as e:
+    raise ImportError("the native marshalling module is missing: build it with `python paper_2503_02508_b200/build.py`") from e
+_WRAPPERS = tuple(globals()[_name] for _name in _NATIVE)
+_marshal.bind(tuple(C.cast(getattr(lib, n), _vp).value for n in _NATIVE), _WRAPPERS, check, qdit_qparams, qdit_epilogue)
+for _name in _NATIVE:
+    globals()[_name] = getattr(_marshal, _name)
+
 __all__ = [n for n in dir() if n.startswith(("qdit_", "QDIT_"))] + [
     "lib", "LIB_PATH", "EXPORTS", "QditError", "ptr", "check", "qparams", "epilogue"]

@@ -1,16 +1,19 @@
-"""Builds libqdit.so (sm_100a only) in-tree with nvcc.  `python paper_2503_02508_b200/build.py`."""
+"""Builds libqdit.so (sm_100a only) in-tree with nvcc, and the module that marshals Python arguments with the host compiler.
+`python paper_2503_02508_b200/build.py`."""
 from __future__ import annotations
 
 import concurrent.futures
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libqdit.so")
 OBJ = os.path.join(ROOT, "_build")
+MARSHAL = os.path.join(PKG, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -69,6 +72,10 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link of libqdit.so failed")
+    source = os.path.join(CSRC, "marshal.c")
+    if force or _stale(MARSHAL, [source, os.path.join(ROOT, "include", "qdit.h")]):
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"],
+                        "-I", os.path.join(ROOT, "include"), source, "-o", MARSHAL], check=True)
     return LIB
 
 
