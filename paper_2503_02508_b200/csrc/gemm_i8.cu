@@ -356,19 +356,18 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
   // are faster (us, single CTAs / pairs: QKV of XL/2 2048 rows 11.0 / 9.0, 8192 26.7 / 24.0, 65536 222 / 182; fc1 40.1 / 35.4 and
   // 310 / 295; fc2 5000 rows 31.2 / 24.4, 8192 35.6 / 34.8, 65536 276 / 256; proj 14.9 / 11.3, 15.2 / 15.1, 117 / 113).  Per-token
   // scales and f32 output take pairs earlier, because their token-major epilogue decides at run time what to do (512 x 3456 x 1152:
-  // 8.6 / 5.9 and 8.2 / 6.4), unless the split reduction, which splits the epilogue too, serves them.  Between one and two waves of
-  // token-major tiles lie row counts at which 128 x 256 channel-major tiles make exactly one (QKV 1280 rows: 7.2 against 7.7 us, with
-  // per-token scales 11.0 / 12.1; proj and fc2 at 4096: 9.7 / 10.5 and 18.4 / 20.3).
+  // 8.6 / 5.9 and 8.2 / 6.4), unless the split reduction, which splits the epilogue too, serves them.  Where 128 x 256
+  // channel-major tiles make exactly one wave they are better still (QKV 1280 rows: 7.2 against 7.7 us, with per-token scales
+  // 11.0 / 12.1; proj and fc2 at 4096: 9.7 / 10.5 and 18.4 / 20.3; one image of 1024 tokens: 1650 us against 1660 with QKV token-major).
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE]) {
     // (8-bit rows leave through TMA stores of whole 16-byte pieces, and a 32-token chunk of a gated layer has one gate row)
     const bool staged = cls == 1 || cls == 5 || cls == 6 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0) || (cls == 3 && p.tokens % 32 == 0);
     const bool slow = cls == 5 || cls == 6;
     const bool one_wave = static_cast<int64_t>((p.M + BM - 1) / BM) * ((p.N + 191) / 192) <= ctx->num_sms;
-    if (staged && (slow ? p.M > BM && pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) == 1 : !one_wave)) {
-      const bool t_wave = p.M >= 1024 && static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) <= ctx->num_sms;
-      if (t_wave && (cls == 3 || (cls != 2 && p.N >= 2304))) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
+    const bool t_wave = p.M >= 1024 && static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) <= ctx->num_sms;
+    if (staged && t_wave && (cls == 3 ? !one_wave : cls != 2 && p.N >= 2304)) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
+    if (staged && (slow ? p.M > BM && pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) == 1 : !one_wave))
       return qdit_launch_gemm_pair(ctx, A, W, p, a_unsigned);
-    }
   }
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0) {
     const bool fast = cls >= 1 && cls <= 3 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE];
