@@ -42,6 +42,9 @@ struct GemmParams {
   int64_t ldo;
   int* status;
   int num_m_tiles, num_n_tiles;
+  // The weights, their scales and biases, the gate and the quantizer scales were written two launches ago or earlier: a kernel that has
+  // started beside its predecessor may read them before it waits for it (every kernel lets its successor start after its own wait).
+  bool early;
 };
 
 // Epilogue classes.  The three block-level layers get kernels whose epilogue flags are compile-time
@@ -182,19 +185,18 @@ struct ChunkInputs {
   uint4 res[4];
 };
 
+// (a warp whose 32 rows lie wholly past M, in a ragged last tile, has no sample: it loads nothing)
 template <int EPI>
-__device__ __forceinline__ void prefetch_chunk(const GemmParams& p, int n, int row_base, int rsub, float a_scale,
-                                               ChunkInputs& in) {
-  const uint32_t flags = epi_flags<EPI>(p);
-  // a warp whose 32 rows lie wholly past M (ragged last tile) has no sample: it loads nothing
-  if (n < p.N && row_base < p.M && !(flags & QDIT_EPI_OUT_I32)) {
-    load_col_params<EPI>(p, n, row_base / p.tokens, a_scale, in.cp);
-    if (flags & QDIT_EPI_RESIDUAL) {
+__device__ __forceinline__ void prefetch_params(const GemmParams& p, int n, int row_base, float a_scale, ChunkInputs& in) {
+  if (n < p.N && row_base < p.M && !(epi_flags<EPI>(p) & QDIT_EPI_OUT_I32)) load_col_params<EPI>(p, n, row_base / p.tokens, a_scale, in.cp);
+}
+template <int EPI>
+__device__ __forceinline__ void prefetch_residual(const GemmParams& p, int n, int row_base, int rsub, ChunkInputs& in) {
+  if (n < p.N && row_base < p.M && (epi_flags<EPI>(p) & QDIT_EPI_RESIDUAL)) {
 #pragma unroll
-      for (int sidx = 0; sidx < 4; ++sidx) {
-        const int row = row_base + sidx * 8 + rsub;
-        if (row < p.M) in.res[sidx] = *reinterpret_cast<const uint4*>(p.residual + static_cast<int64_t>(row) * p.ldo + n);
-      }
+    for (int sidx = 0; sidx < 4; ++sidx) {
+      const int row = row_base + sidx * 8 + rsub;
+      if (row < p.M) in.res[sidx] = *reinterpret_cast<const uint4*>(p.residual + static_cast<int64_t>(row) * p.ldo + n);
     }
   }
 }
@@ -203,10 +205,11 @@ __device__ __forceinline__ void prefetch_chunk(const GemmParams& p, int n, int r
 // `tacc` = TMEM address of the accumulator stage (lane 0 of the CTA, first column); `release()` hands the
 // stage back to the MMA issuer once this warp has read its share.  `stg` = this warp's 4 KB staging patch.
 // The epilogue is bound by the latency chain of one chunk (global loads, TMEM load, transpose, stores), so
-// the tile's chunks are spread over as many warps as the register file allows.
+// the tile's chunks are spread over as many warps as the register file allows, and the global loads of a warp's first chunk
+// (`cur`) have been issued before the accumulator was waited for.
 template <int BN, int EPI, int SPLIT = EPI_SPLIT, typename Release>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc, int m0, int n0, int quad, int half,
-                                              uint32_t stg, int lane, float a_scale, float o_inv, Release release) {
+                                              uint32_t stg, int lane, float a_scale, float o_inv, ChunkInputs& cur, Release release) {
   const int cg = lane & 3;     // after the transpose: column group (8 columns) ...
   const int rsub = lane >> 2;  // ... of rows rsub, rsub + 8, rsub + 16, rsub + 24
   const uint32_t flags = epi_flags<EPI>(p);
@@ -229,8 +232,10 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc
     const int n = n0 + c * 32 + cg * 8;
     const bool col_ok = n < p.N;
     const uint32_t patch = stg;
-    ChunkInputs cur;
-    prefetch_chunk<EPI>(p, n, row_base, rsub, a_scale, cur);
+    if (c != half) {
+      prefetch_params<EPI>(p, n, row_base, a_scale, cur);
+      prefetch_residual<EPI>(p, n, row_base, rsub, cur);
+    }
     uint32_t v[32];
     __syncwarp();
     tmem_ld_32x32(taddr + static_cast<uint32_t>(c * 32), v);

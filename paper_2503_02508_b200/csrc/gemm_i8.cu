@@ -78,10 +78,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
-  // everything above touched only this CTA's shared and tensor memory; from here on the kernel reads what
-  // the previous kernel of the stream wrote
-  grid_dependency_wait();
-  grid_dependency_release();
+  // Everything above touched only this CTA's shared and tensor memory.  The roles that read what the previous kernel of the stream wrote
+  // wait for it themselves.
 
   const int num_kb = (p.K + BK - 1) / BK;
   const int total_tiles = p.num_m_tiles * p.num_n_tiles;
@@ -98,10 +96,26 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true, seen = true;   // seen: the stage about to be filled is known to be free
+      // the first stages' weights come while the previous kernel still runs
+      int ahead = 0;
+      if (p.early && static_cast<int>(blockIdx.x) < total_tiles) {
+        const int n0 = (static_cast<int>(blockIdx.x) % p.num_n_tiles) * BN;
+        for (; ahead < STAGES && ahead < num_kb; ++ahead) {
+          mbar_expect_tx(&full_bar[ahead], C::STAGE_BYTES);
+          tma_load_2d(sB + ahead * C::B_BYTES, &tmap_w, ahead * BK, n0, &full_bar[ahead]);
+        }
+      }
+      grid_dependency_wait();
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
         const int m0 = (tile / p.num_n_tiles) * BM;
         const int n0 = (tile % p.num_n_tiles) * BN;
         for (int kb = 0; kb < num_kb; ++kb) {
+          if (ahead > 0) {   // a fresh stage that has its weights
+            --ahead;
+            tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, kb * BK, m0, &full_bar[stage]);
+            if (++stage == STAGES) { stage = 0; phase ^= 1u; seen = false; }
+            continue;
+          }
           if (!wait_for(seen, &empty_bar[stage], phase ^ 1u)) { ok = false; break; }
           const bool wrap = stage + 1 == STAGES;
           seen = AHEAD && mbar_test_wait(&empty_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 0u : 1u));
@@ -154,20 +168,31 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const int quad = warp & 3;   // TMEM lane quadrant this warp may access
     const int half = e >> 2;     // this warp takes chunks half, half + EPI_SPLIT, ...
     const uint32_t stg = smem_u32(staging + e * (32 * 128));  // [32 rows][8 x 16 B], 16-byte index XOR (row & 7)
+    if (!p.early) grid_dependency_wait();
     const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
     float o_inv = 0.0f;
     if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
     int it = 0;
+    bool waited = !p.early;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
       const int as = it & 1;
       const uint32_t aphase = static_cast<uint32_t>(it >> 1) & 1u;
       const int m0 = (tile / p.num_n_tiles) * BM;
       const int n0 = (tile % p.num_n_tiles) * BN;
+      ChunkInputs cur;   // of this warp's first chunk
+      const int n = n0 + half * 32 + (lane & 3) * 8, row_base = m0 + quad * 32;
+      if (half < BN / 32) prefetch_params<EPI>(p, n, row_base, a_scale, cur);
+      if (!waited) {
+        grid_dependency_wait();
+        waited = true;
+      }
+      if (it == 0) grid_dependency_release();
+      if (half < BN / 32) prefetch_residual<EPI>(p, n, row_base, lane >> 2, cur);
       if (!mbar_wait(&tfull_bar[as], aphase, abort_flag, p.status)) break;
       __syncwarp();
       tc_fence_after();
       uint64_t* release_bar = &tempty_bar[as];
-      epilogue_tile<BN, EPI>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv,
+      epilogue_tile<BN, EPI>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur,
                         [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
   }
@@ -247,10 +272,10 @@ int pick_split(qdit_ctx* ctx, int M, int N, int K, int spare) {
 }  // namespace
 
 // Both linear layers: `packed4` = W holds 4-bit codes two per byte ([N, K/2]); `w8_scratch` = optional [N, K] int8
-// matrix the packed weights of a many-row layer are widened into first.
-static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K, qdit_qparams a_qp,
-                           const float* a_scale_dev, uint32_t flags, const qdit_epilogue* epi, void* out, int64_t ldo,
-                           bool packed4, void* w8_scratch) {
+// matrix the packed weights of a many-row layer are widened into first; `early`: see GemmParams.
+int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K, qdit_qparams a_qp,
+                         const float* a_scale_dev, uint32_t flags, const qdit_epilogue* epi, void* out, int64_t ldo,
+                         bool packed4, void* w8_scratch, bool early) {
   if (!ctx) return QDIT_ERR_INVALID_ARG;
   if (M < 0 || N < 0 || K < 0) return qdit_fail(ctx, QDIT_ERR_SHAPE, "negative size");
   if (M == 0 || N == 0) return QDIT_OK;
@@ -286,6 +311,7 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
   p.ldo = ldo;
   p.status = ctx->d_status;
   p.tokens = 1;
+  p.early = early;
   if (!(flags & QDIT_EPI_OUT_I32)) {
     if (!epi || !epi->w_scale) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "epilogue with w_scale is required");
     if (!aligned16(epi->w_scale)) return qdit_fail(ctx, QDIT_ERR_ALIGN, "w_scale must be 16-byte aligned");
@@ -340,6 +366,7 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
     if (w8_scratch && M >= 1024) {
       QDIT_TRY(qdit_unpack_weight_int4(ctx, W, N, K, w8_scratch));
       W = w8_scratch;
+      p.early = false;
     } else {
       // (few tiles split by the same rule as below: 256 / 512 x 1152 x 4608 take 8.5 / 10.3 us against 17.7 / 17.9)
       const int split = ctx->opt[QDIT_OPT_GEMM_BN] == 0 ? pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) : 1;
@@ -384,11 +411,11 @@ static int32_t linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t 
 extern "C" int32_t qdit_w8a8_linear(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K,
                                     qdit_qparams a_qp, const float* a_scale_dev, uint32_t flags,
                                     const qdit_epilogue* epi, void* out, int64_t ldo) {
-  return linear_impl(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, false, nullptr);
+  return qdit_linear_impl(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, false, nullptr, false);
 }
 
 extern "C" int32_t qdit_w4a8_linear(qdit_ctx* ctx, const void* A, const void* W_packed, int64_t M, int64_t N, int64_t K,
                                     qdit_qparams a_qp, const float* a_scale_dev, uint32_t flags,
                                     const qdit_epilogue* epi, void* out, int64_t ldo, void* w8_scratch) {
-  return linear_impl(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, true, w8_scratch);
+  return qdit_linear_impl(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, true, w8_scratch, false);
 }

@@ -105,9 +105,39 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
   __syncthreads();
   tc_fence_after();
   cluster_arrive();   // every CTA of the cluster has started: waited for before the first remote store
-  const uint32_t tmem = *tmem_holder;
-  grid_dependency_wait();
-  grid_dependency_release();
+  const uint32_t tmem = *tmem_holder;   // (the roles that read what the previous kernel wrote wait for it themselves)
+
+  // Work of this warp after the exchange: 8 rows x 32 columns at a time; what its first piece needs from global memory is asked for
+  // before the products.
+  const int g0 = C::first(rank), units = (C::first(rank + 1) - g0) * SK_CHUNKS;
+  const int cg = lane & 3, rsub = lane >> 2;
+  const uint32_t flags = epi_flags<EPI>(p);
+  float a_scale = 0.0f, o_inv = 0.0f;
+  ColParams cp;
+  uint4 res = make_uint4(0u, 0u, 0u, 0u);
+  auto locate = [&](int u, int& row, int& n) {
+    row = m0 + (g0 + u / SK_CHUNKS) * 8 + rsub;
+    n = n0 + (u % SK_CHUNKS) * 32 + cg * 8;
+  };
+  auto prefetch_columns = [&](int u) {
+    int row, n;
+    locate(u, row, n);
+    if (row < p.M && n < p.N && !(flags & QDIT_EPI_OUT_I32)) load_col_params<EPI>(p, n, row / p.tokens, a_scale, cp);
+  };
+  auto prefetch_row = [&](int u) {
+    int row, n;
+    locate(u, row, n);
+    if (row < p.M && n < p.N && (flags & QDIT_EPI_RESIDUAL)) res = *reinterpret_cast<const uint4*>(p.residual + static_cast<int64_t>(row) * p.ldo + n);
+  };
+  if (warp >= 2) {
+    if (!p.early) grid_dependency_wait();
+    a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
+    if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
+    if (warp - 2 < units) prefetch_columns(warp - 2);
+    if (p.early) grid_dependency_wait();
+    grid_dependency_release();
+    if (warp - 2 < units) prefetch_row(warp - 2);
+  }
 
   bool accumulated = false;
   const int quad = warp & 3, half = (warp - 2) >> 2;
@@ -116,7 +146,24 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     int stage = 0;
     uint32_t phase = 0;
     bool seen = true;   // the stage about to be filled is known to be free
+    // the first stages' weights come while the previous kernel still runs
+    const int ahead = !p.early ? 0 : kb1 - kb0 < STAGES ? kb1 - kb0 : STAGES;
+    if (ahead > 0 && elect_one()) {
+      for (int i = 0; i < ahead; ++i) {
+        mbar_expect_tx(&full_bar[i], C::A_BYTES + (W4 ? C::P_BYTES : C::B_BYTES));
+        if (W4) tma_load_2d(sP + i * C::P_BYTES, &tmap_w, (kb0 + i) * (BK / 2), n0, &full_bar[i]);
+        else tma_load_2d(sB + i * C::B_BYTES, &tmap_w, (kb0 + i) * BK, n0, &full_bar[i]);
+      }
+    }
+    __syncwarp();
+    grid_dependency_wait();
     for (int kb = kb0; kb < kb1; ++kb) {
+      if (kb - kb0 < ahead) {   // a fresh stage that has its weights
+        if (elect_one()) tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, kb * BK, m0, &full_bar[stage]);
+        __syncwarp();
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; seen = false; }
+        continue;
+      }
       if (!mbar_wait_seen(seen, &empty_bar[stage], phase ^ 1u, abort_flag, p.status)) break;
       const bool wrap = stage + 1 == STAGES;
       seen = mbar_test_wait(&empty_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 0u : 1u));
@@ -201,36 +248,15 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     }
     tc_fence_before();
   }
-  // Work of this warp after the exchange: 8 rows x 32 columns at a time; what it needs from global memory is asked for now.
-  const int g0 = C::first(rank), units = (C::first(rank + 1) - g0) * SK_CHUNKS;
-  const int cg = lane & 3, rsub = lane >> 2;
-  const uint32_t flags = epi_flags<EPI>(p);
-  float a_scale = 0.0f, o_inv = 0.0f;
-  ColParams cp;
-  uint4 res = make_uint4(0u, 0u, 0u, 0u);
-  auto locate = [&](int u, int& row, int& n) {
-    row = m0 + (g0 + u / SK_CHUNKS) * 8 + rsub;
-    n = n0 + (u % SK_CHUNKS) * 32 + cg * 8;
-  };
-  auto prefetch = [&](int u) {
-    int row, n;
-    locate(u, row, n);
-    if (row < p.M && n < p.N && !(flags & QDIT_EPI_OUT_I32)) {
-      load_col_params<EPI>(p, n, row / p.tokens, a_scale, cp);
-      if (flags & QDIT_EPI_RESIDUAL) res = *reinterpret_cast<const uint4*>(p.residual + static_cast<int64_t>(row) * p.ldo + n);
-    }
-  };
-  if (warp >= 2) {
-    a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
-    if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
-    if (warp - 2 < units) prefetch(warp - 2);
-  }
   cluster_arrive();
   cluster_wait();
   if (warp >= 2 && !*abort_flag) {
 #pragma unroll 1
     for (int u = warp - 2; u < units; u += SK_EPI_WARPS) {
-      if (u != warp - 2) prefetch(u);
+      if (u != warp - 2) {
+        prefetch_columns(u);
+        prefetch_row(u);
+      }
       int row, n;
       locate(u, row, n);
       uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = lo;

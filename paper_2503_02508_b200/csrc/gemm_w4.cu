@@ -85,30 +85,41 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_holder;
-  grid_dependency_wait();
-  grid_dependency_release();
+  const uint32_t tmem_base = *tmem_holder;   // (the roles that read what the previous kernel wrote wait for it themselves)
 
   const int num_kb = (p.K + BK - 1) / BK;
   const int total_tiles = p.num_m_tiles * p.num_n_tiles;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ------------------------------------------------------------------ TMA producer
       tma_prefetch_desc(&tmap_a);
       tma_prefetch_desc(&tmap_wp);
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
+      int ahead = 0;   // the first stages' weights come while the previous kernel still runs
+      if (p.early && static_cast<int>(blockIdx.x) < total_tiles) {
+        const int n0 = (static_cast<int>(blockIdx.x) / p.num_m_tiles) * BN;
+        for (; ahead < STAGES && ahead < num_kb; ++ahead) {
+          mbar_expect_tx(&full_bar[ahead], C::A_BYTES + C::P_BYTES);
+          tma_load_2d(sP + ahead * C::P_BYTES, &tmap_wp, ahead * (BK / 2), n0, &full_bar[ahead]);
+        }
+      }
+      grid_dependency_wait();
       for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
         // tiles of one weight block are neighbours in time across the CTAs: m fastest
         const int m0 = (tile % p.num_m_tiles) * BM;
         const int n0 = (tile / p.num_m_tiles) * BN;
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
-          mbar_expect_tx(&full_bar[stage], C::A_BYTES + C::P_BYTES);
+          if (ahead > 0) {   // a fresh stage that has its weights
+            --ahead;
+          } else {
+            if (!mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+            mbar_expect_tx(&full_bar[stage], C::A_BYTES + C::P_BYTES);
+            tma_load_2d(sP + stage * C::P_BYTES, &tmap_wp, kb * (BK / 2), n0, &full_bar[stage]);
+          }
           tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, kb * BK, m0, &full_bar[stage]);
-          tma_load_2d(sP + stage * C::P_BYTES, &tmap_wp, kb * (BK / 2), n0, &full_bar[stage]);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
@@ -117,7 +128,7 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ------------------------------------------------------------------ MMA issuer
       int stage = 0;
       uint32_t phase = 0;
@@ -182,6 +193,8 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const int quad = warp & 3;   // TMEM lane quadrant this warp may access
     const int half = e >> 2;
     const uint32_t stg = smem_u32(staging + e * (32 * 128));
+    grid_dependency_wait();
+    grid_dependency_release();
     const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
     float o_inv = 0.0f;
     if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
@@ -191,11 +204,15 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       const uint32_t aphase = static_cast<uint32_t>(it >> 1) & 1u;
       const int m0 = (tile % p.num_m_tiles) * BM;
       const int n0 = (tile / p.num_m_tiles) * BN;
+      ChunkInputs cur;   // of this warp's first chunk
+      const int n = n0 + half * 32 + (lane & 3) * 8, row_base = m0 + quad * 32;
+      prefetch_params<EPI>(p, n, row_base, a_scale, cur);
+      prefetch_residual<EPI>(p, n, row_base, lane >> 2, cur);
       if (!mbar_wait(&tfull_bar[as], aphase, abort_flag, p.status)) break;
       __syncwarp();
       tc_fence_after();
       uint64_t* release_bar = &tempty_bar[as];
-      epilogue_tile<BN, EPI, W4_EPI_WARPS / 4>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv,
+      epilogue_tile<BN, EPI, W4_EPI_WARPS / 4>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur,
                              [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
   }

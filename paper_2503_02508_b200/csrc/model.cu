@@ -198,26 +198,26 @@ int32_t build_model(qdit_ctx* ctx, const qdit_model_desc* desc, qdit_model* m) {
 
 qdit_qparams sym_qp() { return qdit_qparams{1.0f, 0, -127, 127}; }
 
-// One quantized linear of the fused (static-scale) path.
+// One quantized linear of the model.  Its weights, scales and biases are constant, and a gate belongs to a modulation that was computed
+// several launches before; `calib`: the activation scale is what the launch in front leaves.
 // `w8_scratch`: for a layer stored packed, the matrix its weights are widened into when the layer has many rows
 // (NULL: always widened inside the GEMM kernel, which is the form for the weight-streaming modulation GEMM).
 int32_t run_linear(qdit_ctx* ctx, const void* A, const QLinearDev& l, int64_t M, const float* a_scale_dev, uint32_t flags,
-                   qdit_epilogue epi, void* out, void* w8_scratch = nullptr) {
+                   qdit_epilogue epi, void* out, bool calib, void* w8_scratch = nullptr) {
   epi.w_scale = l.scale;
   epi.w_colsum = l.colsum;
   epi.bias = l.bias;
-  if (l.packed4)
-    return qdit_w4a8_linear(ctx, A, l.q, M, l.N, l.K, sym_qp(), a_scale_dev, flags | QDIT_EPI_BIAS, &epi, out, l.N, w8_scratch);
-  return qdit_w8a8_linear(ctx, A, l.q, M, l.N, l.K, sym_qp(), a_scale_dev, flags | QDIT_EPI_BIAS, &epi, out, l.N);
+  return qdit_linear_impl(ctx, A, l.q, M, l.N, l.K, sym_qp(), a_scale_dev, flags | QDIT_EPI_BIAS, &epi, out, l.N, l.packed4,
+                          l.packed4 ? w8_scratch : nullptr, !calib);
 }
 
 // The modulation linears of all blocks on `rows` conditioning rows: out[rows, depth * 6D].  One stacked GEMM; with
 // packed 4-bit weights and many rows (the whole trajectory's conditioning) block by block instead, each block's
 // 6D x D weights widened into the scratch matrix first (the stacked matrix would need a scratch of its own size).
 int32_t run_modulation(qdit_ctx* ctx, const qdit_model* m, const void* A, int64_t rows, const float* a_scale_dev, float* out,
-                       void* w8_scratch) {
+                       bool calib, void* w8_scratch) {
   qdit_epilogue epi{};
-  if (!(m->ada_all.packed4 && w8_scratch && rows >= 1024)) return run_linear(ctx, A, m->ada_all, rows, a_scale_dev, QDIT_EPI_OUT_F32, epi, out);
+  if (!(m->ada_all.packed4 && w8_scratch && rows >= 1024)) return run_linear(ctx, A, m->ada_all, rows, a_scale_dev, QDIT_EPI_OUT_F32, epi, out, calib);
   const int64_t D = m->s.hidden, n6 = 6 * D, ld = static_cast<int64_t>(m->s.depth) * n6;
   for (int i = 0; i < m->s.depth; ++i) {
     const int64_t r0 = i * n6;
@@ -267,7 +267,7 @@ static int32_t forward_impl(qdit_ctx* ctx, qdit_sampler* s, const float* latent,
     } else {
       QDIT_TRY(qdit_quantize_act_dev(ctx, s->sc, B, D, sym_qp(), scales + 0, s->ca));
     }
-    QDIT_TRY(run_modulation(ctx, m, s->ca, B, scales + 0, s->mod, s->w8_scratch));
+    QDIT_TRY(run_modulation(ctx, m, s->ca, B, scales + 0, s->mod, calib, s->w8_scratch));
     mod_all = s->mod;
   }
 
@@ -292,50 +292,51 @@ static int32_t forward_impl(qdit_ctx* ctx, qdit_sampler* s, const float* latent,
         if (mask && mask[2 * i]) {
           QDIT_TRY(qdit_cache_reuse(ctx, s->cache, i, QDIT_BRANCH_ATTN, mod + 2 * D, ld_mod, T, s->x));
         } else {
-          QDIT_TRY(qdit_adaln_modulate(ctx, s->x, M, D, T, 1e-6f, mod, mod + D, ld_mod, s->h, QDIT_I8, &qp, sc_qkv));
+          // (the first block's modulation may be what the launch in front computed)
+          QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod, mod + D, ld_mod, s->h, QDIT_I8, &qp, sc_qkv, i > 0 || pre_mod));
           qdit_epilogue e0{};
-          QDIT_TRY(run_linear(ctx, s->h, m->qkv[i], M, sc_qkv, QDIT_EPI_OUT_BF16, e0, s->qkv, s->w8_scratch));
+          QDIT_TRY(run_linear(ctx, s->h, m->qkv[i], M, sc_qkv, QDIT_EPI_OUT_BF16, e0, s->qkv, calib, s->w8_scratch));
           const __nv_bfloat16* qkv = static_cast<const __nv_bfloat16*>(s->qkv);
           QDIT_TRY(qdit_attention(ctx, qkv, qkv + D, qkv + 2 * D, 3 * D, B, sh.heads, T, D / sh.heads, att_scale, s->a,
                                   QDIT_I8, &qp, sc_proj));
           gated.gate = mod + 2 * D;
           gated.cache_out = store ? qdit_cache_slot(s->cache, i, QDIT_BRANCH_ATTN, 1) : nullptr;
-          QDIT_TRY(run_linear(ctx, s->a, m->proj[i], M, sc_proj, gflags, gated, s->x, s->w8_scratch));
+          QDIT_TRY(run_linear(ctx, s->a, m->proj[i], M, sc_proj, gflags, gated, s->x, calib, s->w8_scratch));
         }
         // ---- MLP branch
         if (mask && mask[2 * i + 1]) {
           QDIT_TRY(qdit_cache_reuse(ctx, s->cache, i, QDIT_BRANCH_MLP, mod + 5 * D, ld_mod, T, s->x));
         } else {
-          QDIT_TRY(qdit_adaln_modulate(ctx, s->x, M, D, T, 1e-6f, mod + 3 * D, mod + 4 * D, ld_mod, s->h, QDIT_I8, &qp, sc_fc1));
+          QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod + 3 * D, mod + 4 * D, ld_mod, s->h, QDIT_I8, &qp, sc_fc1, true));
           qdit_epilogue e1{};
           e1.out_qp = qp;
           e1.out_scale_dev = sc_fc2;
-          QDIT_TRY(run_linear(ctx, s->h, m->fc1[i], M, sc_fc1, QDIT_EPI_GELU | QDIT_EPI_QUANT_OUT, e1, s->u, s->w8_scratch));
+          QDIT_TRY(run_linear(ctx, s->h, m->fc1[i], M, sc_fc1, QDIT_EPI_GELU | QDIT_EPI_QUANT_OUT, e1, s->u, calib, s->w8_scratch));
           gated.gate = mod + 5 * D;
           gated.cache_out = store ? qdit_cache_slot(s->cache, i, QDIT_BRANCH_MLP, 1) : nullptr;
-          QDIT_TRY(run_linear(ctx, s->u, m->fc2[i], M, sc_fc2, gflags, gated, s->x, s->w8_scratch));
+          QDIT_TRY(run_linear(ctx, s->u, m->fc2[i], M, sc_fc2, gflags, gated, s->x, calib, s->w8_scratch));
         }
       } else {
         // ---- calibration: every quantizer input is materialised in f32, its range reduced, then quantized
         QDIT_TRY(qdit_adaln_modulate(ctx, s->x, M, D, T, 1e-6f, mod, mod + D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr));
         QDIT_TRY(dyn_quant(ctx, s, 1 + 4 * i, s->tmpf, M, D, s->h));
         qdit_epilogue e0{};
-        QDIT_TRY(run_linear(ctx, s->h, m->qkv[i], M, sc_qkv, QDIT_EPI_OUT_BF16, e0, s->qkv, s->w8_scratch));
+        QDIT_TRY(run_linear(ctx, s->h, m->qkv[i], M, sc_qkv, QDIT_EPI_OUT_BF16, e0, s->qkv, calib, s->w8_scratch));
         const __nv_bfloat16* qkv = static_cast<const __nv_bfloat16*>(s->qkv);
         QDIT_TRY(qdit_attention(ctx, qkv, qkv + D, qkv + 2 * D, 3 * D, B, sh.heads, T, D / sh.heads, att_scale, s->tmpf,
                                 QDIT_F32, nullptr, nullptr));
         QDIT_TRY(dyn_quant(ctx, s, 2 + 4 * i, s->tmpf, M, D, s->a));
         gated.gate = mod + 2 * D;
         gated.cache_out = store ? qdit_cache_slot(s->cache, i, QDIT_BRANCH_ATTN, 1) : nullptr;
-        QDIT_TRY(run_linear(ctx, s->a, m->proj[i], M, sc_proj, gflags, gated, s->x, s->w8_scratch));
+        QDIT_TRY(run_linear(ctx, s->a, m->proj[i], M, sc_proj, gflags, gated, s->x, calib, s->w8_scratch));
         QDIT_TRY(qdit_adaln_modulate(ctx, s->x, M, D, T, 1e-6f, mod + 3 * D, mod + 4 * D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr));
         QDIT_TRY(dyn_quant(ctx, s, 3 + 4 * i, s->tmpf, M, D, s->h));
         qdit_epilogue e1{};
-        QDIT_TRY(run_linear(ctx, s->h, m->fc1[i], M, sc_fc1, QDIT_EPI_GELU | QDIT_EPI_OUT_F32, e1, s->tmpf, s->w8_scratch));
+        QDIT_TRY(run_linear(ctx, s->h, m->fc1[i], M, sc_fc1, QDIT_EPI_GELU | QDIT_EPI_OUT_F32, e1, s->tmpf, calib, s->w8_scratch));
         QDIT_TRY(dyn_quant(ctx, s, 4 + 4 * i, s->tmpf, M, F, s->u));
         gated.gate = mod + 5 * D;
         gated.cache_out = store ? qdit_cache_slot(s->cache, i, QDIT_BRANCH_MLP, 1) : nullptr;
-        QDIT_TRY(run_linear(ctx, s->u, m->fc2[i], M, sc_fc2, gflags, gated, s->x, s->w8_scratch));
+        QDIT_TRY(run_linear(ctx, s->u, m->fc2[i], M, sc_fc2, gflags, gated, s->x, calib, s->w8_scratch));
       }
     }
   }
@@ -360,7 +361,7 @@ static int32_t trajectory_conditioning(qdit_ctx* ctx, qdit_sampler* s, int first
   QDIT_TRY(launch_batched_linear(ctx, s->traj_hidden, m->w_t2, m->b_t2, m->y_table, s->y, s->traj_c, s->traj_sc, rows, D, D, 0, 0,
                                  s->Beff));
   QDIT_TRY(qdit_quantize_act_dev(ctx, s->traj_sc, rows, D, sym_qp(), m->d_scales + 0, s->traj_ca));
-  QDIT_TRY(run_modulation(ctx, m, s->traj_ca, rows, m->d_scales + 0, s->traj_mod, s->w8_scratch));
+  QDIT_TRY(run_modulation(ctx, m, s->traj_ca, rows, m->d_scales + 0, s->traj_mod, false, s->w8_scratch));
   return launch_batched_linear(ctx, s->traj_c, m->w_ada_f, m->b_ada_f, nullptr, nullptr, s->traj_modf, nullptr, rows, 2 * D, D, 1, 0, 0);
 }
 

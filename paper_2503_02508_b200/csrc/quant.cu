@@ -379,21 +379,27 @@ template <int NV4>
 __global__ void __launch_bounds__(LNQ_WARPS * 32, 2) ln_modulate_q8_kernel(const __nv_bfloat16* __restrict__ x, int M, int T, float eps,
                                                                 const float* __restrict__ shift,
                                                                 const float* __restrict__ scale, int64_t ld_mod,
-                                                                uint8_t* __restrict__ out, QuantArgs qa, int rows_per_cta) {
+                                                                uint8_t* __restrict__ out, QuantArgs qa, int rows_per_cta, int early) {
   constexpr int D = NV4 * 128, D4 = D / 4;
   extern __shared__ float4 s_par[];  // [2 samples][mul, add][D / 4]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int row_begin = blockIdx.x * rows_per_cta;
   const int row_end = row_begin + rows_per_cta < M ? row_begin + rows_per_cta : M;
   if (row_begin >= M) return;
-  grid_dependency_wait();  // x and the modulation come from earlier kernels of the stream
-  grid_dependency_release();
   int row = row_begin + warp;
   uint2 raw[NV4];
-  if (row < row_end) {
-    const uint2* xr = reinterpret_cast<const uint2*>(x + static_cast<int64_t>(row) * D) + lane;
+  auto load_row = [&]() {
+    if (row < row_end) {
+      const uint2* xr = reinterpret_cast<const uint2*>(x + static_cast<int64_t>(row) * D) + lane;
 #pragma unroll
-    for (int j = 0; j < NV4; ++j) raw[j] = xr[32 * j];
+      for (int j = 0; j < NV4; ++j) raw[j] = xr[32 * j];
+    }
+  };
+  // `early`: the modulation and the scale were written two launches ago or earlier and are staged while the previous kernel, which writes
+  // x, still runs
+  if (!early) {
+    grid_dependency_wait();
+    load_row();
   }
   const float inv = __fdiv_rn(1.0f, qa.scale_dev ? __ldg(qa.scale_dev) : qa.scale);
   const int b0 = row_begin / T;
@@ -407,6 +413,11 @@ __global__ void __launch_bounds__(LNQ_WARPS * 32, 2) ln_modulate_q8_kernel(const
       s_par[(s * 2 + 1) * D4 + i] = make_float4(h4.x * inv, h4.y * inv, h4.z * inv, h4.w * inv);
     }
   }
+  if (early) {
+    grid_dependency_wait();
+    load_row();
+  }
+  grid_dependency_release();
   __syncthreads();
   constexpr float inv_d = 1.0f / static_cast<float>(D);
   const int second = (b0 + 1) * T;  // first row of the second staged sample
@@ -462,11 +473,11 @@ __global__ void __launch_bounds__(LNQ_WARPS * 32, 2) ln_modulate_q8_kernel(const
 
 template <int NV4>
 void launch_ln_q8(qdit_ctx* ctx, const void* x, int64_t M, const float* shift, const float* scale, int64_t ld_mod,
-                  int64_t T, float eps, void* out, QuantArgs qa, int64_t rows) {
+                  int64_t T, float eps, void* out, QuantArgs qa, int64_t rows, bool early) {
   const unsigned grid = static_cast<unsigned>((M + rows - 1) / rows);
   qdit_launch_overlapped(ctx, ln_modulate_q8_kernel<NV4>, dim3(grid), dim3(LNQ_WARPS * 32), static_cast<size_t>(NV4) * 128 * 16,
                          static_cast<const __nv_bfloat16*>(x), static_cast<int>(M), static_cast<int>(T), eps, shift, scale,
-                         ld_mod, static_cast<uint8_t*>(out), qa, static_cast<int>(rows));
+                         ld_mod, static_cast<uint8_t*>(out), qa, static_cast<int>(rows), static_cast<int>(early));
 }
 
 // Row range per CTA: `per_sm` CTAs per SM, at least eight rows, at most what keeps a range within two samples.
@@ -621,6 +632,13 @@ int32_t qdit_quantize_weight(qdit_ctx* ctx, const float* w, int64_t N, int64_t K
 int32_t qdit_adaln_modulate(qdit_ctx* ctx, const void* x, int64_t M, int64_t D, int64_t T, float eps,
                             const float* shift, const float* scale, int64_t ld_mod, void* out, int out_dtype,
                             const qdit_qparams* out_qp, const float* out_scale_dev) {
+  return qdit_adaln_impl(ctx, x, M, D, T, eps, shift, scale, ld_mod, out, out_dtype, out_qp, out_scale_dev, false);
+}
+
+}  // extern "C"
+
+int32_t qdit_adaln_impl(qdit_ctx* ctx, const void* x, int64_t M, int64_t D, int64_t T, float eps, const float* shift, const float* scale,
+                        int64_t ld_mod, void* out, int out_dtype, const qdit_qparams* out_qp, const float* out_scale_dev, bool early) {
   if (!ctx) return QDIT_ERR_INVALID_ARG;
   if (M < 0 || D <= 0 || T <= 0) return qdit_fail(ctx, QDIT_ERR_SHAPE, "bad sizes");
   if (M > (int64_t(1) << 30) || T > (int64_t(1) << 30)) return qdit_fail(ctx, QDIT_ERR_SHAPE, "M and T must be at most 2^30");
@@ -645,10 +663,10 @@ int32_t qdit_adaln_modulate(qdit_ctx* ctx, const void* x, int64_t M, int64_t D, 
     const int64_t rows = ln_rows_per_cta(ctx, M, T, 2);
     bool done = true;
     switch (D / 128) {
-      case 3: launch_ln_q8<3>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows); break;
-      case 6: launch_ln_q8<6>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows); break;
-      case 8: launch_ln_q8<8>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows); break;
-      case 9: launch_ln_q8<9>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows); break;
+      case 3: launch_ln_q8<3>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows, early); break;
+      case 6: launch_ln_q8<6>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows, early); break;
+      case 8: launch_ln_q8<8>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows, early); break;
+      case 9: launch_ln_q8<9>(ctx, x, M, shift, scale, ld_mod, T, eps, out, qa, rows, early); break;
       default: done = false; break;
     }
     if (done) return qdit_after_launch(ctx, "ln_modulate_q8_kernel");
@@ -665,5 +683,3 @@ int32_t qdit_adaln_modulate(qdit_ctx* ctx, const void* x, int64_t M, int64_t D, 
   }
   return qdit_after_launch(ctx, "ln_modulate_kernel");
 }
-
-}  // extern "C"
