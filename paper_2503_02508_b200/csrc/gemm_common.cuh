@@ -282,6 +282,7 @@ int32_t qdit_launch_gemm_t(qdit_ctx* ctx, const void* A, const void* W, qgemm::G
 // Token-major tiles of 256 tokens by pairs of CTAs (gemm_i8_p.cu), for the epilogue classes 1, 2 (width and pitch multiples of 16), 3 (samples
 // of whole 32-token chunks), 5 and 6.
 int32_t qdit_launch_gemm_pair(qdit_ctx* ctx, const void* A, const void* W, const qgemm::GemmParams& p, bool a_unsigned);
+double qdit_gemm_pair_cost(const qdit_ctx* ctx, const qgemm::GemmParams& p);   // estimate, in clocks, without what every launch takes
 
 // Token-major tiles of 128 x 64 whose reduction is split over clusters of `split` (2, 3, 4 or 6) CTAs (gemm_i8_sk.cu);
 // K > (split - 1) * 128; packed4: W holds 4-bit codes two per byte.  qdit_gemm_sk_clusters: clusters of that size the device holds at once.

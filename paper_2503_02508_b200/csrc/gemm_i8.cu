@@ -106,16 +106,16 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         }
       }
       grid_dependency_wait();
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      if (ahead > 0) {
+        const int m0 = (static_cast<int>(blockIdx.x) / p.num_n_tiles) * BM;
+        for (; stage < ahead; ++stage) tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, stage * BK, m0, &full_bar[stage]);
+        if (stage == STAGES) { stage = 0; phase ^= 1u; seen = false; }
+      }
+      int kb = ahead;
+      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, kb = 0) {
         const int m0 = (tile / p.num_n_tiles) * BM;
         const int n0 = (tile % p.num_n_tiles) * BN;
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (ahead > 0) {   // a fresh stage that has its weights
-            --ahead;
-            tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, kb * BK, m0, &full_bar[stage]);
-            if (++stage == STAGES) { stage = 0; phase ^= 1u; seen = false; }
-            continue;
-          }
+        for (; kb < num_kb; ++kb) {
           if (!wait_for(seen, &empty_bar[stage], phase ^ 1u)) { ok = false; break; }
           const bool wrap = stage + 1 == STAGES;
           seen = AHEAD && mbar_test_wait(&empty_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 0u : 1u));
@@ -381,18 +381,23 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
   // Kernel choice.  A layer whose 128 x 192 tiles fill no more than one wave runs token-major, one CTA per tile (below): pairs gain
   // nothing there (2048 x 3456 x 384: 4.8 us against 5.0, 1024 x 1152 x 1152 gated 5.3 and 6.5).  From the second wave on pairs of CTAs
   // are faster (us, single CTAs / pairs: QKV of XL/2 2048 rows 11.0 / 9.0, 8192 26.7 / 24.0, 65536 222 / 182; fc1 40.1 / 35.4 and
-  // 310 / 295; fc2 5000 rows 31.2 / 24.4, 8192 35.6 / 34.8, 65536 276 / 256; proj 14.9 / 11.3, 15.2 / 15.1, 117 / 113).  Per-token
-  // scales and f32 output take pairs earlier, because their token-major epilogue decides at run time what to do (512 x 3456 x 1152:
-  // 8.6 / 5.9 and 8.2 / 6.4), unless the split reduction, which splits the epilogue too, serves them.  Where 128 x 256
-  // channel-major tiles make exactly one wave they are better still (QKV 1280 rows: 7.2 against 7.7 us, with per-token scales
-  // 11.0 / 12.1; proj and fc2 at 4096: 9.7 / 10.5 and 18.4 / 20.3; one image of 1024 tokens: 1650 us against 1660 with QKV token-major).
+  // 310 / 295; fc2 5000 rows 31.2 / 24.4, 65536 276 / 256; proj 14.9 / 11.3 and 117 / 113).  Per-token scales and f32 output take pairs
+  // earlier, because their token-major epilogue decides at run time what to do (512 x 3456 x 1152: 8.6 / 5.9 and 8.2 / 6.4), unless the
+  // split reduction, which splits the epilogue too, serves them.  Layers of few columns, or of rows just right for it, fill the chip better
+  // with the 128 x 256 channel-major tiles of single CTAs, at 620 clocks per k-block, 600 per tile and 4500 for the last epilogue; a
+  // pair's launch costs 1500 clocks more (channel-major / pairs: QKV 1280 rows 7.2 / 7.7 us, with per-token scales 11.0 / 12.1; gated fc2 4096 rows
+  // 18.4 / 20.3, 8192 with 4-bit codes 34.2 / 35.9, proj 4096 9.7 / 10.5).
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE]) {
     // (8-bit rows leave through TMA stores of whole 16-byte pieces, and a 32-token chunk of a gated layer has one gate row)
     const bool staged = cls == 1 || cls == 5 || cls == 6 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0) || (cls == 3 && p.tokens % 32 == 0);
     const bool slow = cls == 5 || cls == 6;
     const bool one_wave = static_cast<int64_t>((p.M + BM - 1) / BM) * ((p.N + 191) / 192) <= ctx->num_sms;
-    const bool t_wave = p.M >= 1024 && static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) <= ctx->num_sms;
-    if (staged && t_wave && (cls == 3 ? !one_wave : cls != 2 && p.N >= 2304)) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
+    if (staged && p.M >= 1024 && (cls == 3 ? p.N >= 1024 && !one_wave : cls != 2 && p.N >= 2304)) {
+      const int64_t waves = (static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) + ctx->num_sms - 1) / ctx->num_sms;
+      const double cost = static_cast<double>(waves) * ((p.K + BK - 1) / BK * 620.0 + 600.0) + 4500.0;
+      // (f32 output: with one wave only; there the epilogue is the longer part of a tile, 8192 x 3456 x 1152 36.9 us against 33.9)
+      if (cls == 6 ? waves == 1 : cost <= qdit_gemm_pair_cost(ctx, p) + 1500.0) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
+    }
     if (staged && (slow ? p.M > BM && pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) == 1 : !one_wave))
       return qdit_launch_gemm_pair(ctx, A, W, p, a_unsigned);
   }

@@ -31,6 +31,7 @@ namespace {
 using namespace qgemm;
 
 constexpr int MAX_STAGES = 8;
+constexpr int SHORT_K = 2048;                        // gated layers with a shorter reduction: class 4
 constexpr int A_BYTES = 128 * BK;                    // 128 tokens of a k-block; half of the channels follow (BN / 2 rows)
 constexpr int ACC_COLS = 256;
 
@@ -612,36 +613,40 @@ int32_t launch_p_epi(qdit_ctx* ctx, const void* A, const void* W, const GemmPara
 // more often (fc2 at 65536 rows: 256 us with 256 channels, 316 with 192, which this estimate puts level).
 // Measured: 8192 x 3456 x 1152 24.4 / 24.0 / 24.0 us with 256 / 224 / 192 channels, 2048 rows 10.1 / 9.7 / 9.0; 8192 x 1152 x 4608 40.5 with
 // 256, 34.8 with 192, 36.5 with 128; 1024 x 4608 x 1152 10.1 with 256, 9.4 with 128.
-int pick_pair_bn(int M, int N, int K, int pairs, int chunk) {
-  const int64_t mt = (M + 255) / 256;
-  const double num_kb = (K + BK - 1) / BK;
-  int best = 256;
-  double best_cost = 1e30;
+struct PairTile {
+  int bn;
+  double cost;
+};
+PairTile pick_pair_tile(const GemmParams& p, int pairs) {
+  const int cls = epi_class(p.flags);
+  const int chunk = cls == 1 ? 540 : cls == 2 ? 770 : cls == 3 ? (p.K < SHORT_K ? 650 : 950) : cls == 5 ? 560 : 650;
+  const int64_t mt = (p.M + 255) / 256;
+  const double num_kb = (p.K + BK - 1) / BK;
+  PairTile best{256, 1e30};
   for (int bn = 256; bn >= 64; bn -= 32) {
-    const int64_t waves = (mt * ((N + bn - 1) / bn) + pairs - 1) / pairs;
+    const int64_t waves = (mt * ((p.N + bn - 1) / bn) + pairs - 1) / pairs;
     const double main = num_kb * (200.0 + 1.22 * bn), epilogue = chunk * bn / 32.0;
     const double cost = static_cast<double>(waves) * ((main > epilogue ? main : epilogue) + 600.0) + epilogue;
-    if (cost < best_cost * 0.96) {
-      best_cost = cost;
-      best = bn;
-    }
+    if (cost < best.cost * 0.96) best = PairTile{bn, cost};
   }
   return best;
 }
 
 }  // namespace
 
+double qdit_gemm_pair_cost(const qdit_ctx* ctx, const GemmParams& p) { return pick_pair_tile(p, ctx->num_sms / 2).cost; }
+
 int32_t qdit_launch_gemm_pair(qdit_ctx* ctx, const void* A, const void* W, const GemmParams& p, bool a_unsigned) {
-  auto bn = [&](int chunk) { return pick_pair_bn(p.M, p.N, p.K, ctx->num_sms / 2, chunk); };
+  const int bn = pick_pair_tile(p, ctx->num_sms / 2).bn;
   switch (epi_class(p.flags)) {
-    case 1: return launch_p_epi<1>(ctx, A, W, p, a_unsigned, bn(540));
-    case 2: return launch_p_epi<2>(ctx, A, W, p, a_unsigned, bn(770));
+    case 1: return launch_p_epi<1>(ctx, A, W, p, a_unsigned, bn);
+    case 2: return launch_p_epi<2>(ctx, A, W, p, a_unsigned, bn);
     case 3:
       // A short reduction leaves the gated epilogue as the longer part of a tile: three warps per lane quadrant instead of two, at the
       // price of one pipeline stage (proj of XL/2 at 65536 rows: 125 -> 112 us, 5000 rows 12.0 -> 11.3)
-      if (p.K < 2048) return launch_p_epi<4>(ctx, A, W, p, a_unsigned, bn(650));
-      return launch_p_epi<3>(ctx, A, W, p, a_unsigned, bn(950));
-    case 5: return launch_p_epi<5>(ctx, A, W, p, a_unsigned, bn(560));
-    default: return launch_p_epi<6>(ctx, A, W, p, a_unsigned, bn(650));
+      if (p.K < SHORT_K) return launch_p_epi<4>(ctx, A, W, p, a_unsigned, bn);
+      return launch_p_epi<3>(ctx, A, W, p, a_unsigned, bn);
+    case 5: return launch_p_epi<5>(ctx, A, W, p, a_unsigned, bn);
+    default: return launch_p_epi<6>(ctx, A, W, p, a_unsigned, bn);
   }
 }

@@ -133,7 +133,8 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if (!p.early) grid_dependency_wait();
     a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
     if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
-    if (warp - 2 < units) prefetch_columns(warp - 2);
+    // (warps that widen weights first do not wait for the parameters in front of that)
+    if ((!W4 || p.early) && warp - 2 < units) prefetch_columns(warp - 2);
     if (p.early) grid_dependency_wait();
     grid_dependency_release();
     if (warp - 2 < units) prefetch_row(warp - 2);
@@ -157,13 +158,15 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     }
     __syncwarp();
     grid_dependency_wait();
-    for (int kb = kb0; kb < kb1; ++kb) {
-      if (kb - kb0 < ahead) {   // a fresh stage that has its weights
-        if (elect_one()) tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, kb * BK, m0, &full_bar[stage]);
-        __syncwarp();
-        if (++stage == STAGES) { stage = 0; phase ^= 1u; seen = false; }
-        continue;
+    if (ahead > 0) {
+      if (elect_one()) {
+        for (int i = 0; i < ahead; ++i) tma_load_2d(sA + i * C::A_BYTES, &tmap_a, (kb0 + i) * BK, m0, &full_bar[i]);
       }
+      __syncwarp();
+      stage = ahead;
+      if (stage == STAGES) { stage = 0; phase ^= 1u; seen = false; }
+    }
+    for (int kb = kb0 + ahead; kb < kb1; ++kb) {
       if (!mbar_wait_seen(seen, &empty_bar[stage], phase ^ 1u, abort_flag, p.status)) break;
       const bool wrap = stage + 1 == STAGES;
       seen = mbar_test_wait(&empty_bar[wrap ? 0 : stage + 1], phase ^ (wrap ? 0u : 1u));
@@ -224,6 +227,7 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
+    if (W4 && !p.early && warp - 2 < units) prefetch_columns(warp - 2);
     accumulated = ok && mbar_wait_warp(tfull_bar, 0, abort_flag, p.status);
   }
   cluster_wait();

@@ -107,19 +107,21 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         }
       }
       grid_dependency_wait();
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      if (ahead > 0) {
+        const int m0 = (static_cast<int>(blockIdx.x) % p.num_m_tiles) * BM;
+        for (; stage < ahead; ++stage) tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, stage * BK, m0, &full_bar[stage]);
+        if (stage == STAGES) { stage = 0; phase ^= 1u; }
+      }
+      int kb = ahead;
+      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, kb = 0) {
         // tiles of one weight block are neighbours in time across the CTAs: m fastest
         const int m0 = (tile % p.num_m_tiles) * BM;
         const int n0 = (tile / p.num_m_tiles) * BN;
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (ahead > 0) {   // a fresh stage that has its weights
-            --ahead;
-          } else {
-            if (!mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
-            mbar_expect_tx(&full_bar[stage], C::A_BYTES + C::P_BYTES);
-            tma_load_2d(sP + stage * C::P_BYTES, &tmap_wp, kb * (BK / 2), n0, &full_bar[stage]);
-          }
+        for (; kb < num_kb; ++kb) {
+          if (!mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+          mbar_expect_tx(&full_bar[stage], C::A_BYTES + C::P_BYTES);
           tma_load_2d(sA + stage * C::A_BYTES, &tmap_a, kb * BK, m0, &full_bar[stage]);
+          tma_load_2d(sP + stage * C::P_BYTES, &tmap_wp, kb * (BK / 2), n0, &full_bar[stage]);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
