@@ -28,6 +28,7 @@ struct AttnParams {
   int out_dtype;
   QuantArgs qa;
   int* status;
+  float* absmax;   // f32 output: takes the largest magnitude, if given
 };
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
@@ -266,6 +267,15 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       }
     }
   }
+  if (p.absmax) {
+    float top = 0.0f;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+      for (int i = 0; i < C::NT_O; ++i) top = fmaxf(top, fmaxf(fabsf(o[i][2 * r] * inv_l[r]), fabsf(o[i][2 * r + 1] * inv_l[r])));
+    }
+    publish_absmax(p.absmax, top);
+  }
 }
 
 template <int DH, int QW>
@@ -287,11 +297,16 @@ int32_t launch_attention(qdit_ctx* ctx, const void* q, const void* k, const void
 }  // namespace
 
 int32_t qdit_launch_attention_tc(qdit_ctx* ctx, const void* q, const void* k, const void* v, int64_t ld, int B, int H,
-                                 int T, int dh, float softmax_scale, void* out, int out_dtype, QuantArgs qa);
+                                 int T, int dh, float softmax_scale, void* out, int out_dtype, QuantArgs qa, float* absmax);
 
 extern "C" int32_t qdit_attention(qdit_ctx* ctx, const void* q, const void* k, const void* v, int64_t ld, int B, int H,
                                   int T, int dh, float softmax_scale, void* out, int out_dtype,
                                   const qdit_qparams* out_qp, const float* out_scale_dev) {
+  return qdit_attention_impl(ctx, q, k, v, ld, B, H, T, dh, softmax_scale, out, out_dtype, out_qp, out_scale_dev, nullptr);
+}
+
+int32_t qdit_attention_impl(qdit_ctx* ctx, const void* q, const void* k, const void* v, int64_t ld, int B, int H, int T, int dh, float softmax_scale,
+                            void* out, int out_dtype, const qdit_qparams* out_qp, const float* out_scale_dev, float* absmax) {
   if (!ctx) return QDIT_ERR_INVALID_ARG;
   if (B < 0 || H <= 0 || T < 0) return qdit_fail(ctx, QDIT_ERR_SHAPE, "bad sizes");
   if (B == 0 || T == 0) return QDIT_OK;
@@ -310,6 +325,7 @@ extern "C" int32_t qdit_attention(qdit_ctx* ctx, const void* q, const void* k, c
   p.out = out;
   p.out_dtype = out_dtype;
   p.status = ctx->d_status;
+  p.absmax = absmax;
   if (out_dtype == QDIT_I8) {
     QDIT_TRY(qdit_check_qparams(ctx, out_qp, out_scale_dev != nullptr));
     p.qa = make_quant_args(*out_qp, out_scale_dev);
@@ -320,7 +336,7 @@ extern "C" int32_t qdit_attention(qdit_ctx* ctx, const void* q, const void* k, c
   // so that a sample's bits do not depend on the batch.
   const int choice = ctx->opt[QDIT_OPT_ATTN];
   if (choice == 2 || (choice == 0 && T > 64))
-    return qdit_launch_attention_tc(ctx, q, k, v, ld, B, H, T, dh, softmax_scale, out, out_dtype, p.qa);
+    return qdit_launch_attention_tc(ctx, q, k, v, ld, B, H, T, dh, softmax_scale, out, out_dtype, p.qa, absmax);
   const bool wide = T % 128 == 0;  // 128 queries per CTA when the token count allows
   if (dh == 64) return wide ? launch_attention<64, 8>(ctx, q, k, v, ld, B, H, T, p) : launch_attention<64, 4>(ctx, q, k, v, ld, B, H, T, p);
   return wide ? launch_attention<72, 8>(ctx, q, k, v, ld, B, H, T, p) : launch_attention<72, 4>(ctx, q, k, v, ld, B, H, T, p);

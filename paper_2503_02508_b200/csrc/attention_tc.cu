@@ -70,6 +70,7 @@ struct AttnTcParams {
   int out_dtype;
   QuantArgs qa;
   int* status;
+  float* absmax;       // f32 output: takes the largest magnitude, if given
 };
 
 template <int DH>
@@ -416,6 +417,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
       } else {
         constexpr int ROW = DH * 4 + 16, PIECES = DH / 4;
+        if (p.absmax) {   // (rounding is monotonic: the largest product is that of the largest magnitude)
+          float m = 0.0f;
+#pragma unroll
+          for (int i = 0; i < DH; ++i) m = fmaxf(m, fabsf(__uint_as_float(o[i])));
+          publish_absmax(p.absmax, fmaxf(m * inv_l, 0.0f));
+        }
 #pragma unroll
         for (int g = 0; g < DH / 4; ++g)
           *reinterpret_cast<float4*>(stage + lane * ROW + 16 * g) =
@@ -600,7 +607,7 @@ int32_t launch_tc(qdit_ctx* ctx, const void* q, const void* k, const void* v, in
 
 // Tensor-core attention for T % 64 == 0 and head dim 64 or 72 (arguments already validated by qdit_attention).
 int32_t qdit_launch_attention_tc(qdit_ctx* ctx, const void* q, const void* k, const void* v, int64_t ld, int B, int H,
-                                 int T, int dh, float softmax_scale, void* out, int out_dtype, QuantArgs qa) {
+                                 int T, int dh, float softmax_scale, void* out, int out_dtype, QuantArgs qa, float* absmax) {
   AttnTcParams p{};
   p.T = T;
   p.H = H;
@@ -610,6 +617,7 @@ int32_t qdit_launch_attention_tc(qdit_ctx* ctx, const void* q, const void* k, co
   p.out_dtype = out_dtype;
   p.qa = qa;
   p.status = ctx->d_status;
+  p.absmax = absmax;
   if (dh == 64) return launch_tc<64>(ctx, q, k, v, ld, B, H, T, p);
   return launch_tc<72>(ctx, q, k, v, ld, B, H, T, p);
 }

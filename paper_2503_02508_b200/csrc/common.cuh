@@ -342,6 +342,12 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Folds a warp's largest magnitude (of non-negative values per lane) into *slot, which holds 0 or an earlier one.
+__device__ __forceinline__ void publish_absmax(float* slot, float m) {
+  m = warp_max(m);
+  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(slot), __float_as_int(m));
+}
+
 __device__ __forceinline__ void unpack_bf16x2(uint32_t w, float& a, float& b) {
   a = __uint_as_float(w << 16);
   b = __uint_as_float(w & 0xFFFF0000u);

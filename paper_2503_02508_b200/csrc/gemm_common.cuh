@@ -45,27 +45,30 @@ struct GemmParams {
   // The weights, their scales and biases, the gate and the quantizer scales were written two launches ago or earlier: a kernel that has
   // started beside its predecessor may read them before it waits for it (every kernel lets its successor start after its own wait).
   bool early;
+  float* absmax;   // f32 output: the largest magnitude is folded into this, if given (calibration; run-time-flag and GELU -> f32 epilogues)
 };
 
 // Epilogue classes.  The three block-level layers get kernels whose epilogue flags are compile-time
 // constants (no flag branches, no dead registers, a smaller instruction footprint: instruction-fetch stalls
 // were a top stall reason of the all-in-one kernel); class 0 keeps the flags as run-time values.
 //   1 bias -> bf16; 2 bias, GELU -> 8-bit codes; 3 (and 4, its short-reduction form in gemm_i8_t.cu and gemm_i8_p.cu) bias,
-//   optional cache copy, x gate, + residual -> bf16; pair kernel only: 5 as 1 with per-token activation scales; 6 bias -> f32
+//   optional cache copy, x gate, + residual -> bf16; pair kernel only: 5 as 1 with per-token activation scales; 6 bias -> f32;
+//   7 bias, GELU -> f32
 constexpr uint32_t EPI_FLAGS_QKV = QDIT_EPI_BIAS | QDIT_EPI_OUT_BF16;
 constexpr uint32_t EPI_FLAGS_FC1 = QDIT_EPI_BIAS | QDIT_EPI_GELU | QDIT_EPI_QUANT_OUT;
 constexpr uint32_t EPI_FLAGS_GATED = QDIT_EPI_BIAS | QDIT_EPI_GATE | QDIT_EPI_RESIDUAL | QDIT_EPI_OUT_BF16;
 constexpr uint32_t EPI_FLAGS_QKV_ROW = EPI_FLAGS_QKV | QDIT_EPI_ROW_SCALE;
 constexpr uint32_t EPI_FLAGS_F32 = QDIT_EPI_BIAS | QDIT_EPI_OUT_F32;
+constexpr uint32_t EPI_FLAGS_GELU_F32 = EPI_FLAGS_F32 | QDIT_EPI_GELU;
 template <int EPI>
 __device__ __forceinline__ uint32_t epi_flags(const GemmParams& p) {
   return EPI == 1 ? EPI_FLAGS_QKV : EPI == 2 ? EPI_FLAGS_FC1
          : (EPI == 3 || EPI == 4) ? (EPI_FLAGS_GATED | (p.flags & QDIT_EPI_CACHE_STORE))
-         : EPI == 5 ? EPI_FLAGS_QKV_ROW : EPI == 6 ? EPI_FLAGS_F32 : p.flags;
+         : EPI == 5 ? EPI_FLAGS_QKV_ROW : EPI == 6 ? EPI_FLAGS_F32 : EPI == 7 ? EPI_FLAGS_GELU_F32 : p.flags;
 }
 inline int epi_class(uint32_t flags) {
   return flags == EPI_FLAGS_QKV ? 1 : flags == EPI_FLAGS_FC1 ? 2 : (flags & ~QDIT_EPI_CACHE_STORE) == EPI_FLAGS_GATED ? 3
-         : flags == EPI_FLAGS_QKV_ROW ? 5 : flags == EPI_FLAGS_F32 ? 6 : 0;
+         : flags == EPI_FLAGS_QKV_ROW ? 5 : flags == EPI_FLAGS_F32 ? 6 : flags == EPI_FLAGS_GELU_F32 ? 7 : 0;
 }
 
 // 8 packed bytes (16 4-bit codes) -> 16 sign-extended bytes.
@@ -106,7 +109,7 @@ __device__ __forceinline__ void load_col_params(const GemmParams& p, int n, int 
 // Epilogue for 8 consecutive columns of one row; `res` holds the residual's 8 bf16 values (if used).
 template <int EPI>
 __device__ __forceinline__ void epilogue8(const GemmParams& p, const uint4 lo, const uint4 hi, const ColParams& cp,
-                                          const uint4 res, int row, int n, float o_inv) {
+                                          const uint4 res, int row, int n, float o_inv, float& top) {
   const uint32_t flags = epi_flags<EPI>(p);
   const int64_t o = static_cast<int64_t>(row) * p.ldo + n;
   if (flags & QDIT_EPI_OUT_I32) {
@@ -172,6 +175,10 @@ __device__ __forceinline__ void epilogue8(const GemmParams& p, const uint4 lo, c
   } else if (flags & QDIT_EPI_OUT_BF16) {
     *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) + o) = pack_bf16x8(f);
   } else {
+    if (EPI == 0 && p.absmax) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) top = fmaxf(top, fabsf(f[i]));
+    }
     float* of = static_cast<float*>(p.out) + o;
     *reinterpret_cast<float4*>(of) = make_float4(f[0], f[1], f[2], f[3]);
     *reinterpret_cast<float4*>(of + 4) = make_float4(f[4], f[5], f[6], f[7]);
@@ -209,7 +216,7 @@ __device__ __forceinline__ void prefetch_residual(const GemmParams& p, int n, in
 // (`cur`) have been issued before the accumulator was waited for.
 template <int BN, int EPI, int SPLIT = EPI_SPLIT, typename Release>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc, int m0, int n0, int quad, int half,
-                                              uint32_t stg, int lane, float a_scale, float o_inv, ChunkInputs& cur, Release release) {
+                                              uint32_t stg, int lane, float a_scale, float o_inv, ChunkInputs& cur, float& top, Release release) {
   const int cg = lane & 3;     // after the transpose: column group (8 columns) ...
   const int rsub = lane >> 2;  // ... of rows rsub, rsub + 8, rsub + 16, rsub + 24
   const uint32_t flags = epi_flags<EPI>(p);
@@ -268,7 +275,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc
       if (row < p.M && col_ok) {
         if (!gate_uniform && (flags & QDIT_EPI_GATE))
           Load8<float>::load(p.gate + static_cast<int64_t>(row / p.tokens) * p.ld_gate + n, cur.cp.gt);
-        epilogue8<EPI>(p, lo[sidx], hi[sidx], cur.cp, cur.res[sidx], row, n, o_inv);
+        epilogue8<EPI>(p, lo[sidx], hi[sidx], cur.cp, cur.res[sidx], row, n, o_inv, top);
       }
     }
   }
@@ -280,7 +287,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc
 int32_t qdit_launch_gemm_t(qdit_ctx* ctx, const void* A, const void* W, qgemm::GemmParams& p, bool a_unsigned, int bt);
 
 // Token-major tiles of 256 tokens by pairs of CTAs (gemm_i8_p.cu), for the epilogue classes 1, 2 (width and pitch multiples of 16), 3 (samples
-// of whole 32-token chunks), 5 and 6.
+// of whole 32-token chunks), 5, 6 and 7.
 int32_t qdit_launch_gemm_pair(qdit_ctx* ctx, const void* A, const void* W, const qgemm::GemmParams& p, bool a_unsigned);
 double qdit_gemm_pair_cost(const qdit_ctx* ctx, const qgemm::GemmParams& p);   // estimate, in clocks, without what every launch takes
 

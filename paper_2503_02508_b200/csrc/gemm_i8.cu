@@ -172,6 +172,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
     float o_inv = 0.0f;
     if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
+    float top = 0.0f;
     int it = 0;
     bool waited = !p.early;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
@@ -192,9 +193,11 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       __syncwarp();
       tc_fence_after();
       uint64_t* release_bar = &tempty_bar[as];
-      epilogue_tile<BN, EPI>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur,
+      epilogue_tile<BN, EPI>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur, top,
                         [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
+    __syncwarp();
+    if (EPI == 0 && p.absmax) publish_absmax(p.absmax, top);
   }
 
   tc_fence_before();
@@ -275,7 +278,7 @@ int pick_split(qdit_ctx* ctx, int M, int N, int K, int spare) {
 // matrix the packed weights of a many-row layer are widened into first; `early`: see GemmParams.
 int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K, qdit_qparams a_qp,
                          const float* a_scale_dev, uint32_t flags, const qdit_epilogue* epi, void* out, int64_t ldo,
-                         bool packed4, void* w8_scratch, bool early) {
+                         bool packed4, void* w8_scratch, bool early, float* absmax) {
   if (!ctx) return QDIT_ERR_INVALID_ARG;
   if (M < 0 || N < 0 || K < 0) return qdit_fail(ctx, QDIT_ERR_SHAPE, "negative size");
   if (M == 0 || N == 0) return QDIT_OK;
@@ -312,6 +315,7 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
   p.status = ctx->d_status;
   p.tokens = 1;
   p.early = early;
+  p.absmax = absmax;
   if (!(flags & QDIT_EPI_OUT_I32)) {
     if (!epi || !epi->w_scale) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "epilogue with w_scale is required");
     if (!aligned16(epi->w_scale)) return qdit_fail(ctx, QDIT_ERR_ALIGN, "w_scale must be 16-byte aligned");
@@ -389,10 +393,10 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
   // 18.4 / 20.3, 8192 with 4-bit codes 34.2 / 35.9, proj 4096 9.7 / 10.5).
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE]) {
     // (8-bit rows leave through TMA stores of whole 16-byte pieces, and a 32-token chunk of a gated layer has one gate row)
-    const bool staged = cls == 1 || cls == 5 || cls == 6 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0) || (cls == 3 && p.tokens % 32 == 0);
-    const bool slow = cls == 5 || cls == 6;
+    const bool staged = cls == 1 || cls == 5 || cls == 6 || cls == 7 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0) || (cls == 3 && p.tokens % 32 == 0);
+    const bool slow = cls >= 5;
     const bool one_wave = static_cast<int64_t>((p.M + BM - 1) / BM) * ((p.N + 191) / 192) <= ctx->num_sms;
-    if (staged && p.M >= 1024 && (cls == 3 ? p.N >= 1024 && !one_wave : cls != 2 && p.N >= 2304)) {
+    if (staged && p.M >= 1024 && (cls == 3 ? p.N >= 1024 && !one_wave : (cls == 1 || cls == 5 || cls == 6) && p.N >= 2304)) {
       const int64_t waves = (static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) + ctx->num_sms - 1) / ctx->num_sms;
       const double cost = static_cast<double>(waves) * ((p.K + BK - 1) / BK * 620.0 + 600.0) + 4500.0;
       // (f32 output: with one wave only; there the epilogue is the longer part of a tile, 8192 x 3456 x 1152 36.9 us against 33.9)
@@ -416,11 +420,11 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
 extern "C" int32_t qdit_w8a8_linear(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K,
                                     qdit_qparams a_qp, const float* a_scale_dev, uint32_t flags,
                                     const qdit_epilogue* epi, void* out, int64_t ldo) {
-  return qdit_linear_impl(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, false, nullptr, false);
+  return qdit_linear_impl(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, false, nullptr, false, nullptr);
 }
 
 extern "C" int32_t qdit_w4a8_linear(qdit_ctx* ctx, const void* A, const void* W_packed, int64_t M, int64_t N, int64_t K,
                                     qdit_qparams a_qp, const float* a_scale_dev, uint32_t flags,
                                     const qdit_epilogue* epi, void* out, int64_t ldo, void* w8_scratch) {
-  return qdit_linear_impl(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, true, w8_scratch, false);
+  return qdit_linear_impl(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, true, w8_scratch, false, nullptr);
 }

@@ -14,7 +14,7 @@
 // accumulator of a CTA is its 128 tokens (TMEM lanes) x BN channels (columns), two accumulator stages of 256 columns.
 //
 // Epilogues work on chunks of 32 tokens (a lane quadrant) x 32 channels and hand whole tiles to TMA stores:
-//   16-bit and f32 outputs (classes 1, 3, 5, 6): the accumulator is read in the matrix-fragment layout (tcgen05.ld 16x256b), in
+//   16-bit and f32 outputs (classes 1, 3, 5 to 7): the accumulator is read in the matrix-fragment layout (tcgen05.ld 16x256b), in
 //     which a thread holds pairs of adjacent channels of four tokens; scales, bias and gate of its eight channels are pairs of
 //     registers for two-wide arithmetic, stmatrix lays the finished pairs down as swizzled rows.  The residual of the gated
 //     layers comes by TMA one chunk ahead and is read with ldmatrix.
@@ -113,15 +113,17 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {  
 __device__ __forceinline__ float2 to_float2(uint32_t a, uint32_t b) {
   return make_float2(static_cast<float>(static_cast<int>(a)), static_cast<float>(static_cast<int>(b)));
 }
-// gelu_tanh_f of both (the quotient without the handling of subnormal operands, whose code is zero either way)
+// gelu_tanh_f of both (FTZ: the quotient without the handling of subnormal operands, whose code is zero either way)
 __device__ __forceinline__ float div_approx_ftz(float a, float b) {
   float r;
   asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
+template <bool FTZ>
 __device__ __forceinline__ float2 gelu_tanh_f2(float2 x) {
   const float2 u = __fmul2_rn(x, __ffma2_rn(__fmul2_rn(x, x), make_float2(-0.1029432396f, -0.1029432396f), make_float2(-2.3022081998f, -2.3022081998f)));
   const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(ex2_approx(u.x), ex2_approx(u.y)));
+  if (!FTZ) return make_float2(__fdividef(x.x, d.x), __fdividef(x.y, d.y));
   return make_float2(div_approx_ftz(x.x, d.x), div_approx_ftz(x.y, d.y));
 }
 
@@ -362,8 +364,8 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const float4 s4 = *reinterpret_cast<const float4*>(sc + 4 * j), b4 = *reinterpret_cast<const float4*>(bi + 4 * j);
-            const float2 x0 = gelu_tanh_f2(__ffma2_rn(to_float2(v[4 * j], v[4 * j + 1]), make_float2(s4.x, s4.y), make_float2(b4.x, b4.y)));
-            const float2 x1 = gelu_tanh_f2(__ffma2_rn(to_float2(v[4 * j + 2], v[4 * j + 3]), make_float2(s4.z, s4.w), make_float2(b4.z, b4.w)));
+            const float2 x0 = gelu_tanh_f2<true>(__ffma2_rn(to_float2(v[4 * j], v[4 * j + 1]), make_float2(s4.x, s4.y), make_float2(b4.x, b4.y)));
+            const float2 x1 = gelu_tanh_f2<true>(__ffma2_rn(to_float2(v[4 * j + 2], v[4 * j + 3]), make_float2(s4.z, s4.w), make_float2(b4.z, b4.w)));
             // clip(rne(t) + z, qmin, qmax) == rne(clamp(t, qmin - z, qmax - z)) + z; adding 1.5 * 2^23 rounds to nearest-even
             // and leaves the integer in the low mantissa bits; the low byte is the stored code
             float2 t0 = __fmul2_rn(x0, o2), t1 = __fmul2_rn(x1, o2);
@@ -400,6 +402,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
       };
       // Gated: the residual of a chunk is asked for one chunk ahead, into tile `turn` or the other one
       uint64_t* const rbar = res_bar + 2 * e;
+      float top = 0.0f;          // class 7: largest magnitude
       uint32_t r_phase = 0;      // of both tiles' barriers, one bit each
       bool asked = false;        // the next chunk's residual is on its way
       auto ask_residual = [&](const Tile& t, int c, int tile) {
@@ -477,7 +480,18 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             for (int g = 0; g < 4; ++g)
               x[g][k] = __ffma2_rn(frag_acc(a, b, g, k), EPI == 5 ? __fmul2_rn(make_float2(rs[g], rs[g]), s1) : s1, bi[k]);
           }
-          if constexpr (EPI == 6) {
+          if constexpr (EPI == 7) {
+            // The largest magnitude is taken of what is stored: channels past N and tokens past M hold copies and zeros
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+#pragma unroll
+              for (int g = 0; g < 4; ++g) {
+                x[g][k] = gelu_tanh_f2<false>(x[g][k]);
+                if (row0 + 8 * g + (lane >> 2) < p.M && n0 + 8 * k + 2 * (lane & 3) < p.N) top = fmaxf(top, fmaxf(fabsf(x[g][k].x), fabsf(x[g][k].y)));
+              }
+            }
+          }
+          if constexpr (EPI >= 6) {
             // two tiles of 16 tokens x 32 channels of f32: 128-byte rows, 16-byte pieces swizzled by the row
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -554,6 +568,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           }
         }
       }
+      if (EPI == 7 && p.absmax) publish_absmax(p.absmax, top);
       // (after a time-out) a residual still in flight must land before the CTA's shared memory is released
       if (asked) mbar_wait(&rbar[turn], r_phase >> turn & 1u, abort_flag, p.status);
     }
@@ -590,7 +605,7 @@ int32_t launch_p_epi(qdit_ctx* ctx, const void* A, const void* W, const GemmPara
   QDIT_TRY(qdit_get_tmap(ctx, W, p.N, p.K, p.K, static_cast<uint32_t>(bn / 2), BK, 1, 1, &tw));
   CUtensorMap to;
   if (C::CODES) QDIT_TRY(qdit_get_tmap(ctx, p.out, p.M, p.N, p.ldo, 32, 32, 3, 1, &to));
-  else if (EPI == 6) QDIT_TRY(qdit_get_tmap(ctx, p.out, p.M, p.N, p.ldo, 16, 32, 1, 4, &to));
+  else if (EPI >= 6) QDIT_TRY(qdit_get_tmap(ctx, p.out, p.M, p.N, p.ldo, 16, 32, 1, 4, &to));
   else QDIT_TRY(qdit_get_tmap(ctx, p.out, p.M, p.N, p.ldo, 32, 32, 2, 2, &to));
   CUtensorMap tc = to, tr = to;
   if (C::GATED) {
@@ -619,7 +634,7 @@ struct PairTile {
 };
 PairTile pick_pair_tile(const GemmParams& p, int pairs) {
   const int cls = epi_class(p.flags);
-  const int chunk = cls == 1 ? 540 : cls == 2 ? 770 : cls == 3 ? (p.K < SHORT_K ? 650 : 950) : cls == 5 ? 560 : 650;
+  const int chunk = cls == 1 ? 540 : cls == 2 ? 770 : cls == 3 ? (p.K < SHORT_K ? 650 : 950) : cls == 5 ? 560 : cls == 6 ? 650 : 1000;
   const int64_t mt = (p.M + 255) / 256;
   const double num_kb = (p.K + BK - 1) / BK;
   PairTile best{256, 1e30};
@@ -647,6 +662,7 @@ int32_t qdit_launch_gemm_pair(qdit_ctx* ctx, const void* A, const void* W, const
       if (p.K < SHORT_K) return launch_p_epi<4>(ctx, A, W, p, a_unsigned, bn);
       return launch_p_epi<3>(ctx, A, W, p, a_unsigned, bn);
     case 5: return launch_p_epi<5>(ctx, A, W, p, a_unsigned, bn);
+    case 7: return launch_p_epi<7>(ctx, A, W, p, a_unsigned, bn);
     default: return launch_p_epi<6>(ctx, A, W, p, a_unsigned, bn);
   }
 }

@@ -255,6 +255,7 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
   cluster_arrive();
   cluster_wait();
   if (warp >= 2 && !*abort_flag) {
+    float top = 0.0f;
 #pragma unroll 1
     for (int u = warp - 2; u < units; u += SK_EPI_WARPS) {
       if (u != warp - 2) {
@@ -272,8 +273,10 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         lo.x += l.x; lo.y += l.y; lo.z += l.z; lo.w += l.w;
         hi.x += h.x; hi.y += h.y; hi.z += h.z; hi.w += h.w;
       }
-      if (row < p.M && n < p.N) epilogue8<EPI>(p, lo, hi, cp, res, row, n, o_inv);
+      if (row < p.M && n < p.N) epilogue8<EPI>(p, lo, hi, cp, res, row, n, o_inv, top);
     }
+    __syncwarp();
+    if (EPI == 0 && p.absmax) publish_absmax(p.absmax, top);
   }
   if (*abort_flag && warp == 0) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);  // let copies in flight land before shared memory goes away

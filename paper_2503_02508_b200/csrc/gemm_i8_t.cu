@@ -70,7 +70,7 @@ struct TCfg {
 // One 32-token chunk of one channel (this thread): v[j] = accumulator of token m_base + j.
 template <int EPI>
 __device__ __forceinline__ void epilogue_chunk_t(const GemmParams& p, const uint32_t (&v)[32], int n, int m_base,
-                                                 float sc, float bias, int zcs, float o_inv) {
+                                                 float sc, float bias, int zcs, float o_inv, float& top) {
   const uint32_t flags = epi_flags<EPI>(p);
   const int m_end = p.M - m_base < 32 ? p.M - m_base : 32;  // tokens of this chunk inside the matrix
   if (flags & QDIT_EPI_OUT_I32) {
@@ -115,6 +115,7 @@ __device__ __forceinline__ void epilogue_chunk_t(const GemmParams& p, const uint
         } else if (flags & QDIT_EPI_OUT_BF16) {
           static_cast<__nv_bfloat16*>(p.out)[o] = __float2bfloat16_rn(f);
         } else {
+          if (p.absmax) top = fmaxf(top, fabsf(f));
           static_cast<float*>(p.out)[o] = f;
         }
       }
@@ -502,6 +503,7 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
       if (r_inflight) mbar_wait(rbar, r_phase, abort_flag, p.status);
       if (lane == 0) tma_store_wait_all();
     } else {
+      float top = 0.0f;
       int it = 0;
       for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
         const int as = it & 1;
@@ -539,8 +541,10 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             if (lane == 0) mbar_arrive_relaxed(&tempty_bar[as]);
           }
           const int m_base = t0 + c * 32;
-          if (m_base < p.M && n_ok) epilogue_chunk_t<EPI>(p, v, n, m_base, sc, bias, zcs, o_inv);
+          if (m_base < p.M && n_ok) epilogue_chunk_t<EPI>(p, v, n, m_base, sc, bias, zcs, o_inv, top);
         }
+      __syncwarp();
+      if (p.absmax) publish_absmax(p.absmax, top);
       }
     }
   }

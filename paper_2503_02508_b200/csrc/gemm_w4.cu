@@ -200,6 +200,7 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
     float o_inv = 0.0f;
     if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
+    float top = 0.0f;
     int it = 0;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
       const int as = it & 1;
@@ -214,9 +215,11 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       __syncwarp();
       tc_fence_after();
       uint64_t* release_bar = &tempty_bar[as];
-      epilogue_tile<BN, EPI, W4_EPI_WARPS / 4>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur,
+      epilogue_tile<BN, EPI, W4_EPI_WARPS / 4>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur, top,
                              [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
+    __syncwarp();
+    if (EPI == 0 && p.absmax) publish_absmax(p.absmax, top);
   }
 
   tc_fence_before();

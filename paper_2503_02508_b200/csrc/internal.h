@@ -169,11 +169,16 @@ int32_t launch_absmax_to_scale(qdit_ctx* ctx, const float* absmax_dev, float* sc
 int32_t qdit_quantize_act_dev(qdit_ctx* ctx, const float* x, int64_t M, int64_t K, qdit_qparams qp,
                               const float* scale_dev, uint8_t* q);
 // qdit_w8a8_linear (or qdit_w4a8_linear: packed4) for the model's own layers, whose weights, scales, biases and gates were written at
-// least two launches ago (`early`).
+// least two launches ago (`early`).  In this and the next two calls `absmax`, if given, takes the largest magnitude of an f32 output.
 int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K, qdit_qparams a_qp,
                          const float* a_scale_dev, uint32_t flags, const qdit_epilogue* epi, void* out, int64_t ldo, bool packed4,
-                         void* w8_scratch, bool early);
+                         void* w8_scratch, bool early, float* absmax = nullptr);
 // qdit_adaln_modulate; `early`: modulation and scale were written at least two launches ago (both kernels of a pair of launches may be
 // resident at once, but every kernel lets its successor start only after its own wait, so the launch before the previous one is complete)
 int32_t qdit_adaln_impl(qdit_ctx* ctx, const void* x, int64_t M, int64_t D, int64_t T, float eps, const float* shift, const float* scale,
-                        int64_t ld_mod, void* out, int out_dtype, const qdit_qparams* out_qp, const float* out_scale_dev, bool early);
+                        int64_t ld_mod, void* out, int out_dtype, const qdit_qparams* out_qp, const float* out_scale_dev, bool early, float* absmax = nullptr);
+int32_t qdit_attention_impl(qdit_ctx* ctx, const void* q, const void* k, const void* v, int64_t ld, int B, int H, int T, int dh, float softmax_scale,
+                            void* out, int out_dtype, const qdit_qparams* out_qp, const float* out_scale_dev, float* absmax);
+// The quantizer behind one of these calls whose f32 output's largest magnitude went to *absmax (which was zero before): codes, the scale
+// in *scale, the magnitude folded into *running; x contiguous, K % 16 == 0.
+int32_t launch_quant_absmax(qdit_ctx* ctx, const float* x, int64_t M, int64_t K, const float* absmax, float* scale, float* running, void* q);

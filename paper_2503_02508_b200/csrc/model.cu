@@ -69,6 +69,7 @@ struct qdit_sampler {
   float *c, *sc, *hidden, *feat, *mod, *modf, *net, *latent, *t_all, *tmpf;   // t_all: [S, Beff] timestep of every step
   int32_t *y, *labels;
   float* dyn_scale;              // [1 + 4*depth] scales of this pass's ranges (calibration)
+  float* dyn_absmax;             // [1 + 4*depth] the ranges, folded together by the kernels that write the quantizers' inputs
   int8_t* w8_scratch;            // [max N*K] int8: a packed block-level weight matrix widened for the many-row kernels
   float* vc_table;               // device [S, C] or null
   // Conditioning of the whole trajectory, evaluated at step 0: the conditioning vector, and with it every block's
@@ -203,12 +204,12 @@ qdit_qparams sym_qp() { return qdit_qparams{1.0f, 0, -127, 127}; }
 // `w8_scratch`: for a layer stored packed, the matrix its weights are widened into when the layer has many rows
 // (NULL: always widened inside the GEMM kernel, which is the form for the weight-streaming modulation GEMM).
 int32_t run_linear(qdit_ctx* ctx, const void* A, const QLinearDev& l, int64_t M, const float* a_scale_dev, uint32_t flags,
-                   qdit_epilogue epi, void* out, bool calib, void* w8_scratch = nullptr) {
+                   qdit_epilogue epi, void* out, bool calib, void* w8_scratch = nullptr, float* absmax = nullptr) {
   epi.w_scale = l.scale;
   epi.w_colsum = l.colsum;
   epi.bias = l.bias;
   return qdit_linear_impl(ctx, A, l.q, M, l.N, l.K, sym_qp(), a_scale_dev, flags | QDIT_EPI_BIAS, &epi, out, l.N, l.packed4,
-                          l.packed4 ? w8_scratch : nullptr, !calib);
+                          l.packed4 ? w8_scratch : nullptr, !calib, absmax);
 }
 
 // The modulation linears of all blocks on `rows` conditioning rows: out[rows, depth * 6D].  One stacked GEMM; with
@@ -230,9 +231,13 @@ int32_t run_modulation(qdit_ctx* ctx, const qdit_model* m, const void* A, int64_
   return QDIT_OK;
 }
 
-// Calibration helper: range of an f32 tensor -> this pass's scale slot (and the running range), then codes.
+// Calibration helpers: range of an f32 tensor -> this pass's scale slot (and the running range), then codes.  dyn_quant finds the range,
+// quant_behind takes the one that the tensor's producer has left in the slot.
 int32_t dyn_quant(qdit_ctx* ctx, qdit_sampler* s, int slot, const float* x, int64_t M, int64_t K, uint8_t* q) {
   return launch_quant_dynamic(ctx, x, QDIT_F32, M, K, K, s->dyn_scale + slot, s->model->d_absmax_run + slot, q, K);
+}
+int32_t quant_behind(qdit_ctx* ctx, qdit_sampler* s, int slot, const float* x, int64_t M, int64_t K, uint8_t* q) {
+  return launch_quant_absmax(ctx, x, M, K, s->dyn_absmax + slot, s->dyn_scale + slot, s->model->d_absmax_run + slot, q);
 }
 
 }  // namespace
@@ -255,6 +260,7 @@ static int32_t forward_impl(qdit_ctx* ctx, qdit_sampler* s, const float* latent,
   if (!calib && !m->scales_set) return qdit_fail(ctx, QDIT_ERR_STATE, "activation scales are not set (set them or calibrate)");
   if (reuse && (store || calib)) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "REUSE cannot be combined with STORE_CACHE or CALIBRATE");
   const float* scales = calib ? s->dyn_scale : m->d_scales;
+  if (calib) QDIT_CUDA_CHECK(ctx, cudaMemsetAsync(s->dyn_absmax, 0, m->n_scales() * sizeof(float), ctx->stream));
 
   QDIT_TRY(launch_embed(ctx, latent, latent_batch, m->w_patch, m->w_patch_frag, m->b_patch, m->pos, s->x, M, D, sh.grid, sh.patch, sh.channels));
   const float* mod_all = pre_mod;
@@ -317,23 +323,24 @@ static int32_t forward_impl(qdit_ctx* ctx, qdit_sampler* s, const float* latent,
           QDIT_TRY(run_linear(ctx, s->u, m->fc2[i], M, sc_fc2, gflags, gated, s->x, calib, s->w8_scratch));
         }
       } else {
-        // ---- calibration: every quantizer input is materialised in f32, its range reduced, then quantized
-        QDIT_TRY(qdit_adaln_modulate(ctx, s->x, M, D, T, 1e-6f, mod, mod + D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr));
-        QDIT_TRY(dyn_quant(ctx, s, 1 + 4 * i, s->tmpf, M, D, s->h));
+        // ---- calibration: every quantizer input is materialised in f32, its range found by the kernel that writes it, then quantized
+        float* const top = s->dyn_absmax + 1 + 4 * i;
+        QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod, mod + D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr, false, top));
+        QDIT_TRY(quant_behind(ctx, s, 1 + 4 * i, s->tmpf, M, D, s->h));
         qdit_epilogue e0{};
         QDIT_TRY(run_linear(ctx, s->h, m->qkv[i], M, sc_qkv, QDIT_EPI_OUT_BF16, e0, s->qkv, calib, s->w8_scratch));
         const __nv_bfloat16* qkv = static_cast<const __nv_bfloat16*>(s->qkv);
-        QDIT_TRY(qdit_attention(ctx, qkv, qkv + D, qkv + 2 * D, 3 * D, B, sh.heads, T, D / sh.heads, att_scale, s->tmpf,
-                                QDIT_F32, nullptr, nullptr));
-        QDIT_TRY(dyn_quant(ctx, s, 2 + 4 * i, s->tmpf, M, D, s->a));
+        QDIT_TRY(qdit_attention_impl(ctx, qkv, qkv + D, qkv + 2 * D, 3 * D, B, sh.heads, T, D / sh.heads, att_scale, s->tmpf,
+                                     QDIT_F32, nullptr, nullptr, top + 1));
+        QDIT_TRY(quant_behind(ctx, s, 2 + 4 * i, s->tmpf, M, D, s->a));
         gated.gate = mod + 2 * D;
         gated.cache_out = store ? qdit_cache_slot(s->cache, i, QDIT_BRANCH_ATTN, 1) : nullptr;
         QDIT_TRY(run_linear(ctx, s->a, m->proj[i], M, sc_proj, gflags, gated, s->x, calib, s->w8_scratch));
-        QDIT_TRY(qdit_adaln_modulate(ctx, s->x, M, D, T, 1e-6f, mod + 3 * D, mod + 4 * D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr));
-        QDIT_TRY(dyn_quant(ctx, s, 3 + 4 * i, s->tmpf, M, D, s->h));
+        QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod + 3 * D, mod + 4 * D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr, false, top + 2));
+        QDIT_TRY(quant_behind(ctx, s, 3 + 4 * i, s->tmpf, M, D, s->h));
         qdit_epilogue e1{};
-        QDIT_TRY(run_linear(ctx, s->h, m->fc1[i], M, sc_fc1, QDIT_EPI_GELU | QDIT_EPI_OUT_F32, e1, s->tmpf, calib, s->w8_scratch));
-        QDIT_TRY(dyn_quant(ctx, s, 4 + 4 * i, s->tmpf, M, F, s->u));
+        QDIT_TRY(run_linear(ctx, s->h, m->fc1[i], M, sc_fc1, QDIT_EPI_GELU | QDIT_EPI_OUT_F32, e1, s->tmpf, calib, s->w8_scratch, top + 3));
+        QDIT_TRY(quant_behind(ctx, s, 4 + 4 * i, s->tmpf, M, F, s->u));
         gated.gate = mod + 5 * D;
         gated.cache_out = store ? qdit_cache_slot(s->cache, i, QDIT_BRANCH_MLP, 1) : nullptr;
         QDIT_TRY(run_linear(ctx, s->u, m->fc2[i], M, sc_fc2, gflags, gated, s->x, calib, s->w8_scratch));
@@ -516,6 +523,7 @@ int32_t qdit_sampler_create(qdit_ctx* ctx, qdit_model* m, const qdit_sampler_des
   s->tmpf = a.alloc<float>(M * F);
   s->w8_scratch = m->packed4 ? a.alloc<int8_t>(m->max_block_weight) : nullptr;
   s->dyn_scale = a.alloc<float>(m->n_scales());
+  s->dyn_absmax = a.alloc<float>(m->n_scales());
   // conditioning of as many steps at once as a 4 GB modulation table holds (all of them for the paper's 50- and
   // 100-step settings; a 250-step trajectory at network batch 32 goes in chunks of 173 steps)
   bool traj_ok = true;
@@ -542,7 +550,7 @@ int32_t qdit_sampler_create(qdit_ctx* ctx, qdit_model* m, const qdit_sampler_des
     }
   }
   bool ok = traj_ok && s->x && s->qkv && s->h && s->a && s->u && s->ca && s->c && s->sc && s->hidden && s->feat && s->mod && s->modf && s->net &&
-            s->latent && s->t_all && s->y && s->labels && s->tmpf && s->dyn_scale && (!m->packed4 || s->w8_scratch);
+            s->latent && s->t_all && s->y && s->labels && s->tmpf && s->dyn_scale && s->dyn_absmax && (!m->packed4 || s->w8_scratch);
   if (ok && d->vc_mode != QDIT_VC_NONE) {
     s->vc_table = a.alloc<float>(static_cast<int64_t>(d->num_steps) * C);
     ok = s->vc_table && cudaMemcpy(s->vc_table, d->vc_table, sizeof(float) * d->num_steps * C, cudaMemcpyHostToDevice) == cudaSuccess;

@@ -573,7 +573,8 @@ def test_packed_weights_with_a_split_reduction(q, ctx, M, N, K, kind):
     (19200, 384, 384, 256),     # narrow layer, many tiles per pair
     (300, 44000, 1152, 32),     # weights of more than 48 MB: tiles along the tokens first
 ])
-@pytest.mark.parametrize("kind,zp", [("f32", 0), ("bf16", 0), ("bf16", 131), ("row", 0), ("gelu", 0), ("gelu", 131), ("gated", 0), ("gated_nocache", 131)])
+@pytest.mark.parametrize("kind,zp", [("f32", 0), ("bf16", 0), ("bf16", 131), ("row", 0), ("gelu", 0), ("gelu", 131), ("gelu_f32", 0),
+                                     ("gated", 0), ("gated_nocache", 131)])
 def test_pair_kernel_gives_the_bits_of_the_token_major_kernel(q, ctx, M, N, K, T, kind, zp):
     """Pairs of CTAs: whatever tile width the rule takes, exact integer sums and the same f32 epilogue as the plain token-major
     kernel with run-time epilogue flags; the padding of the rows stays untouched."""
@@ -587,10 +588,10 @@ def test_pair_kernel_gives_the_bits_of_the_token_major_kernel(q, ctx, M, N, K, T
     rows = torch.rand(M, generator=g, device="cuda") + 0.1
     flags = {"f32": q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_F32, "bf16": q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_BF16,
              "row": q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_BF16 | q.QDIT_EPI_ROW_SCALE,
-             "gelu": q.QDIT_EPI_BIAS | q.QDIT_EPI_GELU | q.QDIT_EPI_QUANT_OUT,
+             "gelu": q.QDIT_EPI_BIAS | q.QDIT_EPI_GELU | q.QDIT_EPI_QUANT_OUT, "gelu_f32": q.QDIT_EPI_BIAS | q.QDIT_EPI_GELU | q.QDIT_EPI_OUT_F32,
              "gated": q.QDIT_EPI_BIAS | q.QDIT_EPI_GATE | q.QDIT_EPI_RESIDUAL | q.QDIT_EPI_OUT_BF16 | q.QDIT_EPI_CACHE_STORE,
              "gated_nocache": q.QDIT_EPI_BIAS | q.QDIT_EPI_GATE | q.QDIT_EPI_RESIDUAL | q.QDIT_EPI_OUT_BF16}[kind]
-    dtype = {"f32": torch.float32, "gelu": torch.int8}.get(kind, torch.bfloat16)
+    dtype = {"f32": torch.float32, "gelu_f32": torch.float32, "gelu": torch.int8}.get(kind, torch.bfloat16)
     ldo = -(-N // 16) * 16 + 16
     qp = q.qparams(0.03, zp, 0, 255) if zp else q.qparams(0.03)
 

@@ -42,3 +42,39 @@ def test_overlapped_evaluations_equal_plain_ones(bits, B):
         q.qdit_model_destroy(model)
         q.qdit_destroy(ctx)
     assert torch.isfinite(got[0]).all() and torch.equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("bits,B", [(8, 1), (8, 5), (4, 2)])
+def test_ranges_found_by_the_writing_kernels(bits, B):
+    """Calibration ranges are folded together by the kernels that write the quantizers' inputs (LayerNorm, attention on tcgen05, GELU layer
+    token-major, by pairs and with packed weights): against the same pass of the oracle; a second pass starts from zero."""
+    import paper_2503_02508_b200 as q
+    from oracle import calib, dit
+    cfg = synth.DIT_S2_BLOCK
+    w = synth.model_weights(11, cfg)
+    latent = synth.normal(11, "latent", (B, cfg.channels, cfg.latent_side, cfg.latent_side))
+    t, y = np.full(B, 500.0), synth.uniform_int(11, "y", (B,), 0, cfg.num_classes)
+    ref = calib.calibrate_model(dit.make_qmodel(cfg, w, bits), [(latent, t, y)])
+    ctx = q.qdit_create(0, None)
+    model = q.qdit_model_create(ctx, cfg, w, bits)
+    s = q.qdit_sampler_create(ctx, model, batch=B, num_steps=10)
+    out = torch.empty(B, 2 * cfg.channels, cfg.latent_side, cfg.latent_side, device="cuda")
+    dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (latent, t.astype(np.float32), y.astype(np.int32))]
+    torch.cuda.synchronize()
+    got = []
+    for scale in (8.0, 1.0):     # the larger inputs first: their ranges must not stay
+        x = (dev[0] * scale).contiguous()
+        torch.cuda.synchronize()
+        q.qdit_model_begin_calibration(ctx, model)
+        q.qdit_forward(ctx, s, x, dev[1], dev[2], B, out, q.QDIT_FWD_CALIBRATE)
+        q.qdit_model_finish_calibration(ctx, model)
+        got.append(q.qdit_model_get_act_scales(ctx, model, cfg.depth))
+    q.qdit_sync(ctx)
+    ada, blocks = got[1]
+    want = np.array([[ref.blocks[i][n].scale for n in ("qkv", "proj", "fc1", "fc2")] for i in range(cfg.depth)])
+    # a flipped code in front moves a later maximum by a quantization step of its inputs, not by rounding: 1 % (f32 alone gives 1e-5)
+    assert abs(ada / ref.ada.scale - 1.0) < 1e-5 and np.abs(blocks / want - 1.0).max() < 1e-2
+    assert not np.allclose(got[0][1], blocks, rtol=1e-3)
+    q.qdit_sampler_destroy(s)
+    q.qdit_model_destroy(model)
+    q.qdit_destroy(ctx)
