@@ -42,9 +42,10 @@ struct GemmParams {
   int64_t ldo;
   int* status;
   int num_m_tiles, num_n_tiles;
-  // The weights, their scales and biases, the gate and the quantizer scales were written two launches ago or earlier: a kernel that has
-  // started beside its predecessor may read them before it waits for it (every kernel lets its successor start after its own wait).
-  bool early;
+  // The weights (early_params: their scales and biases, the gate and the quantizer scales too) were written two launches ago or earlier: a
+  // kernel that has started beside its predecessor may read them before it waits for it (every kernel lets its successor start only
+  // after its own wait).
+  bool early, early_params;
   float* absmax;   // f32 output: the largest magnitude is folded into this, if given (calibration; run-time-flag and GELU -> f32 epilogues)
 };
 

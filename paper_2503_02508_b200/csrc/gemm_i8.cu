@@ -168,13 +168,13 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const int quad = warp & 3;   // TMEM lane quadrant this warp may access
     const int half = e >> 2;     // this warp takes chunks half, half + EPI_SPLIT, ...
     const uint32_t stg = smem_u32(staging + e * (32 * 128));  // [32 rows][8 x 16 B], 16-byte index XOR (row & 7)
-    if (!p.early) grid_dependency_wait();
+    if (!p.early_params) grid_dependency_wait();
     const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
     float o_inv = 0.0f;
     if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
     float top = 0.0f;
     int it = 0;
-    bool waited = !p.early;
+    bool waited = !p.early_params;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
       const int as = it & 1;
       const uint32_t aphase = static_cast<uint32_t>(it >> 1) & 1u;
@@ -275,10 +275,10 @@ int pick_split(qdit_ctx* ctx, int M, int N, int K, int spare) {
 }  // namespace
 
 // Both linear layers: `packed4` = W holds 4-bit codes two per byte ([N, K/2]); `w8_scratch` = optional [N, K] int8
-// matrix the packed weights of a many-row layer are widened into first; `early`: see GemmParams.
+// matrix the packed weights of a many-row layer are widened into first; `early`, `early_params`, `absmax`: see GemmParams.
 int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K, qdit_qparams a_qp,
                          const float* a_scale_dev, uint32_t flags, const qdit_epilogue* epi, void* out, int64_t ldo,
-                         bool packed4, void* w8_scratch, bool early, float* absmax) {
+                         bool packed4, void* w8_scratch, bool early, bool early_params, float* absmax) {
   if (!ctx) return QDIT_ERR_INVALID_ARG;
   if (M < 0 || N < 0 || K < 0) return qdit_fail(ctx, QDIT_ERR_SHAPE, "negative size");
   if (M == 0 || N == 0) return QDIT_OK;
@@ -315,6 +315,7 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
   p.status = ctx->d_status;
   p.tokens = 1;
   p.early = early;
+  p.early_params = early_params;
   p.absmax = absmax;
   if (!(flags & QDIT_EPI_OUT_I32)) {
     if (!epi || !epi->w_scale) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "epilogue with w_scale is required");
@@ -420,11 +421,11 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
 extern "C" int32_t qdit_w8a8_linear(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K,
                                     qdit_qparams a_qp, const float* a_scale_dev, uint32_t flags,
                                     const qdit_epilogue* epi, void* out, int64_t ldo) {
-  return qdit_linear_impl(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, false, nullptr, false, nullptr);
+  return qdit_linear_impl(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, false, nullptr, false, false, nullptr);
 }
 
 extern "C" int32_t qdit_w4a8_linear(qdit_ctx* ctx, const void* A, const void* W_packed, int64_t M, int64_t N, int64_t K,
                                     qdit_qparams a_qp, const float* a_scale_dev, uint32_t flags,
                                     const qdit_epilogue* epi, void* out, int64_t ldo, void* w8_scratch) {
-  return qdit_linear_impl(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, true, w8_scratch, false, nullptr);
+  return qdit_linear_impl(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, true, w8_scratch, false, false, nullptr);
 }

@@ -130,12 +130,12 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     if (row < p.M && n < p.N && (flags & QDIT_EPI_RESIDUAL)) res = *reinterpret_cast<const uint4*>(p.residual + static_cast<int64_t>(row) * p.ldo + n);
   };
   if (warp >= 2) {
-    if (!p.early) grid_dependency_wait();
+    if (!p.early_params) grid_dependency_wait();
     a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
     if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
     // (warps that widen weights first do not wait for the parameters in front of that)
-    if ((!W4 || p.early) && warp - 2 < units) prefetch_columns(warp - 2);
-    if (p.early) grid_dependency_wait();
+    if ((!W4 || p.early_params) && warp - 2 < units) prefetch_columns(warp - 2);
+    if (p.early_params) grid_dependency_wait();
     grid_dependency_release();
     if (warp - 2 < units) prefetch_row(warp - 2);
   }
@@ -227,7 +227,7 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
-    if (W4 && !p.early && warp - 2 < units) prefetch_columns(warp - 2);
+    if (W4 && !p.early_params && warp - 2 < units) prefetch_columns(warp - 2);
     accumulated = ok && mbar_wait_warp(tfull_bar, 0, abort_flag, p.status);
   }
   cluster_wait();

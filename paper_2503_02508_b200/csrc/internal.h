@@ -168,11 +168,11 @@ int32_t launch_absmax_to_scale(qdit_ctx* ctx, const float* absmax_dev, float* sc
 // Quantizes an f32 tensor [M,K] (contiguous) with the scale held in device memory.
 int32_t qdit_quantize_act_dev(qdit_ctx* ctx, const float* x, int64_t M, int64_t K, qdit_qparams qp,
                               const float* scale_dev, uint8_t* q);
-// qdit_w8a8_linear (or qdit_w4a8_linear: packed4) for the model's own layers, whose weights, scales, biases and gates were written at
-// least two launches ago (`early`).  In this and the next two calls `absmax`, if given, takes the largest magnitude of an f32 output.
+// qdit_w8a8_linear (or qdit_w4a8_linear: packed4) for the model's own layers, whose weights (`early`), weight scales, biases, gates and
+// quantizer scales (`early_params`) were written at least two launches ago.  In this and the next two calls `absmax`, if given, takes the largest magnitude of an f32 output.
 int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M, int64_t N, int64_t K, qdit_qparams a_qp,
                          const float* a_scale_dev, uint32_t flags, const qdit_epilogue* epi, void* out, int64_t ldo, bool packed4,
-                         void* w8_scratch, bool early, float* absmax = nullptr);
+                         void* w8_scratch, bool early, bool early_params, float* absmax = nullptr);
 // qdit_adaln_modulate; `early`: modulation and scale were written at least two launches ago (both kernels of a pair of launches may be
 // resident at once, but every kernel lets its successor start only after its own wait, so the launch before the previous one is complete)
 int32_t qdit_adaln_impl(qdit_ctx* ctx, const void* x, int64_t M, int64_t D, int64_t T, float eps, const float* shift, const float* scale,

@@ -209,7 +209,7 @@ int32_t run_linear(qdit_ctx* ctx, const void* A, const QLinearDev& l, int64_t M,
   epi.w_colsum = l.colsum;
   epi.bias = l.bias;
   return qdit_linear_impl(ctx, A, l.q, M, l.N, l.K, sym_qp(), a_scale_dev, flags | QDIT_EPI_BIAS, &epi, out, l.N, l.packed4,
-                          l.packed4 ? w8_scratch : nullptr, !calib, absmax);
+                          l.packed4 ? w8_scratch : nullptr, true, !calib, absmax);
 }
 
 // The modulation linears of all blocks on `rows` conditioning rows: out[rows, depth * 6D].  One stacked GEMM; with
@@ -325,7 +325,7 @@ static int32_t forward_impl(qdit_ctx* ctx, qdit_sampler* s, const float* latent,
       } else {
         // ---- calibration: every quantizer input is materialised in f32, its range found by the kernel that writes it, then quantized
         float* const top = s->dyn_absmax + 1 + 4 * i;
-        QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod, mod + D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr, false, top));
+        QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod, mod + D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr, i > 0 || pre_mod, top));
         QDIT_TRY(quant_behind(ctx, s, 1 + 4 * i, s->tmpf, M, D, s->h));
         qdit_epilogue e0{};
         QDIT_TRY(run_linear(ctx, s->h, m->qkv[i], M, sc_qkv, QDIT_EPI_OUT_BF16, e0, s->qkv, calib, s->w8_scratch));
@@ -336,7 +336,7 @@ static int32_t forward_impl(qdit_ctx* ctx, qdit_sampler* s, const float* latent,
         gated.gate = mod + 2 * D;
         gated.cache_out = store ? qdit_cache_slot(s->cache, i, QDIT_BRANCH_ATTN, 1) : nullptr;
         QDIT_TRY(run_linear(ctx, s->a, m->proj[i], M, sc_proj, gflags, gated, s->x, calib, s->w8_scratch));
-        QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod + 3 * D, mod + 4 * D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr, false, top + 2));
+        QDIT_TRY(qdit_adaln_impl(ctx, s->x, M, D, T, 1e-6f, mod + 3 * D, mod + 4 * D, ld_mod, s->tmpf, QDIT_F32, nullptr, nullptr, true, top + 2));
         QDIT_TRY(quant_behind(ctx, s, 3 + 4 * i, s->tmpf, M, D, s->h));
         qdit_epilogue e1{};
         QDIT_TRY(run_linear(ctx, s->h, m->fc1[i], M, sc_fc1, QDIT_EPI_GELU | QDIT_EPI_OUT_F32, e1, s->tmpf, calib, s->w8_scratch, top + 3));

@@ -287,18 +287,19 @@ __global__ void __launch_bounds__(256) ln_modulate_kernel(const __nv_bfloat16* _
                                                           float eps, const float* __restrict__ shift,
                                                           const float* __restrict__ scale, int64_t ld_mod,
                                                           void* __restrict__ out, int out_dtype, QuantArgs qa,
-                                                          int rows_per_cta, float* __restrict__ absmax) {
+                                                          int rows_per_cta, int early, float* __restrict__ absmax) {
   extern __shared__ float4 s_par[];  // [2 samples][mul, add][NV][2 halves][32 lanes]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int row_begin = blockIdx.x * rows_per_cta;
   const int row_end = row_begin + rows_per_cta < M ? row_begin + rows_per_cta : M;
   if (row_begin >= M) return;
-  grid_dependency_wait();  // x and the modulation come from earlier kernels of the stream
-  grid_dependency_release();
   const int nvec = D >> 3;
   int row = row_begin + warp;
   uint4 raw[NV], raw_next[NV];
-  if (row < row_end) ln_load_row<NV>(x + static_cast<int64_t>(row) * D, nvec, lane, raw);
+  if (!early) {   // (see ln_modulate_q8_kernel)
+    grid_dependency_wait();
+    if (row < row_end) ln_load_row<NV>(x + static_cast<int64_t>(row) * D, nvec, lane, raw);
+  }
   float inv = 1.0f;
   if (out_dtype == QDIT_I8) inv = __fdiv_rn(1.0f, qa.scale_dev ? __ldg(qa.scale_dev) : qa.scale);
   const int b0 = row_begin / T;
@@ -317,6 +318,11 @@ __global__ void __launch_bounds__(256) ln_modulate_kernel(const __nv_bfloat16* _
       }
     }
   }
+  if (early) {
+    grid_dependency_wait();
+    if (row < row_end) ln_load_row<NV>(x + static_cast<int64_t>(row) * D, nvec, lane, raw);
+  }
+  grid_dependency_release();
   __syncthreads();
   const float inv_d = 1.0f / static_cast<float>(D);
   const int64_t second = static_cast<int64_t>(b0 + 1) * T;  // first row of the second staged sample
@@ -524,12 +530,12 @@ int64_t ln_rows_per_cta(const qdit_ctx* ctx, int64_t M, int64_t T, int per_sm) {
 
 template <int NV>
 void launch_ln(qdit_ctx* ctx, const void* x, int64_t M, int D, int64_t T, float eps, const float* shift,
-               const float* scale, int64_t ld_mod, void* out, int out_dtype, QuantArgs qa, float* absmax) {
+               const float* scale, int64_t ld_mod, void* out, int out_dtype, QuantArgs qa, bool early, float* absmax) {
   const int64_t rows = ln_rows_per_cta(ctx, M, T, 2);
   const unsigned grid = static_cast<unsigned>((M + rows - 1) / rows);
   qdit_launch_overlapped(ctx, absmax ? ln_modulate_kernel<NV, true> : ln_modulate_kernel<NV, false>, dim3(grid), dim3(256), static_cast<size_t>(NV) * 4096,
                          static_cast<const __nv_bfloat16*>(x), static_cast<int>(M), D, static_cast<int>(T), eps, shift, scale,
-                         ld_mod, out, out_dtype, qa, static_cast<int>(rows), absmax);
+                         ld_mod, out, out_dtype, qa, static_cast<int>(rows), static_cast<int>(early), absmax);
 }
 
 }  // namespace
@@ -714,14 +720,14 @@ int32_t qdit_adaln_impl(qdit_ctx* ctx, const void* x, int64_t M, int64_t D, int6
     if (done) return qdit_after_launch(ctx, "ln_modulate_q8_kernel");
   }
   switch (nv) {
-    case 1: launch_ln<1>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
-    case 2: launch_ln<2>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
-    case 3: launch_ln<3>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
-    case 4: launch_ln<4>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
-    case 5: launch_ln<5>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
-    case 6: launch_ln<6>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
-    case 7: launch_ln<7>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
-    default: launch_ln<8>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, absmax); break;
+    case 1: launch_ln<1>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
+    case 2: launch_ln<2>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
+    case 3: launch_ln<3>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
+    case 4: launch_ln<4>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
+    case 5: launch_ln<5>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
+    case 6: launch_ln<6>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
+    case 7: launch_ln<7>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
+    default: launch_ln<8>(ctx, x, M, d, T, eps, shift, scale, ld_mod, out, out_dtype, qa, early, absmax); break;
   }
   return qdit_after_launch(ctx, "ln_modulate_kernel");
 }
