@@ -25,9 +25,16 @@
 // A row's exponents have its maximum so far as reference.  The accumulator is rescaled in tensor memory when some row of a warp
 // has a new maximum, at the end of the block's softmax, when the product before it has usually ended.
 //
-// 8 x 16 x 1024 x 72 takes 61 us, 32 x 16 x 256 x 72 22 us, 7 x 16 x 576 x 72 27 us and 1 x 16 x 1024 x 72 12.8 us; one stream of
-// blocks per query tile, two tiles per CTA, took 75, 25, 37 and 17.  (There a quarter of the exponentials was a polynomial on the
-// FMA pipe, which shortened the hand-overs.  Here it does not pay: 64 us with a quarter, 79 with half of them.)
+// A block takes about 1600 clocks, which is the chain through the accumulator: product complete, seen by the softmax warps (200),
+// rescaled (350), seen by the issuer (250), the next product (700).  Waits in that chain poll (mbar_poll_warp), and the softmax warps
+// look at their next scores before the last exponentials; the output warps, which wait long, use try_wait.  With try_wait everywhere /
+// polling / and the early look: 8 x 16 x 1024 x 72 61.1 / 56.5 / 55.4 us, 32 x 16 x 256 x 72 23.2 / 20.0 / 19.8, 8 x 16 x 576 x 72 29.5 /
+// 27.9 / 27.7, 1 x 16 x 1024 x 72 12.5 / 12.3 / 12.2.
+//
+// Tried and slower: one stream of blocks per query tile, two tiles per CTA (75 us for 8 x 16 x 1024 x 72); a quarter or half of the
+// exponentials as a polynomial on the FMA pipe (+5 %, +30 %); four more warps that only rescale (2 to 5 % faster above 800 tokens,
+// up to 9 % slower below 320); a fresh accumulator per block, summed in the registers of eight warps (+40 %: their
+// tensor-memory reads hold up the exponentials and the issue of the products).
 //
 // Head dim 72 does not fill a 128-byte swizzle row: columns 0..63 are a 128-byte-swizzled tile, columns 64..71 an
 // 8-column tile without swizzle, which the products read as the first half of a 16-wide step; the second half comes
@@ -225,13 +232,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     };
     grid_dependency_wait();
     int j = group;   // key block of the item
+    bool seen_s = false;
 #pragma unroll 1
     for (int n = group; n < n_total; n += 2, j += 2) {
       while (j >= p.n_blk) j -= p.n_blk;
       const bool full = j > 0 || p.T % TK == 0;  // else 64 keys
       const int buf = n % RING;
       const uint32_t s_col = trow + col_s(buf), p_col = trow + col_p(buf);
-      if (!mbar_wait_warp(&s_full[buf], static_cast<uint32_t>(n / RING) & 1u, abort_flag, p.status)) break;
+      if (!mbar_poll_seen(seen_s, &s_full[buf], static_cast<uint32_t>(n / RING) & 1u, abort_flag, p.status)) break;
       tc_fence_after();
       uint32_t va[32], vb[32], pa[16], pb[16];
       float mx, alpha = 1.0f;
@@ -254,7 +262,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       mx = row_max(vb, mx) * p.scale_log2;
       // The maximum of the blocks before comes from the other group, which is half a block ahead; it is waited for at an item's
       // first block too, so that neither group can be two blocks ahead of the other's look at its barrier.
-      if (!mbar_wait_seen(seen_max, &max_ready[(group ^ 1) * 4 + quad], static_cast<uint32_t>((n - 1) >> 1) & 1u, abort_flag, p.status)) break;
+      if (!mbar_poll_seen(seen_max, &max_ready[(group ^ 1) * 4 + quad], static_cast<uint32_t>((n - 1) >> 1) & 1u, abort_flag, p.status)) break;
       if (j > 0) {
         const float before = *other_max;
         grew = __any_sync(0xffffffffu, mx > before);
@@ -281,10 +289,13 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         probs(vb, pb);
         tmem_st_32x16(p_col, pb);
         tmem_ld_wait_for(va);
+        // looks at the barriers behind this block: the scores of the group's next one and the previous product
+        seen_s = n + 2 < n_total && mbar_test_wait(&s_full[(n + 2) % RING], static_cast<uint32_t>((n + 2) / RING) & 1u);
         seen_pv = grew && mbar_test_wait(&pv_done[(n - 1) % RING], static_cast<uint32_t>((n - 1) / RING) & 1u);
         probs(va, pa);
         tmem_st_32x16(p_col + 16, pa);
       } else {
+        seen_s = false;
         probs(va, pa);
         tmem_st_32x16(p_col, pa);
         probs(vb, pb);
@@ -292,7 +303,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       if (grew) {
         // some row of the warp has a new maximum: rescale what has been summed, once the previous product has added its part
-        if (!mbar_wait_seen(seen_pv, &pv_done[(n - 1) % RING], static_cast<uint32_t>((n - 1) / RING) & 1u, abort_flag, p.status)) break;
+        if (!mbar_poll_seen(seen_pv, &pv_done[(n - 1) % RING], static_cast<uint32_t>((n - 1) / RING) & 1u, abort_flag, p.status)) break;
         tc_fence_after();
         tmem_ld_32x32(trow + COL_O, va);
         tmem_ld_32x32(trow + COL_O + 32, vb);
@@ -450,8 +461,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     for (int t = 0; t < n_total + 2 && ok; ++t) {
       if (t < n_total) {
         const int st = t % RING, qb = ki & 1;
-        if (kj == 0 && ki >= 2) ok = mbar_wait_warp(&q_empty[qb], static_cast<uint32_t>((ki - 2) >> 1) & 1u, abort_flag, p.status);
-        if (ok && t >= RING) ok = mbar_wait_warp(&k_empty[st], static_cast<uint32_t>(t / RING - 1) & 1u, abort_flag, p.status);
+        if (kj == 0 && ki >= 2) ok = mbar_poll_warp(&q_empty[qb], static_cast<uint32_t>((ki - 2) >> 1) & 1u, abort_flag, p.status);
+        if (ok && t >= RING) ok = mbar_poll_warp(&k_empty[st], static_cast<uint32_t>(t / RING - 1) & 1u, abort_flag, p.status);
         if (!ok) break;
         if (elect_one()) {
           mbar_expect_tx(&k_full[st], kj == 0 ? 2 * C::OP_BYTES : C::OP_BYTES);
@@ -471,7 +482,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       if (t >= 2) {
         const int n = t - 2, st = n % RING;
-        if (n >= RING) ok = mbar_wait_warp(&v_empty[st], static_cast<uint32_t>(n / RING - 1) & 1u, abort_flag, p.status);
+        if (n >= RING) ok = mbar_poll_warp(&v_empty[st], static_cast<uint32_t>(n / RING - 1) & 1u, abort_flag, p.status);
         if (!ok) break;
         if (elect_one()) {
           mbar_expect_tx(&v_full[st], C::OP_BYTES);
@@ -502,10 +513,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     for (int n = 0; n < n_total; ++n) {
       const int b = n % RING, qb = i & 1;
       const uint32_t use = static_cast<uint32_t>(n / RING) & 1u;
-      if (!mbar_wait_warp(&k_full[b], use, abort_flag, p.status)) break;
+      if (!mbar_poll_warp(&k_full[b], use, abort_flag, p.status)) break;
       // The buffer held the probabilities of block n - RING: that product has to be complete (the order in which the tensor core
       // executes two products with different accumulators is not defined).
-      if (n >= RING && !mbar_wait_warp(&pv_done[b], use ^ 1u, abort_flag, p.status)) break;
+      if (n >= RING && !mbar_poll_warp(&pv_done[b], use ^ 1u, abort_flag, p.status)) break;
       tc_fence_after();
       const bool last = j + 1 == p.n_blk;
       if (elect_one()) {
@@ -537,10 +548,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     for (int n = 0; n < n_total; ++n) {
       const int b = n % RING;
       const uint32_t use = static_cast<uint32_t>(n / RING) & 1u;
-      if (!mbar_wait_warp(&v_full[b], use, abort_flag, p.status)) break;
+      if (!mbar_poll_warp(&v_full[b], use, abort_flag, p.status)) break;
       // the accumulator is overwritten: the output warps must have read the previous item's
-      if (j == 0 && i > 0 && !mbar_wait_warp(o_empty, static_cast<uint32_t>(i - 1) & 1u, abort_flag, p.status)) break;
-      if (!mbar_wait_warp(&p_full[b], use, abort_flag, p.status)) break;
+      if (j == 0 && i > 0 && !mbar_poll_warp(o_empty, static_cast<uint32_t>(i - 1) & 1u, abort_flag, p.status)) break;
+      if (!mbar_poll_warp(&p_full[b], use, abort_flag, p.status)) break;
       tc_fence_after();
       const bool last = j + 1 == p.n_blk, half = ragged && j == 0;
       if (elect_one()) {

@@ -101,6 +101,29 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
 }
 
+// The same for a wait that other warps' work hangs on: it looks again and again.  try_wait may suspend the thread, and beside warps that
+// keep the special-function unit busy the return from it took 300-500 clocks, a look that succeeds 180-250.  (For long waits
+// that nobody else waits behind, try_wait is the better one: the looks take slots of the queue that everything else goes through.)
+constexpr uint32_t kPollLimit = 1u << 27;
+__device__ __forceinline__ bool mbar_poll_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  bool ok = true;
+  for (uint32_t i = 1; !mbar_test_wait(bar, parity); ++i) {
+    if ((i & 1023u) == 0u && (i >= kPollLimit || *abort_flag)) {
+      ok = false;
+      break;
+    }
+  }
+  ok = __all_sync(0xffffffffu, ok);
+  if (!ok && *abort_flag == 0) {
+    *abort_flag = 1;
+    atomicExch(status, 1);
+  }
+  return ok;
+}
+__device__ __forceinline__ bool mbar_poll_seen(bool seen, uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  return __all_sync(0xffffffffu, seen) || mbar_poll_warp(bar, parity, abort_flag, status);
+}
+
 // The same behind an earlier mbar_test_wait of the same phase.  A look at a barrier takes about 200 clocks in these
 // kernels; a role that looks at its next barrier before it issues the work of the current one does not wait for that.
 __device__ __forceinline__ bool mbar_wait_seen(bool seen, uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
