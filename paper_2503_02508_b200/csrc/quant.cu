@@ -50,9 +50,41 @@ __global__ void __launch_bounds__(256) act_quant_kernel(const T* __restrict__ x,
   }
 }
 
-// Per-token dynamic quantizer: one warp per row finds max|x| of its row, s[m] = max / 127 (1 for a zero row),
-// and writes the symmetric codes; the row is read twice (the second time from L1 / L2).
+// 8 consecutive values as they lie in memory.
 template <typename T>
+struct Raw8;
+template <>
+struct Raw8<__nv_bfloat16> {
+  uint4 w;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { w = *reinterpret_cast<const uint4*>(p); }
+  __device__ __forceinline__ void clear() { w = make_uint4(0u, 0u, 0u, 0u); }
+  __device__ __forceinline__ void widen(float (&v)[8]) const {
+    unpack_bf16x2(w.x, v[0], v[1]);
+    unpack_bf16x2(w.y, v[2], v[3]);
+    unpack_bf16x2(w.z, v[4], v[5]);
+    unpack_bf16x2(w.w, v[6], v[7]);
+  }
+};
+template <>
+struct Raw8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p) {
+    a = *reinterpret_cast<const float4*>(p);
+    b = *reinterpret_cast<const float4*>(p + 4);
+  }
+  __device__ __forceinline__ void clear() { a = b = make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
+  __device__ __forceinline__ void widen(float (&v)[8]) const {
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  }
+};
+
+// Per-token dynamic quantizer: one warp per row finds max|x| of its row, s[m] = max / 127 (1 for a zero row),
+// and writes the symmetric codes.
+//
+// Bound by memory, if enough of it is in flight: with NV > 0 a lane loads its NV pieces of 8 values at once and keeps them for
+// the codes (K <= 256 * NV).  NV = 0: any K, the row is read twice, the second time from L1 / L2.
+template <typename T, int NV>
 __global__ void __launch_bounds__(256) act_quant_token_kernel(const T* __restrict__ x, int64_t M, int64_t K, int64_t ldx,
                                                               float* __restrict__ scales, uint8_t* __restrict__ q,
                                                               int64_t ldq) {
@@ -62,12 +94,28 @@ __global__ void __launch_bounds__(256) act_quant_token_kernel(const T* __restric
   const int64_t row = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= M) return;
   const T* src = x + row * ldx;
+  Raw8<T> raw[NV > 0 ? NV : 1];
   float m = 0.0f;
-  for (int64_t k = lane * 8; k < K; k += 256) {
+  auto widest = [&](const Raw8<T>& r) {
     float v[8];
-    Load8<T>::load(src + k, v);
+    r.widen(v);
 #pragma unroll
     for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
+  };
+  if constexpr (NV > 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int k = lane * 8 + i * 256;
+      if (k < K) raw[i].load(src + k);
+      else raw[i].clear();
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i) widest(raw[i]);
+  } else {
+    for (int64_t k = lane * 8; k < K; k += 256) {
+      raw[0].load(src + k);
+      widest(raw[0]);
+    }
   }
   m = warp_max(m);
   float s = __fdiv_rn(m, 127.0f);
@@ -75,10 +123,20 @@ __global__ void __launch_bounds__(256) act_quant_token_kernel(const T* __restric
   const float inv = __fdiv_rn(1.0f, s);
   if (lane == 0) scales[row] = s;
   uint8_t* dst = q + row * ldq;
-  for (int64_t k = lane * 8; k < K; k += 256) {
-    float v[8];
-    Load8<T>::load(src + k, v);
-    *reinterpret_cast<uint2*>(dst + k) = quantize_pack8(v, inv, 0.0f, -127.0f, 127.0f);
+  float v[8];
+  if constexpr (NV > 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int k = lane * 8 + i * 256;
+      raw[i].widen(v);
+      if (k < K) *reinterpret_cast<uint2*>(dst + k) = quantize_pack8(v, inv, 0.0f, -127.0f, 127.0f);
+    }
+  } else {
+    for (int64_t k = lane * 8; k < K; k += 256) {
+      raw[0].load(src + k);
+      raw[0].widen(v);
+      *reinterpret_cast<uint2*>(dst + k) = quantize_pack8(v, inv, 0.0f, -127.0f, 127.0f);
+    }
   }
 }
 
@@ -579,6 +637,18 @@ int32_t quant_dynamic(qdit_ctx* ctx, const T* x, int64_t M, int64_t K, int64_t l
                                               q, ldq));
   return qdit_after_launch(ctx, "act_quant_kernel");
 }
+
+// The rows stay in registers where enough warps fit beside them: 2 or 5 pieces per lane (us, row read twice / kept, bf16: 65536 x 384
+// 24.8 / 16.2, 5000 x 1152 5.0 / 4.3, 65536 x 1152 45.5 / 38.7; f32 62.8 / 54.8), and 18 of bf16 for few long rows, where only the latency
+// counts (64 x 4608 4.8 / 3.5; 5000 x 4608 12.1 / 14.8, and 5000 x 1536 5.5 / 9.8 with two thirds of the pieces missing).
+template <typename T>
+int32_t quant_token(qdit_ctx* ctx, const T* x, int64_t M, int64_t K, int64_t ldx, float* scales, uint8_t* q, int64_t ldq) {
+  constexpr bool NARROW = sizeof(T) == 2;
+  const auto kernel = K <= 512 ? act_quant_token_kernel<T, 2> : K <= 1280 ? act_quant_token_kernel<T, 5> : NARROW && K > 2304 && K <= 4608 && M <= 512 ? act_quant_token_kernel<T, NARROW ? 18 : 0>
+                                                                                                        : act_quant_token_kernel<T, 0>;
+  QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_TOKEN_CTAS, kernel, dim3(static_cast<unsigned>((M + 7) / 8)), dim3(256), 0, x, M, K, ldx, scales, q, ldq));
+  return qdit_after_launch(ctx, "act_quant_token_kernel");
+}
 }  // namespace
 
 int32_t launch_quant_dynamic(qdit_ctx* ctx, const void* x, int x_dtype, int64_t M, int64_t K, int64_t ldx, float* scale,
@@ -632,14 +702,8 @@ int32_t qdit_quantize_act(qdit_ctx* ctx, const void* x, int x_dtype, int64_t M, 
     qa = make_quant_args(*qp, nullptr);
   } else if (mode == QDIT_QUANT_DYNAMIC_TOKEN) {
     if (!dyn_scale) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "per-token mode needs dyn_scale [M]");
-    const unsigned grid = static_cast<unsigned>((M + 7) / 8);
-    if (x_dtype == QDIT_BF16)
-      QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_TOKEN_CTAS, act_quant_token_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, static_cast<const __nv_bfloat16*>(x), M, K, ldx, dyn_scale,
-                                                                        static_cast<uint8_t*>(q), ldq));
-    else
-      QDIT_CUDA_CHECK(ctx, launch_act_quant(ctx, EARLY_TOKEN_CTAS, act_quant_token_kernel<float>, dim3(grid), dim3(256), 0, static_cast<const float*>(x), M, K, ldx, dyn_scale,
-                                                                   static_cast<uint8_t*>(q), ldq));
-    return qdit_after_launch(ctx, "act_quant_token_kernel");
+    if (x_dtype == QDIT_BF16) return quant_token(ctx, static_cast<const __nv_bfloat16*>(x), M, K, ldx, dyn_scale, static_cast<uint8_t*>(q), ldq);
+    return quant_token(ctx, static_cast<const float*>(x), M, K, ldx, dyn_scale, static_cast<uint8_t*>(q), ldq);
   } else if (mode == QDIT_QUANT_DYNAMIC) {
     if (!dyn_scale) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "dynamic mode needs dyn_scale");
     return launch_quant_dynamic(ctx, x, x_dtype, M, K, ldx, dyn_scale, nullptr, q, ldq);

@@ -135,6 +135,25 @@ def test_quantize_act_per_token_bit_exact(q, ctx, M, K, dtype):
     assert q.lib.qdit_quantize_act(ctx, xd.data_ptr(), code, M, K, K, q.QDIT_QUANT_DYNAMIC_TOKEN, None, None, out.data_ptr(), K) == q.QDIT_ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("K", [8, 512, 520, 1280, 1288, 4608, 4616])   # up to 2, 5 and 18 pieces of 256 per lane in registers, and beyond
+def test_quantize_act_per_token_row_lengths(q, ctx, K, dtype):
+    """Rows that fill the registers of a warp, end inside a piece or do not fit, in wider matrices: bit-exact, nothing written beside them."""
+    M, ldx, ldq = 11, K + 24, K + 16
+    x = synth.outlier_activations(13, f"tokrow{K}", M, ldx)
+    x[:, K:] = 1e4   # not part of the rows
+    x[4, :K] = 0
+    xd = dev(x).to(torch.bfloat16) if dtype == "bf16" else dev(x)
+    out = torch.full((M, ldq), 99, dtype=torch.uint8, device="cuda")
+    sc = torch.empty(M, dtype=torch.float32, device="cuda")
+    q.qdit_quantize_act(ctx, xd, q.QDIT_BF16 if dtype == "bf16" else q.QDIT_F32, M, K, ldx, q.QDIT_QUANT_DYNAMIC_TOKEN, None, sc, out, ldq)
+    q.qdit_sync(ctx)
+    want_q, want_s = quant.quantize_per_token(xd.float().cpu().numpy()[:, :K])
+    np.testing.assert_array_equal(sc.cpu().numpy(), want_s)
+    np.testing.assert_array_equal(host_codes(out[:, :K]), want_q)
+    assert (out[:, K:] == 99).all()
+
+
 @pytest.mark.parametrize("bits", [4, 6, 2])
 def test_quantize_weight_bits_bit_exact(q, ctx, bits):
     """b-bit channel-wise weights (bits = 4: the W4A8 setting of Table 2): codes, scales and code sums."""
