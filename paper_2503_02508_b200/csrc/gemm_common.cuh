@@ -297,5 +297,9 @@ double qdit_gemm_pair_cost(const qdit_ctx* ctx, const qgemm::GemmParams& p);   /
 int qdit_gemm_sk_clusters(qdit_ctx* ctx, int split);
 int32_t qdit_launch_gemm_sk(qdit_ctx* ctx, const void* A, const void* W, qgemm::GemmParams& p, bool a_unsigned, int split, bool packed4);
 
+// One to FEW_ROWS rows, f32 output with a bias (gemm_rows.cu), R * K bytes of shared memory for R = 1, 2 or 4 rows.
+constexpr int FEW_ROWS = 4;
+int32_t qdit_launch_few_rows(qdit_ctx* ctx, const void* A, const void* W, const qgemm::GemmParams& p, bool a_unsigned, bool packed4);
+
 // Packed 4-bit weights widened inside the kernel (gemm_w4.cu): token-major tiles of 128 x 128.
 int32_t qdit_launch_gemm_w4(qdit_ctx* ctx, const void* A, const void* W_packed, qgemm::GemmParams& p, bool a_unsigned);

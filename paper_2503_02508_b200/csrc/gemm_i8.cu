@@ -272,6 +272,8 @@ int pick_split(qdit_ctx* ctx, int M, int N, int K, int spare) {
   return 1;
 }
 
+constexpr int FEW_ROWS_K = 8192;   // 32 KB of activations for four rows
+
 }  // namespace
 
 // Both linear layers: `packed4` = W holds 4-bit codes two per byte ([N, K/2]); `w8_scratch` = optional [N, K] int8
@@ -364,6 +366,13 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
       p.o_qmax = static_cast<float>(epi->out_qp.qmax);
     }
   }
+  // One to four rows, f32 output (the modulation of as many images): the weights are streamed past the rows instead of through the
+  // tensor core (us, 1 and 4 rows, tensor core / streamed: 193536 x 1152 51.2 / 35.1 and 51.4 / 45.4, packed 4-bit weights 73.0 / 22.1 and
+  // 75.9 / 47.7; 6912 x 1152 7.0 / 2.8 and 7.0 / 4.2; 1152 x 4608 7.1 / 4.1 and 7.2 / 5.7; 1152 x 384 3.4 / 2.2 and 3.3 / 2.6).  Beyond
+  // four the dot products take longer than the weights.
+  if (epi_class(p.flags) == 6 && p.M <= FEW_ROWS && !p.absmax && p.K <= FEW_ROWS_K && ctx->opt[QDIT_OPT_GEMM_BN] == 0 && ctx->opt[QDIT_OPT_GEMM_T] == 0 &&
+      !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE])
+    return qdit_launch_few_rows(ctx, A, W, p, a_unsigned, packed4);
   if (packed4) {
     // many rows: the layer is bound by the tensor core and its epilogue, so the weights are widened once into the
     // scratch matrix and the W8A8 kernels run on it; few rows (or no scratch): the weight bytes bound the layer and

@@ -617,3 +617,39 @@ def test_pair_kernel_gives_the_bits_of_the_token_major_kernel(q, ctx, M, N, K, T
         q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, 0)
     assert torch.equal(got[0], ref[0])
     assert torch.equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("M,N,K,zp", [(1, 8, 32, 0), (2, 40, 1152, 7), (3, 4608, 1152, 0), (4, 1160, 1184, 0), (1, 19208, 1152, 11), (4, 24, 8192, 3),
+                                      (4, 24, 8224, 0), (5, 1152, 384, 0)])   # (the last two are served by the tensor-core kernels)
+def test_few_rows_kernel_gives_the_bits_of_the_tensor_core_kernels(q, ctx, bits, M, N, K, zp):
+    """One to four rows with f32 output: exact integer sums and the same f32 epilogue; the padding of the rows stays untouched."""
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    lo, hi = (0, 256) if zp else (-127, 128)
+    A = torch.randint(lo, hi, (M, K), generator=g, device="cuda").to(torch.uint8 if zp else torch.int8)
+    top = 127 if bits == 8 else 7
+    W = torch.randint(-top - 1, top + 1, (N, K), generator=g, device="cuda", dtype=torch.int8)
+    ws, bi = torch.rand(N, generator=g, device="cuda") * 2e-4 + 1e-5, torch.randn(N, generator=g, device="cuda") * 0.5
+    colsum = W.sum(dim=1, dtype=torch.int32)
+    epi = q.epilogue(w_scale=ws, w_colsum=colsum, bias=bi)
+    qp = q.qparams(0.03, zp, 0, 255) if zp else q.qparams(0.03)
+    packed = None
+    if bits == 4:
+        packed = torch.empty((N, K // 2), dtype=torch.uint8, device="cuda")
+        q.qdit_pack_weight_int4(ctx, W, N, K, packed)
+
+    def run(option):
+        out = torch.full((M, N + 8), 3.0, device="cuda")
+        torch.cuda.synchronize()
+        try:
+            q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, option)
+            if bits == 4:
+                q.qdit_w4a8_linear(ctx, A, packed, M, N, K, qp, None, q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_F32, epi, out, N + 8, None)
+            else:
+                q.qdit_w8a8_linear(ctx, A, W, M, N, K, qp, None, q.QDIT_EPI_BIAS | q.QDIT_EPI_OUT_F32, epi, out, N + 8)
+            q.qdit_sync(ctx)
+        finally:
+            q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 0)
+        return out
+
+    assert torch.equal(run(0), run(64))
