@@ -653,3 +653,29 @@ def test_few_rows_kernel_gives_the_bits_of_the_tensor_core_kernels(q, ctx, bits,
         return out
 
     assert torch.equal(run(0), run(64))
+
+
+@pytest.mark.parametrize("step", [4e-39, 2.0 ** -125, 1e-30, 0.01])
+def test_codes_of_tiny_steps(q, ctx, step):
+    """GELU codes by pairs of CTAs equal those of the run-time-flag epilogue down to steps at which subnormal activations count."""
+    M, N, K = 1200, 4608, 64
+    A, W = dev_i8(_codes(101, "a", (M, K), -127, 127)), dev_i8(_codes(101, "w", (N, K), -127, 127))
+    # products of +-50000 or so: the activations are some ten steps
+    ws = torch.full((N,), step / 4096.0 * 1e10, dtype=torch.float32, device="cuda")
+    bi = torch.zeros(N, dtype=torch.float32, device="cuda")
+    scale = torch.tensor([step], dtype=torch.float32, device="cuda")
+    got = []
+    for generic in (0, 1):
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, generic)
+        try:
+            for dev_scale in (None, scale):
+                out = torch.zeros((M, N), dtype=torch.int8, device="cuda")
+                q.qdit_w8a8_linear(ctx, A, W, M, N, K, q.qparams(1e-10), None, q.QDIT_EPI_BIAS | q.QDIT_EPI_GELU | q.QDIT_EPI_QUANT_OUT,
+                                   q.epilogue(w_scale=ws, bias=bi, out_qp=q.qparams(step), out_scale_dev=dev_scale), out, N)
+                q.qdit_sync(ctx)
+                got.append(out)
+        finally:
+            q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, 0)
+    assert (got[2].int().abs() > 0).float().mean() > 0.1
+    for g in (got[0], got[1], got[3]):
+        assert torch.equal(g, got[2])
