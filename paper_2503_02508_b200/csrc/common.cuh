@@ -130,6 +130,13 @@ __device__ __forceinline__ bool mbar_wait_seen(bool seen, uint64_t* bar, uint32_
   return __all_sync(0xffffffffu, seen) || mbar_wait_warp(bar, parity, abort_flag, status);
 }
 
+// For a role whose wait for a copy ran out, or that left through the abort flag: the copies still in flight get 2 ms (a copy takes
+// microseconds) to land before the CTA's shared memory is released.  Their barriers are of no use here: a wait returns at once when the
+// flag is up.
+__device__ __forceinline__ void leave_time_for_copies() {
+  for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+}
+
 // ----------------------------------------------------------------------------- TMA (every copy serves the issuing CTA alone)
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");

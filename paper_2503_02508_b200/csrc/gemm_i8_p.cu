@@ -263,9 +263,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
       }
-      if (!ok) {
-        for (int i = 0; i < 2000; ++i) __nanosleep(1000);  // let copies in flight land before shared memory goes away
-      }
+      if (!ok) leave_time_for_copies();
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -296,6 +294,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         }
         if (ok) pair_commit(&tfull_bar[as]);
       }
+      if (!ok) leave_time_for_copies();   // (the producers may have issued their last copy before)
     }
     __syncwarp();
   } else {
@@ -581,8 +580,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         }
       }
       if (EPI == 7 && p.absmax) publish_absmax(p.absmax, top);
-      // (after a time-out) a residual still in flight must land before the CTA's shared memory is released
-      if (asked) mbar_wait(&rbar[turn], r_phase >> turn & 1u, abort_flag, p.status);
+      if (C::GATED && !ok) leave_time_for_copies();   // residuals of this chunk and of the next one
     }
     if (elect_one()) tma_store_wait_all();
     __syncwarp();

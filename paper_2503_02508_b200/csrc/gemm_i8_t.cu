@@ -279,9 +279,7 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
-      if (!ok) {
-        for (int i = 0; i < 2000; ++i) __nanosleep(1000);  // let copies in flight land before shared memory goes away
-      }
+      if (!ok) leave_time_for_copies();
     }
   } else if (warp == 1) {
     if (elect_one()) {
@@ -313,6 +311,7 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         }
         if (ok) umma_commit(&tfull_bar[as]);
       }
+      if (!ok) leave_time_for_copies();   // (the producer may have issued its last copy before)
     }
   } else {
     // -------------------------------------------------------------------- epilogue warps
@@ -499,8 +498,7 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
           }
         }
       }
-      // a residual tile still in flight must land before the CTA's shared memory is released
-      if (r_inflight) mbar_wait(rbar, r_phase, abort_flag, p.status);
+      if (TW::GATED && !ok) leave_time_for_copies();   // the residual
       if (lane == 0) tma_store_wait_all();
     } else {
       float top = 0.0f;
@@ -543,8 +541,8 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
           const int m_base = t0 + c * 32;
           if (m_base < p.M && n_ok) epilogue_chunk_t<EPI>(p, v, n, m_base, sc, bias, zcs, o_inv, top);
         }
-      __syncwarp();
-      if (p.absmax) publish_absmax(p.absmax, top);
+        __syncwarp();
+        if (p.absmax) publish_absmax(p.absmax, top);
       }
     }
   }
