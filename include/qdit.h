@@ -53,9 +53,10 @@ int32_t qdit_destroy(qdit_ctx* ctx);
 int32_t qdit_sync(qdit_ctx* ctx);
 /* Self-test of the device-side time-out path (the paper has no counterpart): launches one small kernel in which
  * a bounded wait of `polls` polls (1..2^20) on a barrier that nobody signals runs out, and a second waiting
- * thread leaves through the CTA's abort flag, exactly as the roles of the pipelined kernels do.  The kernel ends
- * normally; the next qdit_sync returns QDIT_ERR_TIMEOUT once and the context stays usable.
- * observed_dev: device int[2], set to {1, 1} when both threads left their wait the intended way. */
+ * thread leaves through the CTA's abort flag, exactly as the roles of the pipelined kernels do; the same with the
+ * polling form of the wait, by whole warps.  The kernel ends normally; the next qdit_sync returns QDIT_ERR_TIMEOUT
+ * once and the context stays usable.
+ * observed_dev: device int[2], set to {1, 1} when all waits were left the intended way. */
 int32_t qdit_selftest_wait_timeout(qdit_ctx* ctx, uint32_t polls, int* observed_dev);
 /* Tensor-pipe probe (the paper has no counterpart; bench.py --workload mma_probe reports it): every SM runs
  * `iters` groups of four tcgen05.mma kind::i8 instructions (M 128, N = n in {64, 128, 192, 256}, K 32 each), the

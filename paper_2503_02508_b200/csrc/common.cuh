@@ -104,11 +104,12 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
 // The same for a wait that other warps' work hangs on: it looks again and again.  try_wait may suspend the thread, and beside warps that
 // keep the special-function unit busy the return from it took 300-500 clocks, a look that succeeds 180-250.  (For long waits
 // that nobody else waits behind, try_wait is the better one: the looks take slots of the queue that everything else goes through.)
+// Bounded in the same way: at most `limit` looks, in steps of 1024.
 constexpr uint32_t kPollLimit = 1u << 27;
-__device__ __forceinline__ bool mbar_poll_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+__device__ __forceinline__ bool mbar_poll_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, uint32_t limit = kPollLimit) {
   bool ok = true;
   for (uint32_t i = 1; !mbar_test_wait(bar, parity); ++i) {
-    if ((i & 1023u) == 0u && (i >= kPollLimit || *abort_flag)) {
+    if ((i & 1023u) == 0u && (i >= limit || *abort_flag)) {
       ok = false;
       break;
     }

@@ -63,27 +63,33 @@ ProfScope::~ProfScope() {
   if (on) cudaEventRecord(stop, ctx->stream);
 }
 
-// Self-test of the bounded wait that every pipelined kernel uses: warp 1 waits (with a small poll limit) on a
-// barrier that nobody arrives at, so the wait runs out, raises the CTA's abort flag and the device status word;
-// warp 0 waits on a second such barrier with the full limit and leaves as soon as it sees the abort flag.  The
-// kernel then exits normally: the context stays usable and the next qdit_sync reports the time-out.
+// Self-test of the two bounded waits of the pipelined kernels, mbar_wait (warps 0 and 1) and mbar_poll_warp (warps 2 and 3, every lane).
+// Of each pair the odd warp waits, with a small limit, on a barrier that nobody arrives at, so that the wait runs out and raises the
+// pair's abort flag and the device status word; the even one waits on a second such barrier with the full limit and leaves as soon as it
+// sees the flag.  The kernel then exits normally: the context stays usable and the next qdit_sync reports the time-out.
 __global__ void wait_timeout_selftest_kernel(uint32_t polls, int* status, int* observed) {
-  __shared__ uint64_t bars[2];
-  __shared__ int abort_flag;
+  __shared__ uint64_t bars[4];
+  __shared__ int abort_flag[2];
+  __shared__ int left[4];   // per warp: it left its wait without the barrier
+  const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
-    qd::mbar_init(&bars[0], 1);
-    qd::mbar_init(&bars[1], 1);
-    abort_flag = 0;
+    for (int i = 0; i < 4; ++i) qd::mbar_init(&bars[i], 1);
+    abort_flag[0] = abort_flag[1] = 0;
     qd::mbar_fence_init();
   }
+  if (threadIdx.x < 4) left[threadIdx.x] = 0;
   __syncthreads();
-  volatile int* af = &abort_flag;
-  if (threadIdx.x == 32) {
-    const bool ok = qd::mbar_wait_limited(&bars[0], 0, af, status, polls);
-    observed[0] = ok ? 0 : 1;  // 1: the limited wait ran out
-  } else if (threadIdx.x == 0) {
-    const bool ok = qd::mbar_wait(&bars[1], 0, af, status);
-    observed[1] = ok ? 0 : 1;  // 1: left through the abort flag
+  volatile int* af = &abort_flag[warp >> 1];
+  if (warp >= 2) {
+    const bool ok = qd::mbar_poll_warp(&bars[warp], 0, af, status, (warp & 1) ? polls : qd::kPollLimit);
+    atomicAdd(&left[warp], ok ? 0 : 1);
+  } else if ((threadIdx.x & 31) == 0) {
+    left[warp] = qd::mbar_wait_limited(&bars[warp], 0, af, status, (warp & 1) ? polls : qd::kSpinLimit) ? 0 : 1;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    observed[0] = left[1] == 1 && left[3] == 32;   // the limited waits ran out
+    observed[1] = left[0] == 1 && left[2] == 32;   // the others left through the abort flag
   }
 }
 
@@ -93,7 +99,7 @@ int32_t qdit_selftest_wait_timeout(qdit_ctx* ctx, uint32_t polls, int* observed_
   if (!ctx) return QDIT_ERR_INVALID_ARG;
   if (!observed_dev) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "observed_dev is NULL");
   if (polls == 0 || polls > (1u << 20)) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "polls must be in 1..2^20");
-  wait_timeout_selftest_kernel<<<1, 64, 0, ctx->stream>>>(polls, ctx->d_status, observed_dev);
+  wait_timeout_selftest_kernel<<<1, 128, 0, ctx->stream>>>(polls, ctx->d_status, observed_dev);
   return qdit_after_launch(ctx, "wait_timeout_selftest_kernel");
 }
 
