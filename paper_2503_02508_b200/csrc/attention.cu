@@ -243,7 +243,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   const int g = lane >> 2, t = lane & 3;
   const int64_t ldo = static_cast<int64_t>(p.H) * DH;
   float q_inv = 0.0f;
-  if (p.out_dtype == QDIT_I8) q_inv = __fdiv_rn(1.0f, p.qa.scale_dev ? __ldg(p.qa.scale_dev) : p.qa.scale);
+  if (p.out_dtype == QDIT_I8) q_inv = __fdiv_rn(1.0f, device_value(p.qa.scale_dev, p.qa.scale));
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int64_t row = static_cast<int64_t>(row0) + q0 + warp * 16 + g + r * 8;

@@ -337,7 +337,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     float q_inv = 0.0f;
     grid_dependency_wait();
     grid_dependency_release();
-    if (p.out_dtype == QDIT_I8) q_inv = __fdiv_rn(1.0f, p.qa.scale_dev ? __ldg(p.qa.scale_dev) : p.qa.scale);
+    if (p.out_dtype == QDIT_I8) q_inv = __fdiv_rn(1.0f, device_value(p.qa.scale_dev, p.qa.scale));
 #pragma unroll 1
     for (int i = 0; i < items; ++i) {
       const Item it = item_of<DH>(p, static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x));

@@ -53,6 +53,11 @@ __device__ __forceinline__ void mbar_arrive_relaxed(uint64_t* bar) {
 // a kernel launched without the attribute.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A quantizer's scale: the one in device memory, if there is one.  (Not through the read-only path: the launch in front may write it while
+// this kernel is already resident.)
+__device__ __forceinline__ float device_value(const float* dev, float value) {
+  return dev ? *dev : value;
+}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(

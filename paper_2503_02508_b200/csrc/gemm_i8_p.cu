@@ -300,7 +300,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
   } else {
     // -------------------------------------------------------------------- epilogue warps
     const int e = warp - 2, quad = warp & 3, part = e >> 2;
-    const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
+    const float a_scale = device_value(p.a_scale_dev, p.a_scale);
     const int chunks = bn / 32;
     const int c_last = part < chunks ? part + ((chunks - 1 - part) / C::SPLIT) * C::SPLIT : -1;   // this warp's last chunk
     uint8_t* const stg = staging + e * C::STAGING_PER_WARP;
@@ -314,7 +314,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     int it = 0, turn = 0;
     bool ok = true;
     if constexpr (C::CODES) {
-      const float o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
+      const float o_inv = __fdiv_rn(1.0f, device_value(p.o_scale_dev, p.o_scale));
       const float lo_f = p.o_qmin - p.o_zp, hi_f = p.o_qmax - p.o_zp;
       const uint32_t z4 = (static_cast<uint32_t>(static_cast<int>(p.o_zp)) & 0xFFu) * 0x01010101u;
       const float2 o2 = make_float2(o_inv, o_inv), magic = make_float2(12582912.0f, 12582912.0f);

@@ -131,8 +131,8 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
   };
   if (warp >= 2) {
     if (!p.early_params) grid_dependency_wait();
-    a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
-    if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
+    a_scale = device_value(p.a_scale_dev, p.a_scale);
+    if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, device_value(p.o_scale_dev, p.o_scale));
     // (warps that widen weights first do not wait for the parameters in front of that)
     if ((!W4 || p.early_params) && warp - 2 < units) prefetch_columns(warp - 2);
     if (p.early_params) grid_dependency_wait();

@@ -320,9 +320,9 @@ gemm_i8_t_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     constexpr int T_EPI_SPLIT = TW::SPLIT;
     const int part = e >> 2;     // this warp takes token chunks part, part + T_EPI_SPLIT, ...
     const uint32_t flags = epi_flags<EPI>(p);
-    const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
+    const float a_scale = device_value(p.a_scale_dev, p.a_scale);
     float o_inv = 0.0f;
-    if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
+    if (flags & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, device_value(p.o_scale_dev, p.o_scale));
     constexpr int CHUNKS = BT / 32;
     const int c_last = part < CHUNKS ? part + ((CHUNKS - 1 - part) / T_EPI_SPLIT) * T_EPI_SPLIT : -1;
     // the staged form of the gated epilogue needs a chunk to lie inside one sample (one gate row per chunk)

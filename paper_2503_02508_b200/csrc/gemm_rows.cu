@@ -28,7 +28,7 @@ __device__ __forceinline__ int dot4(uint32_t w, uint32_t x, int acc) {   // sign
 }
 
 template <int R, bool W4, bool U>
-__global__ void __launch_bounds__(ROWS_THREADS, R == 4 ? 3 : 4) few_rows_kernel(const uint8_t* __restrict__ A, const uint8_t* __restrict__ W, const GemmParams p) {
+__global__ void __launch_bounds__(ROWS_THREADS, R == 4 ? 3 : 4) few_rows_kernel(const uint8_t* A, const uint8_t* __restrict__ W, const GemmParams p) {
   constexpr int UN = W4 ? 5 : 9;             // pieces of a lane in flight: 1152 codes are 72 pieces of 16 bytes, packed 36
   constexpr int XV = W4 ? 2 : 1;             // 16-byte pieces of activations per piece of weights
   extern __shared__ uint4 xs[];              // [R][XV][pieces]
@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, R == 4 ? 3 : 4) few_rows_kernel(
       xs[r * pieces + c] = a;
     }
   }
-  const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
+  const float a_scale = device_value(p.a_scale_dev, p.a_scale);
   __syncthreads();
   for (int nb = first; nb < p.N; nb += static_cast<int>(gridDim.x) * (ROWS_THREADS / 32) * 4) {
     const int n = nb + (lane >> 3);

@@ -197,9 +197,9 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const uint32_t stg = smem_u32(staging + e * (32 * 128));
     grid_dependency_wait();
     grid_dependency_release();
-    const float a_scale = p.a_scale_dev ? __ldg(p.a_scale_dev) : p.a_scale;
+    const float a_scale = device_value(p.a_scale_dev, p.a_scale);
     float o_inv = 0.0f;
-    if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, p.o_scale_dev ? __ldg(p.o_scale_dev) : p.o_scale);
+    if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, device_value(p.o_scale_dev, p.o_scale));
     float top = 0.0f;
     int it = 0;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {

@@ -15,8 +15,8 @@ using namespace qd;
 // ----------------------------------------------------------------------------- block-output cache
 // x[m, 8 cols] = bf16(x + gate[b] * slot)
 __global__ void __launch_bounds__(256) cache_reuse_kernel(__nv_bfloat16* __restrict__ x,
-                                                          const __nv_bfloat16* __restrict__ slot,
-                                                          const float* __restrict__ gate, int64_t ld_gate, int64_t M,
+                                                          const __nv_bfloat16* slot,
+                                                          const float* gate, int64_t ld_gate, int64_t M,
                                                           int D, int64_t T) {
   grid_dependency_wait();
   grid_dependency_release();
@@ -40,8 +40,8 @@ __global__ void __launch_bounds__(256) cache_reuse_kernel(__nv_bfloat16* __restr
 // L2 as the cache itself is from HBM) and 2 R independent 16-byte cache loads are in flight per block.
 template <int R>
 __global__ void __launch_bounds__(256, 2) cache_reuse_all_kernel(__nv_bfloat16* __restrict__ x,
-                                                                 const __nv_bfloat16* __restrict__ cache,
-                                                                 const float* __restrict__ mod, int64_t ld_mod, int64_t M,
+                                                                 const __nv_bfloat16* cache,
+                                                                 const float* mod, int64_t ld_mod, int64_t M,
                                                                  int D, int64_t T, int blocks) {
   grid_dependency_wait();
   grid_dependency_release();
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(256) tap_scale_kernel(float* __restrict__ A, c
 
 // ----------------------------------------------------------------------------- guidance + DDIM update
 // net: [Beff, 2C, HW]; eps = first C channels; with guidance, sample b's unconditional twin is b + B.
-__global__ void __launch_bounds__(256) cfg_ddim_kernel(float* __restrict__ latent, const float* __restrict__ net, int B,
+__global__ void __launch_bounds__(256) cfg_ddim_kernel(float* __restrict__ latent, const float* net, int B,
                                                        int C, int HW, int use_cfg, float guidance, DdimCoef k) {
   grid_dependency_wait();
   grid_dependency_release();
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(256) cfg_ddim_kernel(float* __restrict__ laten
 
 // Stochastic (ancestral) step with learned variance: the network's second output group v in [-1, 1] interpolates
 // the log variance between beta' and the posterior variance; v comes from the conditional half under guidance.
-__global__ void __launch_bounds__(256) cfg_ddpm_kernel(float* __restrict__ latent, const float* __restrict__ net,
+__global__ void __launch_bounds__(256) cfg_ddpm_kernel(float* __restrict__ latent, const float* net,
                                                        const float* __restrict__ noise, int B, int C, int HW, int use_cfg,
                                                        float guidance, DdpmCoef k) {
   grid_dependency_wait();
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256) cfg_ddpm_kernel(float* __restrict__ laten
 // a warp are 128 contiguous bytes.
 constexpr int EMB_ROWS = 32;
 template <int PD>
-__global__ void __launch_bounds__(256) embed_kernel(const float* __restrict__ latent, int latent_batch,
+__global__ void __launch_bounds__(256) embed_kernel(const float* latent, int latent_batch,
                                                     const float* __restrict__ wT, const float* __restrict__ bias,
                                                     const float* __restrict__ pos, __nv_bfloat16* __restrict__ x,
                                                     int64_t M, int D, int grid, int patch, int C) {
@@ -345,7 +345,7 @@ __global__ void timestep_features_kernel(const float* __restrict__ t, float* __r
 // into shared memory with cp.async (all copies in flight at once: the copy is one L2 latency, not one per
 // loop trip), f is applied in place, then a warp keeps its weight row in registers and walks the samples.
 constexpr int SL_MAXV = 16;  // float4 per lane: K <= 2048
-__global__ void __launch_bounds__(256) small_linear_kernel(const float* __restrict__ in, const float* __restrict__ w,
+__global__ void __launch_bounds__(256) small_linear_kernel(const float* in, const float* __restrict__ w,
                                                            const float* __restrict__ bias,
                                                            const float* __restrict__ table, const int32_t* __restrict__ y,
                                                            float* __restrict__ out, float* __restrict__ out_silu, int B,
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(256) small_linear_kernel(const float* __restri
 // x 16 k; each thread owns 8 x 4 outputs and sums over k in ascending order, so an output's value does not
 // depend on how many rows the call has or where the row sits.
 constexpr int BL_BM = 128, BL_BN = 64, BL_BK = 16;
-__global__ void __launch_bounds__(256) batched_linear_kernel(const float* __restrict__ in, const float* __restrict__ w,
+__global__ void __launch_bounds__(256) batched_linear_kernel(const float* in, const float* __restrict__ w,
                                                              const float* __restrict__ bias, const float* __restrict__ table,
                                                              const int32_t* __restrict__ y, float* __restrict__ out,
                                                              float* __restrict__ out_silu, int R, int N, int K, int silu_input,
@@ -509,8 +509,8 @@ __global__ void __launch_bounds__(256) batched_linear_kernel(const float* __rest
 // transposing butterfly (31 shuffles per row) after which lane o holds output o.
 constexpr int FIN_OUT = 32;
 template <int NV>
-__global__ void __launch_bounds__(512, 1) final_kernel(const __nv_bfloat16* __restrict__ x, int64_t M, int D, int T,
-                                                       float eps, const float* __restrict__ modf,
+__global__ void __launch_bounds__(512, 1) final_kernel(const __nv_bfloat16* x, int64_t M, int D, int T,
+                                                       float eps, const float* modf,
                                                        const float* __restrict__ w, const float* __restrict__ bias,
                                                        float* __restrict__ net, int grid, int patch) {
   extern __shared__ float4 s_w[];  // [FIN_OUT][NV][2][32] float4: (o, j, h, lane) = w[o][(lane + 32 j) * 8 + 4 h ..]
@@ -678,8 +678,8 @@ __device__ __forceinline__ void split_triple(float z0, float z1, uint32_t& hi, u
   lo2 = *reinterpret_cast<const uint32_t*>(&m);
 }
 
-__global__ void __launch_bounds__(FT_THREADS) final_tc_kernel(const __nv_bfloat16* __restrict__ x, int64_t M, int D, int T, float eps,
-                                                              const float* __restrict__ modf, const float* __restrict__ w,
+__global__ void __launch_bounds__(FT_THREADS) final_tc_kernel(const __nv_bfloat16* x, int64_t M, int D, int T, float eps,
+                                                              const float* modf, const float* __restrict__ w,
                                                               const float* __restrict__ bias, float* __restrict__ net, int grid, int patch,
                                                               int* status) {
   extern __shared__ __align__(16) uint8_t ft_smem[];
@@ -869,7 +869,7 @@ __global__ void embed_fragments_kernel(const float* __restrict__ wT, int D, uint
   frag[i] = f;
 }
 
-__global__ void __launch_bounds__(ET_THREADS, 2) embed_tc_kernel(const float* __restrict__ latent, int latent_batch,
+__global__ void __launch_bounds__(ET_THREADS, 2) embed_tc_kernel(const float* latent, int latent_batch,
                                                                  const uint4* __restrict__ frag, const float* __restrict__ bias,
                                                                  const float* __restrict__ pos, __nv_bfloat16* __restrict__ x, int B,
                                                                  int D, int grid, int C) {
