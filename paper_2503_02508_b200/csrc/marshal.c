@@ -186,13 +186,14 @@ static PyObject* bind(PyObject* self, PyObject* args) {
 }
 
 #define FAST(name) (PyCFunction)(void (*)(void))name, METH_FASTCALL | METH_KEYWORDS
+#define SIGNATURE_ENDS "\n--\n\n"   /* what makes the line a signature that inspect finds */
 static PyMethodDef methods[] = {
     {"bind", bind, METH_VARARGS, "Sets the functions that the calls below reach."},
-    {"qdit_quantize_act", FAST(quantize_act), "qdit_quantize_act(ctx, x, x_dtype, M, K, ldx, mode, qp, dyn_scale, q, ldq)"},
-    {"qdit_w8a8_linear", FAST(w8a8_linear), "qdit_w8a8_linear(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo)"},
-    {"qdit_w4a8_linear", FAST(w4a8_linear), "qdit_w4a8_linear(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, w8_scratch=None)"},
-    {"qdit_attention", FAST(attention), "qdit_attention(ctx, q, k, v, ld, B, H, T, dh, softmax_scale, out, out_dtype, out_qp=None, out_scale_dev=None)"},
-    {"qdit_adaln_modulate", FAST(adaln_modulate), "qdit_adaln_modulate(ctx, x, M, D, T, eps, shift, scale, ld_mod, out, out_dtype, out_qp=None, out_scale_dev=None)"},
+    {"qdit_quantize_act", FAST(quantize_act), "qdit_quantize_act(ctx, x, x_dtype, M, K, ldx, mode, qp, dyn_scale, q, ldq)" SIGNATURE_ENDS},
+    {"qdit_w8a8_linear", FAST(w8a8_linear), "qdit_w8a8_linear(ctx, A, W, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo)" SIGNATURE_ENDS},
+    {"qdit_w4a8_linear", FAST(w4a8_linear), "qdit_w4a8_linear(ctx, A, W_packed, M, N, K, a_qp, a_scale_dev, flags, epi, out, ldo, w8_scratch=None)" SIGNATURE_ENDS},
+    {"qdit_attention", FAST(attention), "qdit_attention(ctx, q, k, v, ld, B, H, T, dh, softmax_scale, out, out_dtype, out_qp=None, out_scale_dev=None)" SIGNATURE_ENDS},
+    {"qdit_adaln_modulate", FAST(adaln_modulate), "qdit_adaln_modulate(ctx, x, M, D, T, eps, shift, scale, ld_mod, out, out_dtype, out_qp=None, out_scale_dev=None)" SIGNATURE_ENDS},
     {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", NULL, -1, methods, NULL, NULL, NULL, NULL};
 

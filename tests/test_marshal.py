@@ -1,5 +1,6 @@
 """The natively marshalled calls hand the library the same arguments as their wrappers, and leave to them what they do not take."""
 import ctypes as C
+import inspect
 
 import numpy as np
 import pytest
@@ -92,3 +93,8 @@ def test_keywords_and_defaults(recorded):
     q.qdit_w4a8_linear(77, X, Y, 1, 2, 3, QP, X, 1, None, Z, 5, w8_scratch=X)
     q.qdit_w4a8_linear(77, X, Y, 1, 2, 3, QP, X, 1, None, Z, 5, X)
     assert log[0] == log[1] and log[2] == log[3]
+
+
+@pytest.mark.parametrize("name", list(CALLS))
+def test_signatures_are_those_of_the_wrappers(name):
+    assert inspect.signature(getattr(q, name)) == inspect.signature(binding._WRAPPERS[binding._NATIVE.index(name)])
