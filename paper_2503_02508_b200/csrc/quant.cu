@@ -340,14 +340,12 @@ __device__ __forceinline__ void ln_load_row(const __nv_bfloat16* __restrict__ xr
   }
 }
 
-// (Four CTAs per SM where rows are short: a launch fills two places and the next one starts beside it.  With 80 registers and three places 8192
-// rows of 392 values with f32 output take 6.9 us back to back instead of 5.8.)
-template <int NV, bool MAX>   // MAX: f32 output whose largest magnitude goes to *absmax
-__global__ void __launch_bounds__(256, NV <= 2 ? 4 : 0) ln_modulate_kernel(const __nv_bfloat16* __restrict__ x, int M, int D, int T,
+template <int NV, bool MAX, bool EARLY>   // MAX: f32 output whose largest magnitude goes to *absmax; EARLY: see ln_modulate_q8_kernel
+__global__ void __launch_bounds__(256) ln_modulate_kernel(const __nv_bfloat16* __restrict__ x, int M, int D, int T,
                                                           float eps, const float* __restrict__ shift,
                                                           const float* __restrict__ scale, int64_t ld_mod,
                                                           void* __restrict__ out, int out_dtype, QuantArgs qa,
-                                                          int rows_per_cta, int early, float* __restrict__ absmax) {
+                                                          int rows_per_cta, float* __restrict__ absmax) {
   extern __shared__ float4 s_par[];  // [2 samples][mul, add][NV][2 halves][32 lanes]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int row_begin = blockIdx.x * rows_per_cta;
@@ -356,12 +354,13 @@ __global__ void __launch_bounds__(256, NV <= 2 ? 4 : 0) ln_modulate_kernel(const
   const int nvec = D >> 3;
   int row = row_begin + warp;
   uint4 raw[NV], raw_next[NV];
-  if (!early) {   // (see ln_modulate_q8_kernel)
+  if constexpr (!EARLY) {
     grid_dependency_wait();
+    grid_dependency_release();
     if (row < row_end) ln_load_row<NV>(x + static_cast<int64_t>(row) * D, nvec, lane, raw);
   }
   float inv = 1.0f;
-  if (out_dtype == QDIT_I8) inv = __fdiv_rn(1.0f, device_value(qa.scale_dev, qa.scale));
+  if (out_dtype == QDIT_I8) inv = __fdiv_rn(1.0f, qa.scale_dev ? __ldg(qa.scale_dev) : qa.scale);
   const int b0 = row_begin / T;
   for (int s = 0; s < 2; ++s) {
     if (static_cast<int64_t>(b0 + s) * T >= row_end) break;
@@ -378,11 +377,11 @@ __global__ void __launch_bounds__(256, NV <= 2 ? 4 : 0) ln_modulate_kernel(const
       }
     }
   }
-  if (early) {
+  if constexpr (EARLY) {
     grid_dependency_wait();
+    grid_dependency_release();
     if (row < row_end) ln_load_row<NV>(x + static_cast<int64_t>(row) * D, nvec, lane, raw);
   }
-  grid_dependency_release();
   __syncthreads();
   const float inv_d = 1.0f / static_cast<float>(D);
   const int64_t second = static_cast<int64_t>(b0 + 1) * T;  // first row of the second staged sample
@@ -474,11 +473,11 @@ __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b
 // 28 warps per SM (two CTAs of 14): at the 8192 rows of the 256-token workload a warp then has two rows; with 24 it had 2.3,
 // that is three turns.  The next row is fetched into the registers of the current one as soon as that one is widened.
 constexpr int LNQ_WARPS = 14;
-template <int NV4>
+template <int NV4, bool EARLY>
 __global__ void __launch_bounds__(LNQ_WARPS * 32, 2) ln_modulate_q8_kernel(const __nv_bfloat16* __restrict__ x, int M, int T, float eps,
                                                                 const float* __restrict__ shift,
                                                                 const float* __restrict__ scale, int64_t ld_mod,
-                                                                uint8_t* __restrict__ out, QuantArgs qa, int rows_per_cta, int early) {
+                                                                uint8_t* __restrict__ out, QuantArgs qa, int rows_per_cta) {
   constexpr int D = NV4 * 128, D4 = D / 4;
   extern __shared__ float4 s_par[];  // [2 samples][mul, add][D / 4]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -494,10 +493,12 @@ __global__ void __launch_bounds__(LNQ_WARPS * 32, 2) ln_modulate_q8_kernel(const
       for (int j = 0; j < NV4; ++j) raw[j] = xr[32 * j];
     }
   };
-  // `early`: the modulation and the scale were written two launches ago or earlier and are staged while the previous kernel, which writes
-  // x, still runs
-  if (!early) {
+  // EARLY: the modulation and the scale were written two launches ago or earlier and are staged while the previous kernel, which writes
+  // x, still runs.  (Not a run-time choice: rows loaded in a branch are waited for behind it, and the two latencies add up: 1024 x 1152 with f32
+  // output 3.5 us by itself instead of 3.2.)
+  if constexpr (!EARLY) {
     grid_dependency_wait();
+    grid_dependency_release();
     load_row();
   }
   const float inv = __fdiv_rn(1.0f, device_value(qa.scale_dev, qa.scale));
@@ -512,11 +513,11 @@ __global__ void __launch_bounds__(LNQ_WARPS * 32, 2) ln_modulate_q8_kernel(const
       s_par[(s * 2 + 1) * D4 + i] = make_float4(h4.x * inv, h4.y * inv, h4.z * inv, h4.w * inv);
     }
   }
-  if (early) {
+  if constexpr (EARLY) {
     grid_dependency_wait();
+    grid_dependency_release();
     load_row();
   }
-  grid_dependency_release();
   __syncthreads();
   constexpr float inv_d = 1.0f / static_cast<float>(D);
   const int second = (b0 + 1) * T;  // first row of the second staged sample
@@ -574,9 +575,9 @@ template <int NV4>
 void launch_ln_q8(qdit_ctx* ctx, const void* x, int64_t M, const float* shift, const float* scale, int64_t ld_mod,
                   int64_t T, float eps, void* out, QuantArgs qa, int64_t rows, bool early) {
   const unsigned grid = static_cast<unsigned>((M + rows - 1) / rows);
-  qdit_launch_overlapped(ctx, ln_modulate_q8_kernel<NV4>, dim3(grid), dim3(LNQ_WARPS * 32), static_cast<size_t>(NV4) * 128 * 16,
+  qdit_launch_overlapped(ctx, early ? ln_modulate_q8_kernel<NV4, true> : ln_modulate_q8_kernel<NV4, false>, dim3(grid), dim3(LNQ_WARPS * 32), static_cast<size_t>(NV4) * 128 * 16,
                          static_cast<const __nv_bfloat16*>(x), static_cast<int>(M), static_cast<int>(T), eps, shift, scale,
-                         ld_mod, static_cast<uint8_t*>(out), qa, static_cast<int>(rows), static_cast<int>(early));
+                         ld_mod, static_cast<uint8_t*>(out), qa, static_cast<int>(rows));
 }
 
 // Row range per CTA: `per_sm` CTAs per SM, at least eight rows, at most what keeps a range within two samples.
@@ -593,9 +594,11 @@ void launch_ln(qdit_ctx* ctx, const void* x, int64_t M, int D, int64_t T, float 
                const float* scale, int64_t ld_mod, void* out, int out_dtype, QuantArgs qa, bool early, float* absmax) {
   const int64_t rows = ln_rows_per_cta(ctx, M, T, 2);
   const unsigned grid = static_cast<unsigned>((M + rows - 1) / rows);
-  qdit_launch_overlapped(ctx, absmax ? ln_modulate_kernel<NV, true> : ln_modulate_kernel<NV, false>, dim3(grid), dim3(256), static_cast<size_t>(NV) * 4096,
+  const auto kernel = absmax ? (early ? ln_modulate_kernel<NV, true, true> : ln_modulate_kernel<NV, true, false>)
+                             : (early ? ln_modulate_kernel<NV, false, true> : ln_modulate_kernel<NV, false, false>);
+  qdit_launch_overlapped(ctx, kernel, dim3(grid), dim3(256), static_cast<size_t>(NV) * 4096,
                          static_cast<const __nv_bfloat16*>(x), static_cast<int>(M), D, static_cast<int>(T), eps, shift, scale,
-                         ld_mod, out, out_dtype, qa, static_cast<int>(rows), static_cast<int>(early), absmax);
+                         ld_mod, out, out_dtype, qa, static_cast<int>(rows), absmax);
 }
 
 }  // namespace
