@@ -412,7 +412,9 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
       // (f32 output: with one wave only; there the epilogue is the longer part of a tile, 8192 x 3456 x 1152 36.9 us against 33.9)
       if (cls == 6 ? waves == 1 : cost <= qdit_gemm_pair_cost(ctx, p) + 1500.0) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
     }
-    if (staged && (slow ? p.M > BM && pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) == 1 : !one_wave))
+    // (at most 128 rows: half of a pair's tokens would be padding; single CTAs / pairs: 1 x 193536 x 128 codes 18.8 / 44.4 us, 33 x 193536 x 384 22.5 / 42.7,
+    // 100 x 65536 x 768 codes 14.9 / 19.0; from 129 rows on 160 x 193536 x 384 codes 63.7 / 46.2, 200 x 30720 x 3072 40 / 26.5)
+    if (staged && p.M > BM && (slow ? pick_split(ctx, p.M, p.N, p.K, SPLIT_SPARE_SLOW) == 1 : !one_wave))
       return qdit_launch_gemm_pair(ctx, A, W, p, a_unsigned);
   }
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0) {

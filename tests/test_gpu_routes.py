@@ -1,0 +1,35 @@
+"""Which kernel serves a linear layer, at sizes on both sides of the rules' lines."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+TOKEN_MAJOR, CHANNEL_MAJOR, PAIRS, ROWS = "gemm_i8_kernel", "gemm_i8_t_kernel", "gemm_i8_pair_kernel", "few_rows_kernel"
+
+
+def _flags(q, kind):
+    return {"bf16": q.QDIT_EPI_OUT_BF16, "codes": q.QDIT_EPI_GELU | q.QDIT_EPI_QUANT_OUT, "f32": q.QDIT_EPI_OUT_F32,
+            "gated": q.QDIT_EPI_GATE | q.QDIT_EPI_RESIDUAL | q.QDIT_EPI_OUT_BF16}[kind] | q.QDIT_EPI_BIAS
+
+
+@pytest.mark.parametrize("kind,M,N,K,kernel", [
+    # at most 128 rows: half of a pair's tokens would be padding
+    ("bf16", 128, 30720, 128, TOKEN_MAJOR), ("bf16", 129, 30720, 128, PAIRS),
+    ("codes", 64, 30720, 128, TOKEN_MAJOR), ("gated", 128, 30720, 128, TOKEN_MAJOR), ("gated", 129, 30720, 128, PAIRS),
+])
+def test_route(kind, M, N, K, kernel):
+    import paper_2503_02508_b200 as q
+    ctx = q.qdit_create(0, None)
+    A = torch.ones((M, K), dtype=torch.int8, device="cuda")
+    W = torch.ones((N, K), dtype=torch.int8, device="cuda")
+    ws, bias, gate = (torch.ones(N, device="cuda") for _ in range(3))
+    out = torch.zeros((M, N), dtype={"codes": torch.int8, "f32": torch.float32}.get(kind, torch.bfloat16), device="cuda")
+    residual = torch.zeros_like(out)
+    epi = q.epilogue(w_scale=ws, bias=bias, gate=gate, ld_gate=N, tokens_per_sample=1 << 20, residual=residual)
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        q.qdit_w8a8_linear(ctx, A, W, M, N, K, q.qparams(1.0), None, _flags(q, kind), epi, out, N)
+        q.qdit_sync(ctx)
+    names = [e.name for e in prof.events() if "_kernel" in e.name]
+    q.qdit_destroy(ctx)
+    assert len(names) == 1 and kernel + "<" in names[0], names
