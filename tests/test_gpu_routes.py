@@ -16,6 +16,9 @@ def _flags(q, kind):
     # at most 128 rows: half of a pair's tokens would be padding
     ("bf16", 128, 30720, 128, TOKEN_MAJOR), ("bf16", 129, 30720, 128, PAIRS),
     ("codes", 64, 30720, 128, TOKEN_MAJOR), ("gated", 128, 30720, 128, TOKEN_MAJOR), ("gated", 129, 30720, 128, PAIRS),
+    # f32 output of many rows: channel-major where the output's own time counts
+    ("f32", 2304, 6144, 768, CHANNEL_MAJOR), ("f32", 2304, 6144, 784, PAIRS), ("f32", 1023, 6144, 128, PAIRS),
+    ("f32", 3072, 4616, 384, CHANNEL_MAJOR), ("f32", 3072, 4616, 400, PAIRS),
 ])
 def test_route(kind, M, N, K, kernel):
     import paper_2503_02508_b200 as q
