@@ -16,6 +16,8 @@ def _flags(q, kind):
     # at most 128 rows: half of a pair's tokens would be padding
     ("bf16", 128, 30720, 128, TOKEN_MAJOR), ("bf16", 129, 30720, 128, PAIRS),
     ("codes", 64, 30720, 128, TOKEN_MAJOR), ("gated", 128, 30720, 128, TOKEN_MAJOR), ("gated", 129, 30720, 128, PAIRS),
+    # bf16 output of one wave of channel-major tiles
+    ("bf16", 1024, 4608, 2048, CHANNEL_MAJOR), ("bf16", 1301, 3456, 512, CHANNEL_MAJOR), ("bf16", 1536, 6912, 768, PAIRS), ("bf16", 1024, 2304, 2048, TOKEN_MAJOR),
     # f32 output of many rows: channel-major where the output's own time counts
     ("f32", 2304, 6144, 768, CHANNEL_MAJOR), ("f32", 2304, 6144, 784, PAIRS), ("f32", 1023, 6144, 128, PAIRS),
     ("f32", 3072, 4616, 384, CHANNEL_MAJOR), ("f32", 3072, 4616, 400, PAIRS),
