@@ -369,8 +369,11 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
   // One to four rows, f32 output (the modulation of as many images): the weights are streamed past the rows instead of through the
   // tensor core (us, 1 and 4 rows, tensor core / streamed: 193536 x 1152 51.2 / 35.1 and 51.4 / 45.4, packed 4-bit weights 73.0 / 22.1 and
   // 75.9 / 47.7; 6912 x 1152 7.0 / 2.8 and 7.0 / 4.2; 1152 x 4608 7.1 / 4.1 and 7.2 / 5.7; 1152 x 384 3.4 / 2.2 and 3.3 / 2.6).  Beyond
-  // four the dot products take longer than the weights.
-  if (epi_class(p.flags) == 6 && p.M <= FEW_ROWS && !p.absmax && p.K <= FEW_ROWS_K && ctx->opt[QDIT_OPT_GEMM_BN] == 0 && ctx->opt[QDIT_OPT_GEMM_T] == 0 &&
+  // four the dot products take longer than the weights; with three and four rows they do so for many channels of a short reduction too
+  // (tensor core / streamed: 193536 x 128 17.6 / 28.1, 65536 x 384 10.7 / 12.2, 24576 x 256 5.1 / 5.7; packed 193536 x 64 25.2 /
+  // 30.7, 65536 x 384 12.9 / 14.5; but 65536 x 768 13.5 / 13.7 and x 1024 17.0 / 15.1, 30720 x 384 7.8 / 6.6, 30720 x 32 7.3 / 6.1, packed 65536 x 512 14.4 / 12.9, 65536 x 32 12.3 / 11.2).
+  const bool many_short = p.M > 2 && (p.N >= 49152 ? (packed4 ? p.K >= 64 && p.K < 512 : p.K < 768) : p.N > 16384 && !packed4 && p.K >= 96 && p.K < 384);
+  if (epi_class(p.flags) == 6 && p.M <= FEW_ROWS && !p.absmax && !many_short && p.K <= FEW_ROWS_K && ctx->opt[QDIT_OPT_GEMM_BN] == 0 && ctx->opt[QDIT_OPT_GEMM_T] == 0 &&
       !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE])
     return qdit_launch_few_rows(ctx, A, W, p, a_unsigned, packed4);
   if (packed4) {

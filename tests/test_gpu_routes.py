@@ -16,6 +16,9 @@ def _flags(q, kind):
     # at most 128 rows: half of a pair's tokens would be padding
     ("bf16", 128, 30720, 128, TOKEN_MAJOR), ("bf16", 129, 30720, 128, PAIRS),
     ("codes", 64, 30720, 128, TOKEN_MAJOR), ("gated", 128, 30720, 128, TOKEN_MAJOR), ("gated", 129, 30720, 128, PAIRS),
+    # three and four rows of many channels of a short reduction: not streamed
+    ("f32", 4, 49152, 752, TOKEN_MAJOR), ("f32", 3, 49152, 768, ROWS), ("f32", 2, 49152, 128, ROWS), ("f32", 3, 16392, 96, TOKEN_MAJOR),
+    ("f32", 3, 16392, 80, ROWS), ("f32", 4, 20480, 384, ROWS), ("f32", 4, 16384, 128, ROWS),
     # bf16 output of one wave of channel-major tiles
     ("bf16", 1024, 4608, 2048, CHANNEL_MAJOR), ("bf16", 1301, 3456, 512, CHANNEL_MAJOR), ("bf16", 1536, 6912, 768, PAIRS), ("bf16", 1024, 2304, 2048, TOKEN_MAJOR),
     # f32 output of many rows: channel-major where the output's own time counts
