@@ -491,9 +491,10 @@ def test_code_output_leaves_the_padding_of_its_rows_alone(q, ctx, N, ldo):
     (256, 1152, 4608),   # three CTAs per tile: row groups 6, 5, 5
     (300, 1152, 800),    # seven k-blocks: not split
     (300, 1152, 5120),   # two CTAs per tile: ragged rows
-    (1040, 2312, 256),   # channel-major kernel: ragged rows and columns
+    (1040, 2312, 256),   # bf16, f32, per-token: channel-major, ragged rows and columns
     (1025, 2304, 1152),
-    (4000, 1160, 1152),  # channel-major gated layer: 32 x 7 token-major tiles of 192 exceed one wave
+    (4000, 1160, 1152),  # gated layer by pairs: 32 x 7 token-major tiles of 192 exceed one wave; ragged rows and columns
+    (8000, 1152, 4608),  # gated layer of a long reduction, channel-major: two waves of 128 x 256 tiles, ragged rows
 ])
 @pytest.mark.parametrize("kind", ["i32", "f32", "bf16", "row", "gelu", "gated", "gated_nocache"])
 def test_automatic_kernel_gives_the_bits_of_the_token_major_kernel(q, ctx, M, N, K, kind):
