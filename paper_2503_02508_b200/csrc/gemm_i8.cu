@@ -411,10 +411,14 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
     const bool one_wave = static_cast<int64_t>((p.M + BM - 1) / BM) * ((p.N + 191) / 192) <= ctx->num_sms;
     if (staged && p.M >= 1024 && (cls == 3 ? p.N >= 1024 && !one_wave : (cls == 1 || cls == 5 || cls == 6) && p.N >= 2304)) {
       const int64_t waves = (static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) + ctx->num_sms - 1) / ctx->num_sms;
-      const double cost = static_cast<double>(waves) * ((p.K + BK - 1) / BK * 620.0 + 600.0) + 4500.0;
-      // (bf16 output: 2500 clocks, 3000 with one wave, in which a pair's longer start is not hidden by anything: channel-major / pairs, 1024 x 4608 x
-      // 2048 9.1 / 10.5 us, 2048 x 2304 x 3072 11.4 / 12.8, 1301 x 3456 x 512 6.5 / 7.4, but 1536 x 6912 x 768 13.8 / 12.0)
-      const double spare = cls != 1 || one_wave ? 1500.0 : waves == 1 ? 3000.0 : 2500.0;
+      // (the epilogue of a gated tile, which also reads the residual, takes at least 4750 clocks, and bounds the tile where the reduction is short: channel-
+      // major / pairs, 5000 x 4608 x 16 33.0 / 27.7 us, 4096 x 3464 x 512 30.9 / 26.0, 5000 x 3456 x 1024 25.8 / 22.0; but 16384 x 1152 x 512 20.5 / 27.0, 8192 x
+      // 4608 x 384 41.6 / 43.5)
+      const double products = (p.K + BK - 1) / BK * 620.0 + 600.0, tile = cls == 3 && products < 4750.0 ? 4750.0 : products;
+      const double cost = static_cast<double>(waves) * tile + 4500.0;
+      // (a pair's start beyond that of a single CTA; with one wave nothing hides it.  Channel-major / pairs, bf16: 1024 x 4608 x 2048 9.1 / 10.5 us, 2048 x
+      // 2304 x 3072 11.4 / 12.8, 1301 x 3456 x 512 6.5 / 7.4, but 1536 x 6912 x 768 13.8 / 12.0; gated: 4096 x 1152 x 1152 9.8 / 10.9)
+      const double spare = cls == 3 ? (waves == 1 ? 3000.0 : 0.0) : cls != 1 || one_wave ? 1500.0 : waves == 1 ? 3000.0 : 2500.0;
       // (f32 output: with one wave, and with reductions short enough that the output's own time counts: a tile's 128 channels are whole 512-byte
       // pieces of a row there, which memory takes at 5.4 TB/s, where a pair's 128-byte pieces reach 3.4; us, channel-major / pairs: 10000 x
       // 20480 x 64 151 / 242, 6144 x 20480 x 384 98 / 152, 8192 x 6912 x 384 44 / 53, 4096 x 30720 x 768 127 / 169, 1728 x 4608 x 256 8.8 /

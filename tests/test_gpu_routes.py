@@ -18,6 +18,7 @@ def _flags(q, kind):
     ("codes", 64, 30720, 128, TOKEN_MAJOR), ("gated", 128, 30720, 128, TOKEN_MAJOR), ("gated", 129, 30720, 128, PAIRS),
     # gated layers of more than one wave of token-major tiles: by estimate
     ("gated", 8192, 1152, 1152, CHANNEL_MAJOR), ("gated", 8000, 1152, 4608, CHANNEL_MAJOR), ("gated", 4000, 1160, 1152, PAIRS), ("gated", 65536, 1152, 4608, PAIRS),
+    ("gated", 4000, 1160, 64, PAIRS), ("gated", 4096, 1152, 1152, CHANNEL_MAJOR), ("gated", 5000, 3456, 1024, PAIRS),
     # three and four rows of many channels of a short reduction: not streamed
     ("f32", 4, 49152, 752, TOKEN_MAJOR), ("f32", 3, 49152, 768, ROWS), ("f32", 2, 49152, 128, ROWS), ("f32", 3, 16392, 96, TOKEN_MAJOR),
     ("f32", 3, 16392, 80, ROWS), ("f32", 4, 20480, 384, ROWS), ("f32", 4, 16384, 128, ROWS),
