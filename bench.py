@@ -42,9 +42,9 @@ STOCHASTIC = {"ddpm250"}
 
 
 # DRAM bytes (read + written) per GEMM launch, from the ncu capture summarised in
-# profiles/gemm_i8_layers_m8192_sections.txt: QKV 18.3 MB, proj 30.0 MB, fc1 14.9 MB, fc2 65.5 MB per launch at
+# profiles/gemm_i8_layers_m8192_sections.txt: QKV 17.9 MB, proj 30.0 MB, fc1 15.0 MB, fc2 65.3 MB per launch at
 # M = 8192 (the shapes of the 50-step workload); each layer is 700 of the trajectory's 2801 GEMM launches.
-NCU_GEMM_DRAM_BYTES_PER_LAUNCH = 700 * (18.3e6 + 30.0e6 + 14.9e6 + 65.5e6) / 2801
+NCU_GEMM_DRAM_BYTES_PER_LAUNCH = 700 * (17.9e6 + 30.0e6 + 15.0e6 + 65.3e6) / 2801
 
 
 def measured_peaks():
@@ -321,7 +321,7 @@ def run_ours(args):
     g_n, g_ms, g_ops = prof[q.QDIT_PROF_GEMM]
     int8_peak = 2.0 * peaks["bf16_sustained"]          # dense int8 : bf16 nominal ratio 4.5 : 2.25
     achieved = g_ops / (g_ms * 1e-3) / 1e12 if g_ms > 0 else 0.0
-    roofline = {"bound": "tensor", "kernel": "int8 GEMMs (gemm_i8_t_kernel, gemm_i8_kernel)", "achieved": achieved,
+    roofline = {"bound": "tensor", "kernel": "int8 GEMMs (gemm_i8_pair_kernel, gemm_i8_t_kernel)", "achieved": achieved,
                 "peak": int8_peak, "unit": "TOP/s", "frac": achieved / int8_peak, "frac_of_nominal_4500": achieved / 4500.0,
                 "traffic": NCU_GEMM_DRAM_BYTES_PER_LAUNCH if args.workload == "ddim50" else None,
                 "traffic_note": "launch-weighted mean of the four block-level layers at M = 8192 (ncu, L2-warm sweep)",

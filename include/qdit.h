@@ -80,6 +80,7 @@ int64_t qdit_launch_count(const qdit_ctx* ctx);
  *                                   a kernel's preamble overlaps the tail of the kernel before it; 0: plain launches
  *   QDIT_OPT_GEMM_BN                0 (default): automatic; 64 | 128 | 192: token-major GEMM kernel with 128 x BN tiles
  *   QDIT_OPT_GEMM_T                 0 (default): automatic; 128 | 256: channel-major GEMM kernel with 128 x BT tiles
+ *                                   (8-bit output with the run-time-flag epilogue, which is slower than any automatic choice)
  *   QDIT_OPT_GEMM_GENERIC_EPILOGUE  1: the GEMM kernels' run-time-flag epilogue instead of the specialised classes
  *   QDIT_OPT_ATTN                   0 (default): the mma.sync attention kernel at 64 tokens, the tcgen05 kernel at more;
  *                                   1: the mma.sync kernel for every token count; 2: the tcgen05 kernel for every token count

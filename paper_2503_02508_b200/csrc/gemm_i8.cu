@@ -396,14 +396,14 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
   const bool row_scale = (flags & QDIT_EPI_ROW_SCALE) != 0;
   if (!row_scale && ctx->opt[QDIT_OPT_GEMM_T] != 0) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, ctx->opt[QDIT_OPT_GEMM_T]);
   // Kernel choice.  A layer whose 128 x 192 tiles fill no more than one wave runs token-major, one CTA per tile (below): pairs gain
-  // nothing there (2048 x 3456 x 384: 4.8 us against 5.0, 1024 x 1152 x 1152 gated 5.3 and 6.5).  From the second wave on pairs of CTAs
-  // are faster (us, single CTAs / pairs: QKV of XL/2 2048 rows 11.0 / 9.0, 8192 26.7 / 24.0, 65536 222 / 182; fc1 40.1 / 35.4 and
-  // 310 / 295; fc2 5000 rows 31.2 / 24.4, 65536 276 / 256; proj 14.9 / 11.3 and 117 / 113).  Per-token scales and f32 output take pairs
-  // earlier, because their token-major epilogue decides at run time what to do (512 x 3456 x 1152: 8.6 / 5.9 and 8.2 / 6.4), unless the
-  // split reduction, which splits the epilogue too, serves them.  Layers of few columns, or of rows just right for it, fill the chip better
-  // with the 128 x 256 channel-major tiles of single CTAs, at 620 clocks per k-block, 600 per tile and 4500 for the last epilogue; a
-  // pair's launch costs 1500 clocks more (channel-major / pairs: QKV 1280 rows 7.2 / 7.7 us, with per-token scales 11.0 / 12.1; gated fc2 4096 rows
-  // 18.4 / 20.3, 8192 with 4-bit codes 34.2 / 35.9, proj 4096 9.7 / 10.5).
+  // nothing there, with short reductions or long ones (us, single CTAs / pairs: 2048 x 3456 x 384 4.8 / 5.0, 1024 x 1152 x 1152 gated 5.3 / 6.5, 2048 x
+  // 1152 x 4608 gated 11.7 / 11.8, 3072 rows 13.7 / 14.8).  From the second wave on pairs of CTAs are faster (QKV of XL/2 2048 rows 11.0 / 9.0, 8192
+  // 26.7 / 24.0, 65536 222 / 182; fc1 40.1 / 35.4 and 310 / 270; fc2 5000 rows 31.2 / 24.4, 65536 276 / 252; proj 14.9 / 11.3 and 117 / 105).  Per-token
+  // scales and f32 output take pairs earlier, because their token-major epilogue decides at run time what to do (512 x 3456 x 1152: 8.6 / 5.9 and 8.2 /
+  // 6.4), unless the split reduction, which splits the epilogue too, serves them.  Layers of few columns, or of rows just right for it, fill the chip better
+  // with the 128 x 256 channel-major tiles of single CTAs, at 620 clocks per k-block, 600 per tile and 4500 for the last epilogue (channel-major / pairs: QKV
+  // 1280 rows 7.2 / 7.7 us, with per-token scales 11.0 / 12.1; gated 4096 rows proj 9.1 / 10.0, fc2 17.4 / 18.3; level at 8192 rows, without / with a cache
+  // copy: proj 13.3 / 13.2 and 15.5 / 14.8, fc2 33.8 / 34.0 and 37.8 / 37.6, with 4-bit codes 34.2 / 35.9; 16384 rows fc2 66.0 / 67.8 and 73.0 / 75.0).
   if (ctx->opt[QDIT_OPT_GEMM_BN] == 0 && !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE]) {
     // (8-bit rows leave through TMA stores of whole 16-byte pieces, and a 32-token chunk of a gated layer has one gate row)
     const bool staged = cls == 1 || cls == 5 || cls == 6 || cls == 7 || (cls == 2 && p.N % 16 == 0 && ldo % 16 == 0) || (cls == 3 && p.tokens % 32 == 0);

@@ -7,7 +7,7 @@
 // channels, and reads no more than those (the tensor cores exchange the halves): 64 KB, 512 clocks as well.  Measured without an
 // epilogue, 8192 x 4608 x 4608: 0.30 us per k-block against 0.355 with single CTAs, 0.26 with operands that stay in shared memory.
 // 8192 x 3456 x 1152 takes 24.0 us (26.9 with single CTAs), 65536 x 3456 x 1152 182-188 (222): 2.8 POP/s at 1.4 GHz, where the power cap
-// leaves the clock; 8192 x 4608 x 1152 with GELU and codes 35.5 (40.1); 65536 x 1152 x 4608 gated 256 (276).
+// leaves the clock; 8192 x 4608 x 1152 with GELU and codes 36.4 (40.1); 65536 x 1152 x 4608 gated 256 (276).
 //
 // CTA = 2 + EPI_WARPS warps: warp 0 TMA producer (of its own half of the operands; both CTAs' copies report to the leader's
 // barrier), warp 1 MMA issuer (the leader, CTA 0 of the pair, issues for both; commits arrive in both), the others epilogue: the

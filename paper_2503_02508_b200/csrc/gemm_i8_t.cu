@@ -25,8 +25,8 @@
 // stores (warp-level stores of 64-byte row pieces reach 4.2 TB/s on this chip, TMA stores of the same tiles
 // 6.7 TB/s, and they do not hold the issuing warp), and the residual of the gated epilogue arrives the same way
 // in reverse (TMA load one chunk ahead, ldmatrix.trans).
-// It serves the row counts at which its tiles make exactly one wave of the chip (see the dispatch in gemm_i8.cu); pairs of CTAs
-// (gemm_i8_p.cu) serve the others.
+// It serves the layers of many rows for which its estimate is below that of pairs of CTAs (gemm_i8_p.cu; the dispatch in gemm_i8.cu has both):
+// row counts at which its tiles fill their waves, among them the gated layers of XL/2 at 8192 and 16384 rows, and f32 output of short reductions.
 #include "gemm_common.cuh"
 
 
