@@ -7,7 +7,7 @@
 // channels, and reads no more than those (the tensor cores exchange the halves): 64 KB, 512 clocks as well.  Measured without an
 // epilogue, 8192 x 4608 x 4608: 0.30 us per k-block against 0.355 with single CTAs, 0.26 with operands that stay in shared memory.
 // 8192 x 3456 x 1152 takes 24.0 us (26.9 with single CTAs), 65536 x 3456 x 1152 182-188 (222): 2.8 POP/s at 1.4 GHz, where the power cap
-// leaves the clock; 8192 x 4608 x 1152 with GELU and codes 36.4 (40.1); 65536 x 1152 x 4608 gated 256 (276).
+// leaves the clock; 8192 x 4608 x 1152 with GELU and codes 36.2 (40.1); 65536 x 1152 x 4608 gated 256 (276).
 //
 // CTA = 2 + EPI_WARPS warps: warp 0 TMA producer (of its own half of the operands; both CTAs' copies report to the leader's
 // barrier), warp 1 MMA issuer (the leader, CTA 0 of the pair, issues for both; commits arrive in both), the others epilogue: the
@@ -127,11 +127,6 @@ __device__ __forceinline__ float2 gelu_tanh_f2(float2 x) {
   return make_float2(div_approx_ftz(x.x, d.x), div_approx_ftz(x.y, d.y));
 }
 
-template <bool B>
-struct Flush {
-  static constexpr bool value = B;
-};
-
 // Accumulators of a chunk (32 tokens x 32 channels) in fragments: a = tokens 0..15, b = tokens 16..31; the pair of channels
 // 8k + 2(t%4), + 1 of token 8g + t/4.
 __device__ __forceinline__ float2 frag_acc(const uint32_t (&a)[16], const uint32_t (&b)[16], int g, int k) {
@@ -150,6 +145,44 @@ struct PairParams {
   int tokens_first;
   uint32_t idesc;
 };
+
+// The epilogue of class 2 for an output step below 2^-125, at which subnormal activations have codes (see there): the codes of a warp's chunks, one
+// after the other and by plain stores.  Not inlined, so that the usual loop is compiled as if this were not there.
+struct TinySteps {
+  uint64_t* tfull_bar;
+  volatile int* abort_flag;
+  uint32_t taddr, tempty0;      // this lane quadrant's rows of the accumulators; the leader's barriers that take them back
+  float a_scale, o_inv;
+  int pair, num_pairs, row, part, split;   // row: of this thread's token in the pair's tile
+};
+__device__ __noinline__ void codes_of_tiny_steps(const PairParams& pp, const TinySteps s) {
+  const GemmParams& p = pp.g;
+  const int chunks = pp.bn / 32, total = p.num_m_tiles * p.num_n_tiles, lane = static_cast<int>(threadIdx.x) & 31;
+  int it = 0;
+  for (int i = s.pair; i < total; i += s.num_pairs, ++it) {
+    const int as = it & 1;
+    const int m = (pp.tokens_first ? i % p.num_m_tiles : i / p.num_n_tiles) * 256 + s.row, n0 = (pp.tokens_first ? i / p.num_m_tiles : i % p.num_n_tiles) * pp.bn;
+    if (!mbar_wait_warp(&s.tfull_bar[as], static_cast<uint32_t>(it >> 1) & 1u, s.abort_flag, p.status)) return;
+    tc_fence_after();
+    for (int c = s.part; c < chunks; c += s.split) {
+      uint32_t v[32];
+      __syncwarp();
+      tmem_ld_32x32(s.taddr + static_cast<uint32_t>(as * ACC_COLS + c * 32), v);
+      tmem_ld_wait_for(v);
+#pragma unroll 1
+      for (int j = 0; j < 32; ++j) {
+        const int n = n0 + c * 32 + j;
+        if (m >= p.M || n >= p.N) continue;
+        const int acc = static_cast<int>(v[j]) - (p.a_zp != 0 ? p.a_zp * p.w_colsum[n] : 0);
+        const float x = gelu_tanh_f(__fmaf_rn(static_cast<float>(acc), __fmul_rn(s.a_scale, p.w_scale[n]), p.bias[n]));
+        static_cast<uint8_t*>(p.out)[static_cast<int64_t>(m) * p.ldo + n] = static_cast<uint8_t>(__float2int_rn(quantize_code(x, s.o_inv, p.o_zp, p.o_qmin, p.o_qmax)));
+      }
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) arrive_at_leader(s.tempty0 + static_cast<uint32_t>(as) * 8u);
+  }
+}
 
 template <int EPI>
 __global__ void __launch_bounds__(PCfg<EPI>::THREADS, 1)
@@ -333,73 +366,73 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         }
       };
       fetch(first, part);
-      // A subnormal activation has a code other than zero only if a step is below 2^-125.  Those loops are apart: the choice inside the
-      // loop costs 8 to 15 %, this way 1 % (8192 x 4608 x 1152 36.1 / 36.4 us, 65536 rows 282 / 283, 5000 x 6912 x 384 36.6 / 37.1).
-      auto all_tiles = [&](auto flush) {
-        constexpr bool FTZ = decltype(flush)::value;
-        for (Tile t = first; t.i < total_tiles && ok; next(t), ++it) {
-          const int as = it & 1;
-          const int row0 = m_of(t) + rank * 128 + quad * 32, n0 = n_of(t);
-          if (!mbar_wait_warp(&tfull_bar[as], static_cast<uint32_t>(it >> 1) & 1u, abort_flag, p.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(as * ACC_COLS);
-          if (c_last < 0) release(as);
+      // A subnormal activation has a code other than zero only if a step is below 2^-125.  Such steps have a function of their own, which costs the
+      // others 0.1 to 0.2 us per launch (2048 x 4608 x 1152 13.4 / 13.6, 65536 rows 280.5 / 280.6): a choice inside the loop costs 8 to 15 % (its registers
+      // and its schedule are full), a second copy of it 1 %.
+      if (!(o_inv <= 0x1p125f)) {   // (infinite too)
+        codes_of_tiny_steps(pp, TinySteps{tfull_bar, abort_flag, tmem_base + (static_cast<uint32_t>(quad * 32) << 16), tempty0, a_scale, o_inv, pair, num_pairs,
+                                          rank * 128 + quad * 32 + lane, part, C::SPLIT});
+      } else
+      for (Tile t = first; t.i < total_tiles && ok; next(t), ++it) {
+        const int as = it & 1;
+        const int row0 = m_of(t) + rank * 128 + quad * 32, n0 = n_of(t);
+        if (!mbar_wait_warp(&tfull_bar[as], static_cast<uint32_t>(it >> 1) & 1u, abort_flag, p.status)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(as * ACC_COLS);
+        if (c_last < 0) release(as);
 #pragma unroll 1
-          for (int c = part; c < chunks; c += C::SPLIT) {
-            const bool live = row0 < p.M && n0 + c * 32 < p.N;   // uniform over the warp
-            uint32_t v[32];
-            if (live) tmem_ld_32x32(taddr + static_cast<uint32_t>(c * 32), v);
-            __syncwarp();   // the last chunk's parameters have been read
-            sc[lane] = __fmul_rn(a_scale, sc_next);
-            bi[lane] = bi_next;
-            __syncwarp();
-            if (c + C::SPLIT < chunks) {
-              fetch(t, c + C::SPLIT);
-            } else {
-              Tile ahead = t;
-              next(ahead);
-              fetch(ahead, part);
-            }
-            if (live) tmem_ld_wait_for(v);
-            if (c == c_last) release(as);
-            if (!live) continue;
-            if (p.a_zp != 0) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (n0 + c * 32 + j < p.N) v[j] -= static_cast<uint32_t>(p.a_zp * __ldg(p.w_colsum + n0 + c * 32 + j));
-            }
-            uint32_t w[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const float4 s4 = *reinterpret_cast<const float4*>(sc + 4 * j), b4 = *reinterpret_cast<const float4*>(bi + 4 * j);
-              const float2 x0 = gelu_tanh_f2<FTZ>(__ffma2_rn(to_float2(v[4 * j], v[4 * j + 1]), make_float2(s4.x, s4.y), make_float2(b4.x, b4.y)));
-              const float2 x1 = gelu_tanh_f2<FTZ>(__ffma2_rn(to_float2(v[4 * j + 2], v[4 * j + 3]), make_float2(s4.z, s4.w), make_float2(b4.z, b4.w)));
-              // clip(rne(t) + z, qmin, qmax) == rne(clamp(t, qmin - z, qmax - z)) + z; adding 1.5 * 2^23 rounds to nearest-even
-              // and leaves the integer in the low mantissa bits; the low byte is the stored code
-              float2 t0 = __fmul2_rn(x0, o2), t1 = __fmul2_rn(x1, o2);
-              t0 = __fadd2_rn(make_float2(fminf(fmaxf(t0.x, lo_f), hi_f), fminf(fmaxf(t0.y, lo_f), hi_f)), magic);
-              t1 = __fadd2_rn(make_float2(fminf(fmaxf(t1.x, lo_f), hi_f), fminf(fmaxf(t1.y, lo_f), hi_f)), magic);
-              w[j] = __byte_perm(__byte_perm(__float_as_uint(t0.x), __float_as_uint(t0.y), 0x0040),
-                                 __byte_perm(__float_as_uint(t1.x), __float_as_uint(t1.y), 0x0040), 0x5410);
-              if (z4 != 0u) w[j] = __vadd4(w[j], z4);   // code + z stays inside a byte
-            }
-            if (elect_one()) tma_store_wait_read<1>();   // the store that used this tile two chunks ago has read it
-            __syncwarp();
-            const uint32_t dst = row_addr + static_cast<uint32_t>(turn) * 1024u;
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + sw), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (sw ^ 16u)), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-            fence_async_smem();
-            __syncwarp();
-            if (elect_one()) {
-              tma_store_2d(&tmap_out, stg + turn * 1024, n0 + c * 32, row0);
-              tma_store_commit();
-            }
-            turn ^= 1;
+        for (int c = part; c < chunks; c += C::SPLIT) {
+          const bool live = row0 < p.M && n0 + c * 32 < p.N;   // uniform over the warp
+          uint32_t v[32];
+          if (live) tmem_ld_32x32(taddr + static_cast<uint32_t>(c * 32), v);
+          __syncwarp();   // the last chunk's parameters have been read
+          sc[lane] = __fmul_rn(a_scale, sc_next);
+          bi[lane] = bi_next;
+          __syncwarp();
+          if (c + C::SPLIT < chunks) {
+            fetch(t, c + C::SPLIT);
+          } else {
+            Tile ahead = t;
+            next(ahead);
+            fetch(ahead, part);
           }
+          if (live) tmem_ld_wait_for(v);
+          if (c == c_last) release(as);
+          if (!live) continue;
+          if (p.a_zp != 0) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (n0 + c * 32 + j < p.N) v[j] -= static_cast<uint32_t>(p.a_zp * __ldg(p.w_colsum + n0 + c * 32 + j));
+          }
+          uint32_t w[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float4 s4 = *reinterpret_cast<const float4*>(sc + 4 * j), b4 = *reinterpret_cast<const float4*>(bi + 4 * j);
+            const float2 x0 = gelu_tanh_f2<true>(__ffma2_rn(to_float2(v[4 * j], v[4 * j + 1]), make_float2(s4.x, s4.y), make_float2(b4.x, b4.y)));
+            const float2 x1 = gelu_tanh_f2<true>(__ffma2_rn(to_float2(v[4 * j + 2], v[4 * j + 3]), make_float2(s4.z, s4.w), make_float2(b4.z, b4.w)));
+            // clip(rne(t) + z, qmin, qmax) == rne(clamp(t, qmin - z, qmax - z)) + z; adding 1.5 * 2^23 rounds to nearest-even
+            // and leaves the integer in the low mantissa bits; the low byte is the stored code
+            float2 t0 = __fmul2_rn(x0, o2), t1 = __fmul2_rn(x1, o2);
+            t0 = __fadd2_rn(make_float2(fminf(fmaxf(t0.x, lo_f), hi_f), fminf(fmaxf(t0.y, lo_f), hi_f)), magic);
+            t1 = __fadd2_rn(make_float2(fminf(fmaxf(t1.x, lo_f), hi_f), fminf(fmaxf(t1.y, lo_f), hi_f)), magic);
+            w[j] = __byte_perm(__byte_perm(__float_as_uint(t0.x), __float_as_uint(t0.y), 0x0040),
+                               __byte_perm(__float_as_uint(t1.x), __float_as_uint(t1.y), 0x0040), 0x5410);
+            if (z4 != 0u) w[j] = __vadd4(w[j], z4);   // code + z stays inside a byte
+          }
+          if (elect_one()) tma_store_wait_read<1>();   // the store that used this tile two chunks ago has read it
+          __syncwarp();
+          const uint32_t dst = row_addr + static_cast<uint32_t>(turn) * 1024u;
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + sw), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (sw ^ 16u)), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+          fence_async_smem();
+          __syncwarp();
+          if (elect_one()) {
+            tma_store_2d(&tmap_out, stg + turn * 1024, n0 + c * 32, row0);
+            tma_store_commit();
+          }
+          turn ^= 1;
         }
-      };
-      if (o_inv <= 0x1p125f) all_tiles(Flush<true>());
-      else all_tiles(Flush<false>());   // (o_inv infinite too)
+      }
     } else {
       // row this thread addresses in stmatrix: row lane % 8 of a token group, 16-byte piece lane / 8 (64-byte swizzle)
       const uint32_t row_off = static_cast<uint32_t>(lane & 7) * 64u + ((static_cast<uint32_t>(lane >> 3) ^ (static_cast<uint32_t>(lane & 7) >> 1)) << 4);
