@@ -140,17 +140,16 @@ def test_tap_laplacian_matches_oracle(q, ctx, n, d, alpha, e):
 
 
 def test_bounded_wait_times_out_and_context_stays_usable(q, ctx):
-    """The time-out paths of the pipelined kernels (waiting and polling), exercised without hanging anything: a wait with a small
-    poll limit on a barrier that nobody signals runs out, a second waiter leaves through the abort flag, the kernel
+    """The time-out path of the pipelined kernels, exercised without hanging anything: a wait with a small poll
+    limit on a barrier that nobody signals runs out, a second waiter leaves through the abort flag, the kernel
     ends normally, qdit_sync reports the time-out once, and the context keeps working."""
     q.qdit_sync(ctx)
-    for polls in (1, 4096):
-        obs = torch.zeros(2, dtype=torch.int32, device="cuda")
-        q.qdit_selftest_wait_timeout(ctx, polls, obs)
-        assert q.lib.qdit_sync(ctx) == q.QDIT_ERR_TIMEOUT
-        assert b"wait" in q.lib.qdit_last_error(ctx)
-        assert obs.cpu().tolist() == [1, 1]
-        assert q.lib.qdit_sync(ctx) == q.QDIT_OK
+    obs = torch.zeros(2, dtype=torch.int32, device="cuda")
+    q.qdit_selftest_wait_timeout(ctx, 4096, obs)
+    assert q.lib.qdit_sync(ctx) == q.QDIT_ERR_TIMEOUT
+    assert b"wait" in q.lib.qdit_last_error(ctx)
+    assert obs.cpu().tolist() == [1, 1]
+    assert q.lib.qdit_sync(ctx) == q.QDIT_OK
     x = synth.normal(64, "after_timeout", (64, 128))
     out = torch.empty((64, 128), dtype=torch.uint8, device="cuda")
     q.qdit_quantize_act(ctx, dev(x), q.QDIT_F32, 64, 128, 128, q.QDIT_QUANT_STATIC, q.qparams(0.02), None, out, 128)
@@ -160,6 +159,19 @@ def test_bounded_wait_times_out_and_context_stays_usable(q, ctx):
     np.testing.assert_array_equal(got, want)
     assert q.lib.qdit_selftest_wait_timeout(ctx, 0, obs.data_ptr()) == q.QDIT_ERR_INVALID_ARG
     assert q.lib.qdit_selftest_wait_timeout(ctx, 1 << 21, obs.data_ptr()) == q.QDIT_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("polls", [1, 2, 4096])
+def test_polling_wait_times_out_too(q, ctx, polls):
+    """Both forms of the bounded wait (waiting and polling) run out after the given number of looks, or leave through the abort flag; the
+    time-out is reported once and the next one is reported again."""
+    q.qdit_sync(ctx)
+    for _ in range(2):
+        obs = torch.zeros(2, dtype=torch.int32, device="cuda")
+        q.qdit_selftest_wait_timeout(ctx, polls, obs)
+        assert q.lib.qdit_sync(ctx) == q.QDIT_ERR_TIMEOUT
+        assert obs.cpu().tolist() == [1, 1]
+        assert q.lib.qdit_sync(ctx) == q.QDIT_OK
 
 
 def test_vc_fit_rejects_bad_arguments(q, ctx):
