@@ -195,6 +195,21 @@ struct ChunkInputs {
 
 // (a warp whose 32 rows lie wholly past M, in a ragged last tile, has no sample: it loads nothing)
 template <int EPI>
+__device__ __forceinline__ void prefetch_chunk(const GemmParams& p, int n, int row_base, int rsub, float a_scale, ChunkInputs& in) {
+  const uint32_t flags = epi_flags<EPI>(p);
+  if (n < p.N && row_base < p.M && !(flags & QDIT_EPI_OUT_I32)) {
+    load_col_params<EPI>(p, n, row_base / p.tokens, a_scale, in.cp);
+    if (flags & QDIT_EPI_RESIDUAL) {
+#pragma unroll
+      for (int sidx = 0; sidx < 4; ++sidx) {
+        const int row = row_base + sidx * 8 + rsub;
+        if (row < p.M) in.res[sidx] = *reinterpret_cast<const uint4*>(p.residual + static_cast<int64_t>(row) * p.ldo + n);
+      }
+    }
+  }
+}
+// Its two parts, for what may be read at different times.
+template <int EPI>
 __device__ __forceinline__ void prefetch_params(const GemmParams& p, int n, int row_base, float a_scale, ChunkInputs& in) {
   if (n < p.N && row_base < p.M && !(epi_flags<EPI>(p) & QDIT_EPI_OUT_I32)) load_col_params<EPI>(p, n, row_base / p.tokens, a_scale, in.cp);
 }
@@ -213,9 +228,12 @@ __device__ __forceinline__ void prefetch_residual(const GemmParams& p, int n, in
 // `tacc` = TMEM address of the accumulator stage (lane 0 of the CTA, first column); `release()` hands the
 // stage back to the MMA issuer once this warp has read its share.  `stg` = this warp's 4 KB staging patch.
 // The epilogue is bound by the latency chain of one chunk (global loads, TMEM load, transpose, stores), so
-// the tile's chunks are spread over as many warps as the register file allows, and the global loads of a warp's first chunk
-// (`cur`) have been issued before the accumulator was waited for.
-template <int BN, int EPI, int SPLIT = EPI_SPLIT, typename Release>
+// the tile's chunks are spread over as many warps as the register file allows.  PREFETCH: the global loads of a warp's first chunk (`cur`) have
+// been issued before the accumulator was waited for; that is for launches of one tile per CTA, and for layers that load parameters only (classes 1 and
+// 2: 100 x 65536 x 1152 bf16 14.8 us, 15.4 without).  Otherwise the accumulator of a later tile is usually there, and all loads of a chunk go out
+// together beside its read: parameters and residual apart are waited for one after the other (us, ahead / together: gated, packed weights
+// 22203 x 4096 x 768 222 / 189, 4096 x 6912 x 384 69 / 62; one code per byte, 100 tokens per sample, 5480 x 3456 x 1536 42.5 / 40.2).
+template <int BN, int EPI, bool PREFETCH, int SPLIT = EPI_SPLIT, typename Release>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc, int m0, int n0, int quad, int half,
                                               uint32_t stg, int lane, float a_scale, float o_inv, ChunkInputs& cur, float& top, Release release) {
   const int cg = lane & 3;     // after the transpose: column group (8 columns) ...
@@ -240,10 +258,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc
     const int n = n0 + c * 32 + cg * 8;
     const bool col_ok = n < p.N;
     const uint32_t patch = stg;
-    if (c != half) {
-      prefetch_params<EPI>(p, n, row_base, a_scale, cur);
-      prefetch_residual<EPI>(p, n, row_base, rsub, cur);
-    }
+    if (!PREFETCH || c != half) prefetch_chunk<EPI>(p, n, row_base, rsub, a_scale, cur);
     uint32_t v[32];
     __syncwarp();
     tmem_ld_32x32(taddr + static_cast<uint32_t>(c * 32), v);

@@ -32,7 +32,8 @@ struct Cfg {
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + STAGING_BYTES + BAR_BYTES + 1024;  // + alignment slack
 };
 
-template <int BN, int EPI>
+// PREFETCH: see epilogue_tile
+template <int BN, int EPI, bool PREFETCH>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                const GemmParams p, const uint32_t idesc) {
@@ -168,32 +169,33 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     const int quad = warp & 3;   // TMEM lane quadrant this warp may access
     const int half = e >> 2;     // this warp takes chunks half, half + EPI_SPLIT, ...
     const uint32_t stg = smem_u32(staging + e * (32 * 128));  // [32 rows][8 x 16 B], 16-byte index XOR (row & 7)
-    if (!p.early_params) grid_dependency_wait();
+    if (!PREFETCH || !p.early_params) grid_dependency_wait();
+    if (!PREFETCH) grid_dependency_release();
     const float a_scale = device_value(p.a_scale_dev, p.a_scale);
     float o_inv = 0.0f;
     if (epi_flags<EPI>(p) & QDIT_EPI_QUANT_OUT) o_inv = __fdiv_rn(1.0f, device_value(p.o_scale_dev, p.o_scale));
     float top = 0.0f;
     int it = 0;
-    bool waited = !p.early_params;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++it) {
       const int as = it & 1;
       const uint32_t aphase = static_cast<uint32_t>(it >> 1) & 1u;
       const int m0 = (tile / p.num_n_tiles) * BM;
       const int n0 = (tile % p.num_n_tiles) * BN;
-      ChunkInputs cur;   // of this warp's first chunk
-      const int n = n0 + half * 32 + (lane & 3) * 8, row_base = m0 + quad * 32;
-      if (half < BN / 32) prefetch_params<EPI>(p, n, row_base, a_scale, cur);
-      if (!waited) {
-        grid_dependency_wait();
-        waited = true;
+      ChunkInputs cur;   // of this warp's chunk
+      if (PREFETCH) {
+        const int n = n0 + half * 32 + (lane & 3) * 8, row_base = m0 + quad * 32;
+        if (half < BN / 32) prefetch_params<EPI>(p, n, row_base, a_scale, cur);
+        if (it == 0) {
+          if (p.early_params) grid_dependency_wait();
+          grid_dependency_release();
+        }
+        if (half < BN / 32) prefetch_residual<EPI>(p, n, row_base, lane >> 2, cur);
       }
-      if (it == 0) grid_dependency_release();
-      if (half < BN / 32) prefetch_residual<EPI>(p, n, row_base, lane >> 2, cur);
       if (!mbar_wait(&tfull_bar[as], aphase, abort_flag, p.status)) break;
       __syncwarp();
       tc_fence_after();
       uint64_t* release_bar = &tempty_bar[as];
-      epilogue_tile<BN, EPI>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur, top,
+      epilogue_tile<BN, EPI, PREFETCH>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur, top,
                         [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
     __syncwarp();
@@ -208,21 +210,27 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   }
 }
 
-template <int BN, int EPI>
-int32_t launch_gemm_epi(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p, bool a_unsigned) {
+template <int BN, int EPI, bool PREFETCH>
+int32_t launch_tiles(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p, bool a_unsigned) {
   using C = Cfg<BN>;
-  QDIT_TRY(qdit_allow_smem(ctx, gemm_i8_kernel<BN, EPI>, C::SMEM_BYTES));
+  QDIT_TRY(qdit_allow_smem(ctx, gemm_i8_kernel<BN, EPI, PREFETCH>, C::SMEM_BYTES));
   CUtensorMap ta, tw;
   QDIT_TRY(qdit_get_tmap(ctx, A, p.M, p.K, p.K, BM, BK, 1, 1, &ta));
   QDIT_TRY(qdit_get_tmap(ctx, W, p.N, p.K, p.K, BN, BK, 1, 1, &tw));
-  p.num_m_tiles = (p.M + BM - 1) / BM;
-  p.num_n_tiles = (p.N + BN - 1) / BN;
   const int total = p.num_m_tiles * p.num_n_tiles;
   const int grid = total < ctx->num_sms ? total : ctx->num_sms;
   const uint32_t idesc = umma_idesc_i8(BM, BN, a_unsigned);
   ProfScope prof(ctx, QDIT_PROF_GEMM, 2.0 * p.M * static_cast<double>(p.N) * p.K);
-  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, gemm_i8_kernel<BN, EPI>, dim3(grid), dim3(NUM_THREADS), C::SMEM_BYTES, ta, tw, p, idesc));
+  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, gemm_i8_kernel<BN, EPI, PREFETCH>, dim3(grid), dim3(NUM_THREADS), C::SMEM_BYTES, ta, tw, p, idesc));
   return qdit_after_launch(ctx, "gemm_i8_kernel");
+}
+
+template <int BN, int EPI>
+int32_t launch_gemm_epi(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p, bool a_unsigned) {
+  p.num_m_tiles = (p.M + BM - 1) / BM;
+  p.num_n_tiles = (p.N + BN - 1) / BN;
+  if (EPI == 1 || EPI == 2 || p.num_m_tiles * p.num_n_tiles <= ctx->num_sms) return launch_tiles<BN, EPI, true>(ctx, A, W, p, a_unsigned);
+  return launch_tiles<BN, EPI, false>(ctx, A, W, p, a_unsigned);
 }
 
 template <int BN>

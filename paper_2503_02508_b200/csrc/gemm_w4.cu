@@ -41,7 +41,7 @@ struct W4Cfg {
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + W4_STAGING_BYTES + BAR_BYTES + 1024;
 };
 
-template <int EPI>
+template <int EPI, bool PREFETCH>   // PREFETCH: see epilogue_tile
 __global__ void __launch_bounds__(W4_THREADS, 1)
 gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_wp,
                const GemmParams p, const uint32_t idesc) {
@@ -207,15 +207,13 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
       const uint32_t aphase = static_cast<uint32_t>(it >> 1) & 1u;
       const int m0 = (tile % p.num_m_tiles) * BM;
       const int n0 = (tile / p.num_m_tiles) * BN;
-      ChunkInputs cur;   // of this warp's first chunk
-      const int n = n0 + half * 32 + (lane & 3) * 8, row_base = m0 + quad * 32;
-      prefetch_params<EPI>(p, n, row_base, a_scale, cur);
-      prefetch_residual<EPI>(p, n, row_base, lane >> 2, cur);
+      ChunkInputs cur;   // of this warp's chunk
+      if (PREFETCH) prefetch_chunk<EPI>(p, n0 + half * 32 + (lane & 3) * 8, m0 + quad * 32, lane >> 2, a_scale, cur);
       if (!mbar_wait(&tfull_bar[as], aphase, abort_flag, p.status)) break;
       __syncwarp();
       tc_fence_after();
       uint64_t* release_bar = &tempty_bar[as];
-      epilogue_tile<BN, EPI, W4_EPI_WARPS / 4>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur, top,
+      epilogue_tile<BN, EPI, PREFETCH, W4_EPI_WARPS / 4>(p, tmem_base + static_cast<uint32_t>(as * BN), m0, n0, quad, half, stg, lane, a_scale, o_inv, cur, top,
                              [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
     __syncwarp();
@@ -263,21 +261,27 @@ __global__ void __launch_bounds__(256) pack_w4_kernel(const int8_t* __restrict__
   if (bad) atomicExch(out_of_range, 1);
 }
 
-template <int EPI>
-int32_t launch_w4_epi(qdit_ctx* ctx, const void* A, const void* Wp, GemmParams& p, bool a_unsigned) {
+template <int EPI, bool PREFETCH>
+int32_t launch_w4_tiles(qdit_ctx* ctx, const void* A, const void* Wp, GemmParams& p, bool a_unsigned) {
   using C = W4Cfg;
-  QDIT_TRY(qdit_allow_smem(ctx, gemm_w4_kernel<EPI>, C::SMEM_BYTES));
+  QDIT_TRY(qdit_allow_smem(ctx, gemm_w4_kernel<EPI, PREFETCH>, C::SMEM_BYTES));
   CUtensorMap ta, tw;
   QDIT_TRY(qdit_get_tmap(ctx, A, p.M, p.K, p.K, BM, BK, 1, 1, &ta));
   QDIT_TRY(qdit_get_tmap(ctx, Wp, p.N, p.K / 2, p.K / 2, W4_BN, BK / 2, 0, 1, &tw));
-  p.num_m_tiles = (p.M + BM - 1) / BM;
-  p.num_n_tiles = (p.N + W4_BN - 1) / W4_BN;
   const int total = p.num_m_tiles * p.num_n_tiles;
   const int grid = total < ctx->num_sms ? total : ctx->num_sms;
   const uint32_t idesc = umma_idesc_i8(BM, W4_BN, a_unsigned);
   ProfScope prof(ctx, QDIT_PROF_GEMM, 2.0 * p.M * static_cast<double>(p.N) * p.K);
-  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, gemm_w4_kernel<EPI>, dim3(grid), dim3(W4_THREADS), C::SMEM_BYTES, ta, tw, p, idesc));
+  QDIT_CUDA_CHECK(ctx, qdit_launch_overlapped(ctx, gemm_w4_kernel<EPI, PREFETCH>, dim3(grid), dim3(W4_THREADS), C::SMEM_BYTES, ta, tw, p, idesc));
   return qdit_after_launch(ctx, "gemm_w4_kernel");
+}
+
+template <int EPI>
+int32_t launch_w4_epi(qdit_ctx* ctx, const void* A, const void* Wp, GemmParams& p, bool a_unsigned) {
+  p.num_m_tiles = (p.M + BM - 1) / BM;
+  p.num_n_tiles = (p.N + W4_BN - 1) / W4_BN;
+  if (EPI == 1 || EPI == 2 || p.num_m_tiles * p.num_n_tiles <= ctx->num_sms) return launch_w4_tiles<EPI, true>(ctx, A, Wp, p, a_unsigned);
+  return launch_w4_tiles<EPI, false>(ctx, A, Wp, p, a_unsigned);
 }
 
 }  // namespace

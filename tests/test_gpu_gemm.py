@@ -680,3 +680,44 @@ def test_codes_of_tiny_steps(q, ctx, step):
     assert (got[2].int().abs() > 0).float().mean() > 0.1
     for g in (got[0], got[1], got[3]):
         assert torch.equal(g, got[2])
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("M,tiles", [(128, 148), (128, 149), (90, 148), (300, 149), (300, 444), (300, 447)])
+@pytest.mark.parametrize("T", [100, 128])
+def test_gated_layer_with_as_many_tiles_as_ctas_and_more(q, ctx, bits, M, tiles, T):
+    """One tile per CTA (what the epilogue reads comes before the accumulator is complete) and more give the bits of tiles of 64 channels with
+    run-time flags; `tiles` of 192 channels, with packed weights of 128, samples that end inside a tile."""
+    width, K = (192, 256) if bits == 8 else (128, 256)
+    N = tiles // -(-M // 128) * width - 8
+    g = torch.Generator(device="cuda").manual_seed(M + tiles)
+    top = 127 if bits == 8 else 7
+    A = torch.randint(-127, 128, (M, K), generator=g, device="cuda", dtype=torch.int8)
+    W = torch.randint(-top, top + 1, (N, K), generator=g, device="cuda", dtype=torch.int8)
+    ws, bi = torch.rand(N, generator=g, device="cuda") * 2e-4 + 1e-5, torch.randn(N, generator=g, device="cuda") * 0.5
+    gate, resid = torch.randn((-(-M // T), N), generator=g, device="cuda"), torch.randn((M, N), generator=g, device="cuda").bfloat16()
+    packed = torch.empty((N, K // 2), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    if bits == 4:
+        q.qdit_pack_weight_int4(ctx, W, N, K, packed)
+    flags = q.QDIT_EPI_BIAS | q.QDIT_EPI_GATE | q.QDIT_EPI_RESIDUAL | q.QDIT_EPI_OUT_BF16 | q.QDIT_EPI_CACHE_STORE
+
+    def run(plain):
+        out, cache = (torch.full((M, N), 3.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        epi = q.epilogue(w_scale=ws, bias=bi, gate=gate, ld_gate=N, tokens_per_sample=T, residual=resid, cache_out=cache)
+        torch.cuda.synchronize()
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 64 if plain else 192)
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, int(plain))
+        try:
+            if bits == 4 and not plain:
+                q.qdit_w4a8_linear(ctx, A, packed, M, N, K, q.qparams(0.03), None, flags, epi, out, N, None)
+            else:
+                q.qdit_w8a8_linear(ctx, A, W, M, N, K, q.qparams(0.03), None, flags, epi, out, N)
+            q.qdit_sync(ctx)
+        finally:
+            q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 0)
+            q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, 0)
+        return out, cache
+
+    got, ref = run(False), run(True)
+    assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
