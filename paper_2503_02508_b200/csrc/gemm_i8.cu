@@ -199,7 +199,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                         [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
     __syncwarp();
-    if (EPI == 0 && p.absmax) publish_absmax(p.absmax, top);
+    if (EPI == 7) publish_absmax(p.absmax, top);
   }
 
   tc_fence_before();
@@ -235,11 +235,11 @@ int32_t launch_gemm_epi(qdit_ctx* ctx, const void* A, const void* W, GemmParams&
 
 template <int BN>
 int32_t launch_gemm(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p, bool a_unsigned) {
-  const int cls = ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE] ? 0 : epi_class(p.flags);
-  switch (cls) {
+  switch (epi_token_major(p, ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE] != 0)) {
     case 1: return launch_gemm_epi<BN, 1>(ctx, A, W, p, a_unsigned);
     case 2: return launch_gemm_epi<BN, 2>(ctx, A, W, p, a_unsigned);
     case 3: return launch_gemm_epi<BN, 3>(ctx, A, W, p, a_unsigned);
+    case 7: return launch_gemm_epi<BN, 7>(ctx, A, W, p, a_unsigned);
     default: return launch_gemm_epi<BN, 0>(ctx, A, W, p, a_unsigned);
   }
 }
@@ -327,6 +327,7 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
   p.early = early;
   p.early_params = early_params;
   p.absmax = absmax;
+  if (absmax && epi_class(flags) != 7) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "the largest magnitude is found behind bias and GELU with f32 output only");
   if (!(flags & QDIT_EPI_OUT_I32)) {
     if (!epi || !epi->w_scale) return qdit_fail(ctx, QDIT_ERR_INVALID_ARG, "epilogue with w_scale is required");
     if (!aligned16(epi->w_scale)) return qdit_fail(ctx, QDIT_ERR_ALIGN, "w_scale must be 16-byte aligned");

@@ -276,7 +276,7 @@ gemm_i8_sk_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
       if (row < p.M && n < p.N) epilogue8<EPI>(p, lo, hi, cp, res, row, n, o_inv, top);
     }
     __syncwarp();
-    if (EPI == 0 && p.absmax) publish_absmax(p.absmax, top);
+    if (EPI == 7) publish_absmax(p.absmax, top);
   }
   if (*abort_flag && warp == 0) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);  // let copies in flight land before shared memory goes away
@@ -307,10 +307,11 @@ int32_t launch_sk_epi(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p
 
 template <int S, bool W4>
 int32_t launch_sk(qdit_ctx* ctx, const void* A, const void* W, GemmParams& p, bool a_unsigned) {
-  switch (ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE] ? 0 : epi_class(p.flags)) {
+  switch (epi_token_major(p, ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE] != 0)) {
     case 1: return launch_sk_epi<S, 1, W4>(ctx, A, W, p, a_unsigned);
     case 2: return launch_sk_epi<S, 2, W4>(ctx, A, W, p, a_unsigned);
     case 3: return launch_sk_epi<S, 3, W4>(ctx, A, W, p, a_unsigned);
+    case 7: return launch_sk_epi<S, 7, W4>(ctx, A, W, p, a_unsigned);
     default: return launch_sk_epi<S, 0, W4>(ctx, A, W, p, a_unsigned);
   }
 }

@@ -217,7 +217,7 @@ gemm_w4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                              [release_bar]() { mbar_arrive_relaxed(release_bar); });
     }
     __syncwarp();
-    if (EPI == 0 && p.absmax) publish_absmax(p.absmax, top);
+    if (EPI == 7) publish_absmax(p.absmax, top);
   }
 
   tc_fence_before();
@@ -287,10 +287,11 @@ int32_t launch_w4_epi(qdit_ctx* ctx, const void* A, const void* Wp, GemmParams& 
 }  // namespace
 
 int32_t qdit_launch_gemm_w4(qdit_ctx* ctx, const void* A, const void* Wp, qgemm::GemmParams& p, bool a_unsigned) {
-  switch (ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE] ? 0 : epi_class(p.flags)) {
+  switch (epi_token_major(p, ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE] != 0)) {
     case 1: return launch_w4_epi<1>(ctx, A, Wp, p, a_unsigned);
     case 2: return launch_w4_epi<2>(ctx, A, Wp, p, a_unsigned);
     case 3: return launch_w4_epi<3>(ctx, A, Wp, p, a_unsigned);
+    case 7: return launch_w4_epi<7>(ctx, A, Wp, p, a_unsigned);
     default: return launch_w4_epi<0>(ctx, A, Wp, p, a_unsigned);
   }
 }
