@@ -426,13 +426,16 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
       const double products = (p.K + BK - 1) / BK * 620.0 + 600.0, tile = cls == 3 && products < 4750.0 ? 4750.0 : products;
       const double cost = static_cast<double>(waves) * tile + 4500.0;
       // (a pair's start beyond that of a single CTA; with one wave nothing hides it.  Channel-major / pairs, bf16: 1024 x 4608 x 2048 9.1 / 10.5 us, 2048 x
-      // 2304 x 3072 11.4 / 12.8, 1301 x 3456 x 512 6.5 / 7.4, but 1536 x 6912 x 768 13.8 / 12.0; gated: 4096 x 1152 x 1152 9.8 / 10.9)
+      // 2304 x 3072 11.4 / 12.8, 1301 x 3456 x 512 6.5 / 7.4, but 1536 x 6912 x 768 13.8 / 12.0; gated: 4096 x 1152 x 1152 9.8 / 10.9.)
+      // (a zero point costs a gated pair's epilogue 8 to 15 %, whose registers hold nothing ahead; a channel-major thread has one channel: 8192 x 3456 x 1152
+      // 39.8 / 44.5, 2048 x 4096 x 1024 13.0 / 14.1, but 6144 x 1152 x 3072 21.9 / 18.2)
+      const double pairs = qdit_gemm_pair_cost(ctx, p) * (cls == 3 && p.a_zp != 0 ? 1.15 : 1.0);
       const double spare = cls == 3 ? (waves == 1 ? 3000.0 : 0.0) : cls != 1 || one_wave ? 1500.0 : waves == 1 ? 3000.0 : 2500.0;
       // (f32 output: with one wave, and with reductions short enough that the output's own time counts: a tile's 128 channels are whole 512-byte
       // pieces of a row there, which memory takes at 5.4 TB/s, where a pair's 128-byte pieces reach 3.4; us, channel-major / pairs: 10000 x
       // 20480 x 64 151 / 242, 6144 x 20480 x 384 98 / 152, 8192 x 6912 x 384 44 / 53, 4096 x 30720 x 768 127 / 169, 1728 x 4608 x 256 8.8 /
       // 9.8; but 3072 x 3456 x 768 14.1 / 12.2, 5000 x 4608 x 768 29.8 / 26, 8192 x 3456 x 1152 36.9 / 33.9, where its epilogue is the longer part of a tile)
-      if (cls == 6 ? waves == 1 || p.K <= (p.N >= 6144 ? 768 : 384) : cost <= qdit_gemm_pair_cost(ctx, p) + spare) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
+      if (cls == 6 ? waves == 1 || p.K <= (p.N >= 6144 ? 768 : 384) : cost <= pairs + spare) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
     }
     // (at most 128 rows: half of a pair's tokens would be padding; single CTAs / pairs: 1 x 193536 x 128 codes 18.8 / 44.4 us, 33 x 193536 x 384 22.5 / 42.7,
     // 100 x 65536 x 768 codes 14.9 / 19.0; from 129 rows on 160 x 193536 x 384 codes 63.7 / 46.2, 200 x 30720 x 3072 40 / 26.5)

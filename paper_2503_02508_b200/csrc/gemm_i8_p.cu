@@ -45,7 +45,7 @@ struct PCfg {
   // two of them, used in turn; gated: each receives the residual of a chunk and is overwritten by its output, a third one takes the
   // cache copy
   static constexpr int STAGING_PER_WARP = (GATED ? 3 : 2) * TILE_BYTES;
-  static constexpr int PARAM_BYTES = CODES ? EPI_WARPS * 256 : 0;        // per warp [scale, bias][channel of a chunk]
+  static constexpr int PARAM_BYTES = CODES ? EPI_WARPS * 384 : 0;        // per warp [scale, bias, zero-point term][channel of a chunk]
   static constexpr int BAR_BYTES = 512;
   static constexpr int EXTRA_BYTES = EPI_WARPS * STAGING_PER_WARP + PARAM_BYTES + BAR_BYTES + 1024;
   static constexpr int SMEM_BYTES = 232448;              // what the other parts leave holds the stages: 5 or 6 of 256 channels, more of fewer
@@ -355,8 +355,9 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
       const uint32_t row_addr = tile0 + static_cast<uint32_t>(lane) * 32u, sw = (static_cast<uint32_t>(lane) >> 2 & 1u) << 4;
       // Parameters of a chunk's channels: a lane holds those of one channel, fetched one chunk ahead, and hands them to its warp
       // through shared memory (no barrier between warps: they drift apart, and one's exponentials run beside another's loads)
-      float* const sc = params + e * 64;
+      float* const sc = params + e * 96;
       float* const bi = sc + 32;
+      int* const zt = reinterpret_cast<int*>(sc + 64);
       float sc_next = 0.0f, bi_next = 0.0f;
       auto fetch = [&](const Tile& t, int c) {
         const int n = n_of(t) + c * 32 + lane;
@@ -388,6 +389,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           __syncwarp();   // the last chunk's parameters have been read
           sc[lane] = __fmul_rn(a_scale, sc_next);
           bi[lane] = bi_next;
+          if (p.a_zp != 0) zt[lane] = n0 + c * 32 + lane < p.N ? p.a_zp * p.w_colsum[n0 + c * 32 + lane] : 0;
           __syncwarp();
           if (c + C::SPLIT < chunks) {
             fetch(t, c + C::SPLIT);
@@ -401,8 +403,13 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           if (!live) continue;
           if (p.a_zp != 0) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (n0 + c * 32 + j < p.N) v[j] -= static_cast<uint32_t>(p.a_zp * __ldg(p.w_colsum + n0 + c * 32 + j));
+            for (int j = 0; j < 8; ++j) {
+              const int4 z = *reinterpret_cast<const int4*>(zt + 4 * j);
+              v[4 * j] -= static_cast<uint32_t>(z.x);
+              v[4 * j + 1] -= static_cast<uint32_t>(z.y);
+              v[4 * j + 2] -= static_cast<uint32_t>(z.z);
+              v[4 * j + 3] -= static_cast<uint32_t>(z.w);
+            }
           }
           uint32_t w[8];
 #pragma unroll
@@ -484,6 +491,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           uint32_t a[16], b[16];
           // parameters of this thread's channels n0 + 8k + 2(lane%4), + 1 (past N: those of the last pair, whose results are not stored)
           float2 sc[4], bi[4], gate[4];
+          int2 zt[4];   // zero-point terms
           bool landed = false;   // a look at the residual's barrier, whose phase has usually ended by now
           auto channel = [&](int k) {
             const int n = n0 + 8 * k + 2 * (lane & 3);
@@ -499,6 +507,10 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             }
             tmem_ld_16x256b_x4(taddr + static_cast<uint32_t>(c * 32), a);
             tmem_ld_16x256b_x4(taddr + (16u << 16) + static_cast<uint32_t>(c * 32), b);
+            if (!C::GATED && p.a_zp != 0) {   // (while the accumulator comes; the gated layers have no registers left for it)
+#pragma unroll
+              for (int k = 0; k < 4; ++k) zt[k] = *reinterpret_cast<const int2*>(p.w_colsum + channel(k));
+            }
             tmem_ld_wait();
           }
           if (c == c_last) release(as);
@@ -506,13 +518,14 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           if (p.a_zp != 0) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const int2 z = *reinterpret_cast<const int2*>(p.w_colsum + channel(k));
+              if (C::GATED) zt[k] = *reinterpret_cast<const int2*>(p.w_colsum + channel(k));
+              const uint32_t z0 = static_cast<uint32_t>(p.a_zp * zt[k].x), z1 = static_cast<uint32_t>(p.a_zp * zt[k].y);
 #pragma unroll
               for (int i = 0; i < 4; i += 2) {
-                a[4 * k + i] -= static_cast<uint32_t>(p.a_zp * z.x);
-                a[4 * k + i + 1] -= static_cast<uint32_t>(p.a_zp * z.y);
-                b[4 * k + i] -= static_cast<uint32_t>(p.a_zp * z.x);
-                b[4 * k + i + 1] -= static_cast<uint32_t>(p.a_zp * z.y);
+                a[4 * k + i] -= z0;
+                a[4 * k + i + 1] -= z1;
+                b[4 * k + i] -= z0;
+                b[4 * k + i + 1] -= z1;
               }
             }
           }

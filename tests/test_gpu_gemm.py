@@ -721,3 +721,36 @@ def test_gated_layer_with_as_many_tiles_as_ctas_and_more(q, ctx, bits, M, tiles,
 
     got, ref = run(False), run(True)
     assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("kind", ["codes", "f32", "gelu_f32", "bf16", "gated"])
+@pytest.mark.parametrize("M,N,K,zp", [(2304, 3472, 320, 7), (1300, 4624, 784, 255), (600, 12304, 128, 128), (1300, 4624, 784, 0)])
+def test_many_rows_with_a_zero_point(q, ctx, kind, M, N, K, zp):
+    """Unsigned activations with a zero point through the automatic choice (pairs of CTAs, channel-major tiles; ragged in both directions): the bits of
+    tiles of 64 channels with run-time flags.  The weights' sums are distinct, so that a channel with another one's term shows."""
+    T = 32
+    g = torch.Generator(device="cuda").manual_seed(M + N + zp)
+    A = torch.randint(0, 256, (M, K), generator=g, device="cuda").to(torch.uint8)
+    W = torch.randint(-127, 128, (N, K), generator=g, device="cuda", dtype=torch.int8)
+    colsum = W.sum(dim=1, dtype=torch.int32)
+    ws, bi = torch.rand(N, generator=g, device="cuda") * 2e-4 + 1e-5, torch.randn(N, generator=g, device="cuda") * 0.5
+    gate, resid = torch.randn((-(-M // T), N), generator=g, device="cuda"), torch.randn((M, N), generator=g, device="cuda").bfloat16()
+    flags = q.QDIT_EPI_BIAS | {"codes": q.QDIT_EPI_GELU | q.QDIT_EPI_QUANT_OUT, "f32": q.QDIT_EPI_OUT_F32, "gelu_f32": q.QDIT_EPI_GELU | q.QDIT_EPI_OUT_F32,
+                               "bf16": q.QDIT_EPI_OUT_BF16, "gated": q.QDIT_EPI_GATE | q.QDIT_EPI_RESIDUAL | q.QDIT_EPI_OUT_BF16}[kind]
+    dtype = {"codes": torch.int8, "f32": torch.float32, "gelu_f32": torch.float32}.get(kind, torch.bfloat16)
+
+    def run(plain):
+        out = torch.full((M, N), 3, dtype=dtype, device="cuda")
+        epi = q.epilogue(w_scale=ws, w_colsum=colsum, bias=bi, gate=gate, ld_gate=N, tokens_per_sample=T, residual=resid, out_qp=q.qparams(0.02))
+        torch.cuda.synchronize()
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 64 * plain)
+        q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, plain)
+        try:
+            q.qdit_w8a8_linear(ctx, A, W, M, N, K, q.qparams(0.03, zp, 0, 255), None, flags, epi, out, N)
+            q.qdit_sync(ctx)
+        finally:
+            q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_BN, 0)
+            q.qdit_set_option(ctx, q.QDIT_OPT_GEMM_GENERIC_EPILOGUE, 0)
+        return out
+
+    assert torch.equal(run(0), run(1))
