@@ -680,8 +680,9 @@ int32_t launch_p_epi(qdit_ctx* ctx, const void* A, const void* W, const GemmPara
 
 // Channels per tile: the least of waves x (time of a tile) + the last tile's epilogue, in clocks.  A k-block takes 200 + 1.22 BN (512 with 256
 // channels: the tensor core's own time; 434 with 192: the fill and the operand reads of shared memory), a tile 600 more; an epilogue
-// takes `chunk` for 32 channels and bounds the tile where that is longer; codes no less than what three chunks take (four warps
-// share a lane quadrant: tiles of 64 channels leave half of them idle, 640 x 9728 x 512 13.4 us, 10.6 token-major).  A narrower tile has to be
+// takes `chunk` for 32 channels and bounds the tile where that is longer; codes no less than what four chunks take, and from five on what six and a half
+// do (four warps share a lane quadrant and take a chunk each: 640 x 9728 x 512 13.4 us with 64 channels, 10.6 token-major; 2048 x 4096 x 768 15.3 / 13.0 / 12.2 / 13.7 /
+// 13.9 / 14.6 / 12.5 with 64 / 96 / 128 / 160 / 192 / 224 / 256).  A narrower tile has to be
 // 4 % better: it reads the tokens more often (fc2 at 65536 rows: 256 us with 256 channels, 316 with 192, which this estimate puts level).
 // Measured: 8192 x 3456 x 1152 24.4 / 24.0 / 24.0 us with 256 / 224 / 192 channels, 2048 rows 10.1 / 9.7 / 9.0; 8192 x 1152 x 4608 40.5 with
 // 256, 34.8 with 192, 36.5 with 128; 1024 x 4608 x 1152 10.1 with 256, 9.4 with 128.
@@ -692,13 +693,13 @@ struct PairTile {
 PairTile pick_pair_tile(const GemmParams& p, int pairs) {
   const int cls = epi_class(p.flags);
   const int chunk = cls == 1 ? 540 : cls == 2 ? 770 : cls == 3 ? (p.K < SHORT_K ? 650 : 950) : cls == 5 ? 560 : cls == 6 ? 650 : 1000;
-  const int least = cls == 2 ? 3 : 1;   // chunks
   const int64_t mt = (p.M + 255) / 256;
   const double num_kb = (p.K + BK - 1) / BK;
   PairTile best{256, 1e30};
   for (int bn = 256; bn >= 64; bn -= 32) {
     const int64_t waves = (mt * ((p.N + bn - 1) / bn) + pairs - 1) / pairs;
-    const double main = num_kb * (200.0 + 1.22 * bn), epilogue = chunk * (bn / 32 < least ? least : bn / 32);
+    const int n = bn / 32;
+    const double main = num_kb * (200.0 + 1.22 * bn), epilogue = chunk * (cls != 2 || n >= 7 ? n : n <= 4 ? 4.0 : 6.5);
     const double cost = static_cast<double>(waves) * ((main > epilogue ? main : epilogue) + 600.0) + epilogue;
     if (cost < best.cost * 0.96) best = PairTile{bn, cost};
   }
