@@ -27,6 +27,9 @@ def _flags(q, kind):
     # f32 output of many rows: channel-major where the output's own time counts
     ("f32", 2304, 6144, 768, CHANNEL_MAJOR), ("f32", 2304, 6144, 784, PAIRS), ("f32", 1023, 6144, 128, PAIRS),
     ("f32", 3072, 4616, 384, CHANNEL_MAJOR), ("f32", 3072, 4616, 400, PAIRS),
+    ("f32", 4096, 12288, 1024, CHANNEL_MAJOR), ("f32", 4096, 12280, 1024, PAIRS), ("f32", 1152, 16384, 1152, CHANNEL_MAJOR), ("f32", 1152, 16376, 1152, PAIRS),
+    ("f32", 1152, 43688, 1152, CHANNEL_MAJOR), ("f32", 1152, 43696, 1152, PAIRS), ("f32", 2048, 4096, 768, CHANNEL_MAJOR), ("f32", 2048, 4096, 1024, PAIRS),
+    ("f32", 1792, 4608, 448, CHANNEL_MAJOR), ("f32", 1792, 4480, 448, PAIRS),
 ])
 def test_route(kind, M, N, K, kernel):
     import paper_2503_02508_b200 as q
