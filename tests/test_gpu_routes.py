@@ -23,7 +23,7 @@ def _flags(q, kind):
     ("f32", 4, 49152, 752, TOKEN_MAJOR), ("f32", 3, 49152, 768, ROWS), ("f32", 2, 49152, 128, ROWS), ("f32", 3, 16392, 96, TOKEN_MAJOR),
     ("f32", 3, 16392, 80, ROWS), ("f32", 4, 20480, 384, ROWS), ("f32", 4, 16384, 128, ROWS),
     # bf16 output of one wave of channel-major tiles
-    ("bf16", 1024, 4608, 2048, CHANNEL_MAJOR), ("bf16", 1301, 3456, 512, CHANNEL_MAJOR), ("bf16", 1536, 6912, 768, PAIRS), ("bf16", 1024, 2304, 2048, TOKEN_MAJOR),
+    ("bf16", 1426, 3072, 4608, CHANNEL_MAJOR), ("bf16", 1024, 4608, 2048, CHANNEL_MAJOR), ("bf16", 1301, 3456, 512, CHANNEL_MAJOR), ("bf16", 1536, 6912, 768, PAIRS), ("bf16", 1024, 2304, 2048, TOKEN_MAJOR),
     # f32 output of many rows: channel-major where the output's own time counts
     ("f32", 2304, 6144, 768, CHANNEL_MAJOR), ("f32", 2304, 6144, 784, PAIRS), ("f32", 1023, 6144, 128, PAIRS),
     ("f32", 3072, 4616, 384, CHANNEL_MAJOR), ("f32", 3072, 4616, 400, PAIRS),
