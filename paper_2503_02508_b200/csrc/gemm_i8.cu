@@ -428,20 +428,20 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
       // (a pair's start beyond that of a single CTA; with one wave nothing hides it.  Channel-major / pairs, bf16: 1024 x 4608 x 2048 9.1 / 10.5 us, 2048 x
       // 2304 x 3072 11.4 / 12.8, 1301 x 3456 x 512 6.5 / 7.4, but 1536 x 6912 x 768 13.8 / 12.0; gated: 4096 x 1152 x 1152 9.8 / 10.9.  Nor does a pair's k-block take less than a single
       // CTA's then: 1426 x 3072 x 4608 15.0 / 16.2, per-token scales 1024 x 4096 x 3072 12.2 / 13.0, 1024 x 4608 x 4096 14.5 / 15.6)
-      // (a zero point costs a gated pair's epilogue 8 to 15 %, whose registers hold nothing ahead; a channel-major thread has one channel: 8192 x 3456 x 1152
-      // 39.8 / 44.5, 2048 x 4096 x 1024 13.0 / 14.1, but 6144 x 1152 x 3072 21.9 / 18.2)
-      const double pairs = qdit_gemm_pair_cost(ctx, p) * (cls == 3 && p.a_zp != 0 ? 1.15 : 1.0);
+      // (a zero point costs a gated pair's epilogue up to 10 %, whose registers hold nothing ahead; a channel-major thread has one channel: 8192 x 3456 x 1152
+      // 39.8 / 44.5, 2048 x 4096 x 1024 13.0 / 14.1, but 4096 x 4608 x 1488 40.5 / 32.8, 6144 x 1152 x 3072 21.9 / 18.2)
+      const double pairs = qdit_gemm_pair_cost(ctx, p) * (cls == 3 && p.a_zp != 0 ? 1.05 : 1.0);
       const double spare = cls == 3 ? (waves == 1 ? 3000.0 : 0.0) : cls != 1 || one_wave ? 1500.0 : waves == 1 ? 3000.0 : 2500.0;
       const double first = waves == 1 ? (p.K + BK - 1) / BK * 110.0 : 0.0;
       // (f32 output: with one wave, with two or three that are almost full, and with reductions short enough that the output's own time counts: a tile's 128
       // channels are whole 512-byte pieces of a row there, which memory takes at 5.4 TB/s, where a pair's 128-byte pieces reach 3.4; us, channel-major /
       // pairs: 10000 x 20480 x 64 151 / 242, 6144 x 20480 x 384 98 / 152, 8192 x 6912 x 384 44 / 53, 4096 x 30720 x 768 127 / 169, 4611 x 15448 x 1024
-      // 83 / 94, 2048 x 30720 x 1152 78 / 86, 1728 x 4608 x 256 8.8 / 9.8, 2048 x 4096 x 768 11.0 / 12.0, 3072 x 4096 x 768 14.7 / 16.2; but 3072 x 3456 x 768 14.1 / 12.2, 5000 x 4608 x
+      // 83 / 94, 8192 x 9216 x 1024 88 / 95, 2048 x 30720 x 1152 78 / 86, 1728 x 4608 x 256 8.8 / 9.8, 2048 x 4096 x 768 11.0 / 12.0, 3072 x 4096 x 768 14.7 / 16.2; but 3072 x 3456 x 768 14.1 / 12.2, 5000 x 4608 x
       // 768 29.8 / 26, 8192 x 3456 x 1152 38.5 / 34.8, and 1600 x 98304 x 1152, whose weights a pair reads once, 243 / 194)
       const bool wide = static_cast<int64_t>(p.N) * p.K <= (48 << 20);   // (weights that stay in L2)
-      const int short_k = wide && p.N >= 16384 ? 1152 : wide && p.N >= 12288 ? 1024 : p.N >= 6144 ? 768 : 384;
+      const int short_k = wide && p.N >= 16384 ? 1152 : wide && p.N >= 9216 ? 1024 : p.N >= 6144 ? 768 : 384;
       const bool full = waves <= 3 && static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) * 20 >= 17 * waves * ctx->num_sms;
-      const bool f32 = cls == 6 && (waves == 1 || p.K <= short_k || (full && cost <= 0.9 * pairs));
+      const bool f32 = cls == 6 && (waves == 1 || p.K <= short_k || (full && p.K <= 768 && cost <= 0.9 * pairs));
       if (f32 || (cls != 6 && cost <= pairs + spare + first)) return qdit_launch_gemm_t(ctx, A, W, p, a_unsigned, 256);
     }
     // (at most 128 rows: half of a pair's tokens would be padding; single CTAs / pairs: 1 x 193536 x 128 codes 18.8 / 44.4 us, 33 x 193536 x 384 22.5 / 42.7,

@@ -682,7 +682,8 @@ int32_t launch_p_epi(qdit_ctx* ctx, const void* A, const void* W, const GemmPara
 // channels: the tensor core's own time; 434 with 192: the fill and the operand reads of shared memory), a tile 600 more; an epilogue
 // takes `chunk` for 32 channels and bounds the tile where that is longer; codes no less than what four chunks take, and from five on what six and a half
 // do (four warps share a lane quadrant and take a chunk each: 640 x 9728 x 512 13.4 us with 64 channels, 10.6 token-major; 2048 x 4096 x 768 15.3 / 13.0 / 12.2 / 13.7 /
-// 13.9 / 14.6 / 12.5 with 64 / 96 / 128 / 160 / 192 / 224 / 256).  A narrower tile has to be
+// 13.9 / 14.6 / 12.5 with 64 / 96 / 128 / 160 / 192 / 224 / 256); with the three warps of short gated reductions three, and five and a third for four or five chunks (8192
+// x 768 x 384 11.7 / 9.9 / 10.9 / 11.1 / 9.6 / 10.9 / 11.1).  A narrower tile has to be
 // 4 % better: it reads the tokens more often (fc2 at 65536 rows: 256 us with 256 channels, 316 with 192, which this estimate puts level).
 // Measured: 8192 x 3456 x 1152 24.4 / 24.0 / 24.0 us with 256 / 224 / 192 channels, 2048 rows 10.1 / 9.7 / 9.0; 8192 x 1152 x 4608 40.5 with
 // 256, 34.8 with 192, 36.5 with 128; 1024 x 4608 x 1152 10.1 with 256, 9.4 with 128.
@@ -696,10 +697,12 @@ PairTile pick_pair_tile(const GemmParams& p, int pairs) {
   const int64_t mt = (p.M + 255) / 256;
   const double num_kb = (p.K + BK - 1) / BK;
   PairTile best{256, 1e30};
-  for (int bn = 256; bn >= 64; bn -= 32) {
+  const int widest = p.N > 224 ? 256 : p.N <= 64 ? 64 : (p.N + 31) / 32 * 32;
+  for (int bn = widest; bn >= 64; bn -= 32) {
     const int64_t waves = (mt * ((p.N + bn - 1) / bn) + pairs - 1) / pairs;
     const int n = bn / 32;
-    const double main = num_kb * (200.0 + 1.22 * bn), epilogue = chunk * (cls != 2 || n >= 7 ? n : n <= 4 ? 4.0 : 6.5);
+    const double taken = cls == 2 ? (n <= 4 ? 4.0 : n < 7 ? 6.5 : n) : cls == 3 && p.K < SHORT_K ? (n <= 3 ? 3.0 : n < 6 ? 5.3 : n) : n;   // chunks, in time
+    const double main = num_kb * (200.0 + 1.22 * bn), epilogue = chunk * taken;
     const double cost = static_cast<double>(waves) * ((main > epilogue ? main : epilogue) + 600.0) + epilogue;
     if (cost < best.cost * 0.96) best = PairTile{bn, cost};
   }

@@ -26,8 +26,8 @@ def _flags(q, kind):
     ("bf16", 1426, 3072, 4608, CHANNEL_MAJOR), ("bf16", 1024, 4608, 2048, CHANNEL_MAJOR), ("bf16", 1301, 3456, 512, CHANNEL_MAJOR), ("bf16", 1536, 6912, 768, PAIRS), ("bf16", 1024, 2304, 2048, TOKEN_MAJOR),
     # f32 output of many rows: channel-major where the output's own time counts
     ("f32", 2304, 6144, 768, CHANNEL_MAJOR), ("f32", 2304, 6144, 784, PAIRS), ("f32", 1023, 6144, 128, PAIRS),
-    ("f32", 3072, 4616, 384, CHANNEL_MAJOR), ("f32", 3072, 4616, 400, PAIRS),
-    ("f32", 4096, 12288, 1024, CHANNEL_MAJOR), ("f32", 4096, 12280, 1024, PAIRS), ("f32", 1152, 16384, 1152, CHANNEL_MAJOR), ("f32", 1152, 16376, 1152, PAIRS),
+    ("f32", 2560, 4616, 384, CHANNEL_MAJOR), ("f32", 2560, 4616, 400, PAIRS), ("f32", 3072, 4616, 400, CHANNEL_MAJOR),
+    ("f32", 4096, 9216, 1024, CHANNEL_MAJOR), ("f32", 4096, 9208, 1024, PAIRS), ("f32", 1152, 16384, 1152, CHANNEL_MAJOR), ("f32", 1152, 16376, 1152, PAIRS),
     ("f32", 1152, 43688, 1152, CHANNEL_MAJOR), ("f32", 1152, 43696, 1152, PAIRS), ("f32", 2048, 4096, 768, CHANNEL_MAJOR), ("f32", 2048, 4096, 1024, PAIRS),
     ("f32", 1792, 4608, 448, CHANNEL_MAJOR), ("f32", 1792, 4480, 448, PAIRS),
 ])
