@@ -375,12 +375,12 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
       p.o_qmax = static_cast<float>(epi->out_qp.qmax);
     }
   }
-  // One to four rows, f32 output (the modulation of as many images): the weights are streamed past the rows instead of through the
-  // tensor core (us, 1 and 4 rows, tensor core / streamed: 193536 x 1152 51.2 / 35.1 and 51.4 / 45.4, packed 4-bit weights 73.0 / 22.1 and
-  // 75.9 / 47.7; 6912 x 1152 7.0 / 2.8 and 7.0 / 4.2; 1152 x 4608 7.1 / 4.1 and 7.2 / 5.7; 1152 x 384 3.4 / 2.2 and 3.3 / 2.6).  Beyond
-  // four the dot products take longer than the weights; with three and four rows they do so for many channels of a short reduction too
-  // (tensor core / streamed: 193536 x 128 17.6 / 28.1, 65536 x 384 10.7 / 12.2, 24576 x 256 5.1 / 5.7; packed 193536 x 64 25.2 /
-  // 30.7, 65536 x 384 12.9 / 14.5; but 65536 x 768 13.5 / 13.7 and x 1024 17.0 / 15.1, 30720 x 384 7.8 / 6.6, 30720 x 32 7.3 / 6.1, packed 65536 x 512 14.4 / 12.9, 65536 x 32 12.3 / 11.2).
+  // One to four rows, f32 output (the modulation of as many images): the weights are streamed past the rows instead of through the tensor core (us, 1
+  // and 4 rows, tensor core / streamed: 193536 x 1152 51.2 / 35.1 and 51.4 / 45.4, packed 4-bit weights 73.0 / 22.1 and 75.9 / 47.7; 6912 x 1152 7.0 /
+  // 2.8 and 7.0 / 4.2; 1152 x 4608 7.1 / 4.1 and 7.2 / 5.7; 1152 x 384 3.4 / 2.2 and 3.3 / 2.6).  Beyond four the dot products take longer than the
+  // weights; with three and four rows they do so for many channels of a short reduction too (tensor core / streamed: 193536 x 128 17.6 / 28.1, 65536 x
+  // 384 10.7 / 12.2, 24576 x 256 5.1 / 5.7; packed 193536 x 64 25.2 / 30.7, 65536 x 384 12.9 / 14.5; but 65536 x 768 13.5 / 13.7 and x 1024 17.0 /
+  // 15.1, 30720 x 384 7.8 / 6.6, 30720 x 32 7.3 / 6.1, packed 65536 x 512 14.4 / 12.9, 65536 x 32 12.3 / 11.2).
   const bool many_short = p.M > 2 && (p.N >= 49152 ? (packed4 ? p.K >= 64 && p.K < 512 : p.K < 768) : p.N > 16384 && !packed4 && p.K >= 96 && p.K < 384);
   if (epi_class(p.flags) == 6 && p.M <= FEW_ROWS && !p.absmax && !many_short && p.K <= FEW_ROWS_K && ctx->opt[QDIT_OPT_GEMM_BN] == 0 && ctx->opt[QDIT_OPT_GEMM_T] == 0 &&
       !ctx->opt[QDIT_OPT_GEMM_GENERIC_EPILOGUE])
@@ -425,19 +425,21 @@ int32_t qdit_linear_impl(qdit_ctx* ctx, const void* A, const void* W, int64_t M,
       // 4608 x 384 41.6 / 43.5)
       const double products = (p.K + BK - 1) / BK * 620.0 + 600.0, tile = cls == 3 && products < 4750.0 ? 4750.0 : products;
       const double cost = static_cast<double>(waves) * tile + 4500.0;
-      // (a pair's start beyond that of a single CTA; with one wave nothing hides it.  Channel-major / pairs, bf16: 1024 x 4608 x 2048 9.1 / 10.5 us, 2048 x
-      // 2304 x 3072 11.4 / 12.8, 1301 x 3456 x 512 6.5 / 7.4, but 1536 x 6912 x 768 13.8 / 12.0; gated: 4096 x 1152 x 1152 9.8 / 10.9.  Nor does a pair's k-block take less than a single
-      // CTA's then: 1426 x 3072 x 4608 15.0 / 16.2, per-token scales 1024 x 4096 x 3072 12.2 / 13.0, 1024 x 4608 x 4096 14.5 / 15.6)
-      // (a zero point costs a gated pair's epilogue up to 10 %, whose registers hold nothing ahead; a channel-major thread has one channel: 8192 x 3456 x 1152
-      // 39.8 / 44.5, 2048 x 4096 x 1024 13.0 / 14.1, but 4096 x 4608 x 1488 40.5 / 32.8, 6144 x 1152 x 3072 21.9 / 18.2)
+      // (a pair's start beyond that of a single CTA; with one wave nothing hides it.  Channel-major / pairs, bf16: 1024 x 4608 x 2048 9.1 / 10.5 us,
+      // 2048 x 2304 x 3072 11.4 / 12.8, 1301 x 3456 x 512 6.5 / 7.4, but 1536 x 6912 x 768 13.8 / 12.0; gated: 4096 x 1152 x 1152 9.8 / 10.9.  Nor does
+      // a pair's k-block take less than a single CTA's then: 1426 x 3072 x 4608 15.0 / 16.2, per-token scales 1024 x 4096 x 3072 12.2 / 13.0, 1024 x
+      // 4608 x 4096 14.5 / 15.6)
+      // (a zero point costs a gated pair's epilogue up to 10 %, whose registers hold nothing ahead; a channel-major thread has one channel: 8192 x 3456
+      // x 1152 39.8 / 44.5, 2048 x 4096 x 1024 13.0 / 14.1, but 4096 x 4608 x 1488 40.5 / 32.8, 6144 x 1152 x 3072 21.9 / 18.2)
       const double pairs = qdit_gemm_pair_cost(ctx, p) * (cls == 3 && p.a_zp != 0 ? 1.05 : 1.0);
       const double spare = cls == 3 ? (waves == 1 ? 3000.0 : 0.0) : cls != 1 || one_wave ? 1500.0 : waves == 1 ? 3000.0 : 2500.0;
       const double first = waves == 1 ? (p.K + BK - 1) / BK * 110.0 : 0.0;
-      // (f32 output: with one wave, with two or three that are almost full, and with reductions short enough that the output's own time counts: a tile's 128
-      // channels are whole 512-byte pieces of a row there, which memory takes at 5.4 TB/s, where a pair's 128-byte pieces reach 3.4; us, channel-major /
-      // pairs: 10000 x 20480 x 64 151 / 242, 6144 x 20480 x 384 98 / 152, 8192 x 6912 x 384 44 / 53, 4096 x 30720 x 768 127 / 169, 4611 x 15448 x 1024
-      // 83 / 94, 8192 x 9216 x 1024 88 / 95, 2048 x 30720 x 1152 78 / 86, 1728 x 4608 x 256 8.8 / 9.8, 2048 x 4096 x 768 11.0 / 12.0, 3072 x 4096 x 768 14.7 / 16.2; but 3072 x 3456 x 768 14.1 / 12.2, 5000 x 4608 x
-      // 768 29.8 / 26, 8192 x 3456 x 1152 38.5 / 34.8, and 1600 x 98304 x 1152, whose weights a pair reads once, 243 / 194)
+      // (f32 output: with one wave, with two or three that are almost full, and with reductions short enough that the output's own time counts: a
+      // tile's 128 channels are whole 512-byte pieces of a row there, which memory takes at 5.4 TB/s, where a pair's 128-byte pieces reach 3.4; us,
+      // channel-major / pairs: 10000 x 20480 x 64 151 / 242, 6144 x 20480 x 384 98 / 152, 8192 x 6912 x 384 44 / 53, 4096 x 30720 x 768 127 / 169, 4611
+      // x 15448 x 1024 83 / 94, 8192 x 9216 x 1024 88 / 95, 2048 x 30720 x 1152 78 / 86, 1728 x 4608 x 256 8.8 / 9.8, 2048 x 4096 x 768 11.0 / 12.0,
+      // 3072 x 4096 x 768 14.7 / 16.2; but 3072 x 3456 x 768 14.1 / 12.2, 5000 x 4608 x 768 29.8 / 26, 8192 x 3456 x 1152 38.5 / 34.8, and 1600 x 98304
+      // x 1152, whose weights a pair reads once, 243 / 194)
       const bool wide = static_cast<int64_t>(p.N) * p.K <= (48 << 20);   // (weights that stay in L2)
       const int short_k = wide && p.N >= 16384 ? 1152 : wide && p.N >= 9216 ? 1024 : p.N >= 6144 ? 768 : 384;
       const bool full = waves <= 3 && static_cast<int64_t>((p.M + 255) / 256) * ((p.N + 127) / 128) * 20 >= 17 * waves * ctx->num_sms;

@@ -679,14 +679,14 @@ int32_t launch_p_epi(qdit_ctx* ctx, const void* A, const void* W, const GemmPara
 }
 
 // Channels per tile: the least of waves x (time of a tile) + the last tile's epilogue, in clocks.  A k-block takes 200 + 1.22 BN (512 with 256
-// channels: the tensor core's own time; 434 with 192: the fill and the operand reads of shared memory), a tile 600 more; an epilogue
-// takes `chunk` for 32 channels and bounds the tile where that is longer; codes no less than what four chunks take, and from five on what six and a half
-// do (four warps share a lane quadrant and take a chunk each: 640 x 9728 x 512 13.4 us with 64 channels, 10.6 token-major; 2048 x 4096 x 768 15.3 / 13.0 / 12.2 / 13.7 /
-// 13.9 / 14.6 / 12.5 with 64 / 96 / 128 / 160 / 192 / 224 / 256); with the three warps of short gated reductions three, and five and a third for four or five chunks (8192
-// x 768 x 384 11.7 / 9.9 / 10.9 / 11.1 / 9.6 / 10.9 / 11.1).  A narrower tile has to be
-// 4 % better: it reads the tokens more often (fc2 at 65536 rows: 256 us with 256 channels, 316 with 192, which this estimate puts level).
-// Measured: 8192 x 3456 x 1152 24.4 / 24.0 / 24.0 us with 256 / 224 / 192 channels, 2048 rows 10.1 / 9.7 / 9.0; 8192 x 1152 x 4608 40.5 with
-// 256, 34.8 with 192, 36.5 with 128; 1024 x 4608 x 1152 10.1 with 256, 9.4 with 128.
+// channels: the tensor core's own time; 434 with 192: the fill and the operand reads of shared memory), a tile 600 more; an epilogue takes `chunk` for
+// 32 channels and bounds the tile where that is longer; codes no less than what four chunks take, and from five on what six and a half do (four warps
+// share a lane quadrant and take a chunk each: 640 x 9728 x 512 13.4 us with 64 channels, 10.6 token-major; 2048 x 4096 x 768 15.3 / 13.0 / 12.2 / 13.7
+// / 13.9 / 14.6 / 12.5 with 64 / 96 / 128 / 160 / 192 / 224 / 256); with the three warps of short gated reductions three, and five and a third for four
+// or five chunks (8192 x 768 x 384 11.7 / 9.9 / 10.9 / 11.1 / 9.6 / 10.9 / 11.1).  A narrower tile has to be 4 % better: it reads the tokens more often
+// (fc2 at 65536 rows: 256 us with 256 channels, 316 with 192, which this estimate puts level). Measured: 8192 x 3456 x 1152 24.4 / 24.0 / 24.0 us with
+// 256 / 224 / 192 channels, 2048 rows 10.1 / 9.7 / 9.0; 8192 x 1152 x 4608 40.5 with 256, 34.8 with 192, 36.5 with 128; 1024 x 4608 x 1152 10.1 with
+// 256, 9.4 with 128.
 struct PairTile {
   int bn;
   double cost;
