@@ -491,7 +491,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           uint32_t a[16], b[16];
           // parameters of this thread's channels n0 + 8k + 2(lane%4), + 1 (past N: those of the last pair, whose results are not stored)
           float2 sc[4], bi[4], gate[4];
-          int2 zt[4];   // zero-point terms
+          [[maybe_unused]] int2 zt[4];   // f32 output: zero-point terms
           bool landed = false;   // a look at the residual's barrier, whose phase has usually ended by now
           auto channel = [&](int k) {
             const int n = n0 + 8 * k + 2 * (lane & 3);
@@ -507,7 +507,7 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             }
             tmem_ld_16x256b_x4(taddr + static_cast<uint32_t>(c * 32), a);
             tmem_ld_16x256b_x4(taddr + (16u << 16) + static_cast<uint32_t>(c * 32), b);
-            if (!C::GATED && p.a_zp != 0) {   // (while the accumulator comes; the gated layers have no registers left for it)
+            if (EPI >= 6 && p.a_zp != 0) {   // (while the accumulator comes; the gated layers have no registers left for it, and bf16 gains nothing)
 #pragma unroll
               for (int k = 0; k < 4; ++k) zt[k] = *reinterpret_cast<const int2*>(p.w_colsum + channel(k));
             }
@@ -518,8 +518,8 @@ gemm_i8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
           if (p.a_zp != 0) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              if (C::GATED) zt[k] = *reinterpret_cast<const int2*>(p.w_colsum + channel(k));
-              const uint32_t z0 = static_cast<uint32_t>(p.a_zp * zt[k].x), z1 = static_cast<uint32_t>(p.a_zp * zt[k].y);
+              const int2 z = EPI >= 6 ? zt[k] : *reinterpret_cast<const int2*>(p.w_colsum + channel(k));
+              const uint32_t z0 = static_cast<uint32_t>(p.a_zp * z.x), z1 = static_cast<uint32_t>(p.a_zp * z.y);
 #pragma unroll
               for (int i = 0; i < 4; i += 2) {
                 a[4 * k + i] -= z0;
